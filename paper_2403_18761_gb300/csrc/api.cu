@@ -64,6 +64,8 @@ void release_events(int dev, cudaEvent_t* ev, int n) {
         if (ev[k]) P.free_ev[dev].push_back(ev[k]);
 }
 
+}  // namespace
+
 // One stream-ordered memory pool per device, owned by the library, that keeps
 // freed workspace cached (release threshold = max) so that repeated builds
 // reuse it instead of mapping fresh memory at every synchronisation.
@@ -87,8 +89,6 @@ cudaMemPool_t library_pool() {
     }
     return pools[dev];
 }
-
-}  // namespace
 
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
@@ -149,8 +149,8 @@ struct rpd_ctx {
     // boundary triangles of the mesh for sphere shrinking (built on first use)
     double* btri = nullptr;
     int32_t* btri_face = nullptr;
-    float4* btri_ball = nullptr;   // FP32 bounding balls of the boundary triangles
     long long nbtri = -1;
+    ShrinkIndex shrink_index;   // their search structure (built with the first shrinking)
     // batches (rpd_build_batch): shape offsets of vertices, tets and spheres
     // (device copies and the host's), and the largest per-shape grid
     int nshapes = 1;
@@ -1119,18 +1119,37 @@ static rpd_status ensure_boundary(rpd_ctx* c, double** tri, int32_t** face_of) {
         }
         double* t = c->alloc<double>(9 * nb + 9);
         int32_t* f = c->alloc<int32_t>(nb + 1);
-        float4* b = c->alloc<float4>(nb + 1);
-        if (!t || !f || !b) return fail(c, RPD_E_OOM, "device allocation failed");
+        if (!t || !f) return fail(c, RPD_E_OOM, "device allocation failed");
         launch_boundary_fill(c->tets, c->adj, c->Xi, c->nt, pos, ldexp(1.0, -c->opt.grid_bits), t, f, s);
-        launch_boundary_spheres(t, nb, b, s);
         TRY(cuda_check(c, "boundary launch"));
         c->btri = t;
         c->btri_face = f;
-        c->btri_ball = b;
         c->nbtri = nb;
     }
     *tri = c->btri;
     *face_of = c->btri_face;
+    return RPD_OK;
+}
+
+// The shrinking's search structure over the boundary triangles, built on
+// first use.
+static rpd_status ensure_shrink_index(rpd_ctx* c, double** tri) {
+    int32_t* face_of = nullptr;
+    TRY(ensure_boundary(c, tri, &face_of));
+    if (c->shrink_index.order || c->nbtri == 0) return RPD_OK;
+    const long long nb = c->nbtri, ng = (nb + 31) / 32;
+    ShrinkIndex S;
+    S.order = c->alloc<uint32_t>(nb);
+    S.ball = c->alloc<float4>(nb);
+    S.nrm = c->alloc<float4>(nb);
+    S.glo = c->alloc<float4>(ng);
+    S.ghi = c->alloc<float4>(ng);
+    void* tmp = c->alloc<char>(shrink_index_tmp_bytes(nb));
+    if (!S.order || !S.ball || !S.nrm || !S.glo || !S.ghi || !tmp)
+        return fail(c, RPD_E_OOM, "device allocation failed");
+    launch_shrink_index(*tri, face_of, nb, c->Xi, c->nv, ldexp(1.0, -c->opt.grid_bits), S, tmp, c->stream);
+    TRY(cuda_check(c, "shrink index launch"));
+    c->shrink_index = S;
     return RPD_OK;
 }
 
@@ -1143,11 +1162,10 @@ rpd_status rpd_shrink(rpd_ctx* ctx, const double* d_pins, const double* d_normal
         return fail(ctx, RPD_E_INVALID, "null pointer");
     if (n >= (1ll << 31)) return fail(ctx, RPD_E_INVALID, "n must be < 2^31");
     double* tri = nullptr;
-    int32_t* face_of = nullptr;
-    TRY(ensure_boundary(ctx, &tri, &face_of));
+    TRY(ensure_shrink_index(ctx, &tri));
     // a first radius above twice any diameter the grid allows
     const double r0 = ldexp(1.0, 23 - ctx->opt.grid_bits);
-    launch_shrink(tri, ctx->btri_ball, ctx->nbtri, face_of, d_pins, d_normals, d_faces, n, r0, nullptr, d_centers,
+    launch_shrink(tri, ctx->shrink_index, ctx->nbtri, d_pins, d_normals, d_faces, n, r0, nullptr, d_centers,
                   d_radii, d_iters, nullptr, ctx->stream);
     return cuda_check(ctx, "shrink launch");
 }
@@ -1162,10 +1180,9 @@ rpd_status rpd_shrink_warm(rpd_ctx* ctx, const double* d_pins, const double* d_n
         return fail(ctx, RPD_E_INVALID, "null pointer");
     if (n >= (1ll << 31)) return fail(ctx, RPD_E_INVALID, "n must be < 2^31");
     double* tri = nullptr;
-    int32_t* face_of = nullptr;
-    TRY(ensure_boundary(ctx, &tri, &face_of));
+    TRY(ensure_shrink_index(ctx, &tri));
     const double r0 = ldexp(1.0, 23 - ctx->opt.grid_bits);
-    launch_shrink(tri, ctx->btri_ball, ctx->nbtri, face_of, d_pins, d_normals, d_faces, n, r0, d_r_start, d_centers,
+    launch_shrink(tri, ctx->shrink_index, ctx->nbtri, d_pins, d_normals, d_faces, n, r0, d_r_start, d_centers,
                   d_radii, d_iters, d_restarted, ctx->stream);
     return cuda_check(ctx, "shrink launch");
 }

@@ -217,21 +217,32 @@ void launch_batch_cut(const int32_t* lead, long long rows, int stride, const lon
 void launch_batch_cut_pieces(const int64_t* pair_off, const int64_t* piece_off, const long long* toff, int nshapes,
                              long long* out, cudaStream_t s);
 
+// Search structure of the shrinking over the boundary triangles: order[i] =
+// the i-th triangle in Morton order, its bounding ball, and its unit normal
+// with the boundary face's bits; boxes of the groups of 32 (low, high corner).
+struct ShrinkIndex {
+    uint32_t* order = nullptr;
+    float4 *ball = nullptr, *nrm = nullptr, *glo = nullptr, *ghi = nullptr;
+};
+size_t shrink_index_tmp_bytes(long long nb);
+void launch_shrink_index(const double* tri, const int32_t* face_of, long long nb, const int32_t* Xi, long long nv,
+                         double unit, const ShrinkIndex& S, void* tmp, cudaStream_t s);
 // Sphere shrinking from n pins against the boundary triangles; r_start
 // (NULL or per pin, 0 = plain) proposes the first radius, restarted (NULL or
 // per pin) flags proposals that were rejected.
-// FP32 bounding balls (centre, radius) of the boundary triangles, for the
-// shrinking's cull.
-void launch_boundary_spheres(const double* tri, long long n, float4* bs, cudaStream_t s);
-void launch_shrink(const double* tri, const float4* bs, long long ntri, const int32_t* face_of, const double* pins,
-                   const double* normals, const int32_t* faces, long long n, double r0, const double* r_start,
-                   double* centres, double* radii, int32_t* iters, int32_t* restarted, cudaStream_t s);
+void launch_shrink(const double* tri, const ShrinkIndex& S, long long ntri, const double* pins, const double* normals,
+                   const int32_t* faces, long long n, double r0, const double* r_start, double* centres, double* radii,
+                   int32_t* iters, int32_t* restarted, cudaStream_t s);
 // Learned proposer glue: pin features (and log2(r / diag) targets), the
 // decoded first radius, and the grid vertices' bounding box (int[6]).
 void launch_pin_features(const double* pins, const double* normals, const double* radii, long long n,
                          const double* bc, double bh, double diag, float* x, float* t, cudaStream_t s);
 void launch_radius_start(const float* y, long long n, double diag, double margin, double* rs, cudaStream_t s);
 void launch_bbox(const int32_t* X, long long nv, int* b, cudaStream_t s);
+
+// ----------------------------------------------------------------- api.cu
+// The library's stream-ordered memory pool of the current device (NULL on error).
+cudaMemPool_t library_pool();
 
 // ---------------------------------------------------------------- topo.cu
 // Iteration bound for ClipArgs::uf_limit (a test hook may lower it).

@@ -17,7 +17,6 @@
 // neighbour); a pin is the centroid of such a triangle, its normal points
 // into the tet.  Which component a piece belongs to is read from the
 // union-find parents the finalisation left for that element kind.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -30,6 +29,7 @@
 namespace {
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
+inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 __device__ __forceinline__ void face_corners(int f, int& a, int& b, int& c) {
     a = f == 0 ? 1 : 0;
@@ -265,25 +265,90 @@ __global__ void k_not_flag(const uint8_t* __restrict__ flag, long long n, uint8_
     if (i < n) out[i] = flag[i] ? 0 : 1;
 }
 
-// Bounding ball of each boundary triangle for the shrinking's cull: the
-// centroid rounded to FP32, and a radius, measured in FP64 from that rounded
-// centre to the corners, rounded up to FP32 with a 2^-20 relative margin.
-__global__ void k_bnd_spheres(const double* __restrict__ tri, long long n, float4* __restrict__ bs) {
+// Search structure of the shrinking: the boundary triangles in Morton order,
+// in groups of 32 (one per lane of a warp).  Per triangle, in that order: a
+// bounding ball (the centroid rounded to FP32; a radius measured in FP64 from
+// the rounded centre to the corners and rounded up with a 2^-20 relative
+// margin), the unit normal and the boundary face; per group an axis-aligned
+// box rounded outwards.
+__device__ __forceinline__ uint64_t spread10(uint32_t v) {
+    uint64_t x = v & 1023u;
+    x = (x | x << 16) & 0x030000ffull;
+    x = (x | x << 8) & 0x0300f00full;
+    x = (x | x << 4) & 0x030c30c3ull;
+    x = (x | x << 2) & 0x09249249ull;
+    return x;
+}
+
+// Morton code of a triangle's centroid, 10 bits per axis over the mesh's box
+// (box: grid units, lo then hi).
+__global__ void k_bnd_key(const double* __restrict__ tri, long long n, double scale, const int* __restrict__ box,
+                          uint64_t* __restrict__ key, uint32_t* __restrict__ val) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double* T = tri + 9 * i;
-    float g[3];
-    for (int k = 0; k < 3; k++) g[k] = (float)((T[k] + T[3 + k] + T[6 + k]) / 3.0);
-    double r = 0.0;
-    for (int v = 0; v < 3; v++) {
-        double d2 = 0.0;
-        for (int k = 0; k < 3; k++) {
-            const double d = T[3 * v + k] - (double)g[k];
-            d2 += d * d;
-        }
-        r = fmax(r, sqrt(d2));
+    const int ext = max(box[3] - box[0], max(box[4] - box[1], box[5] - box[2]));
+    const int shift = max(0, 22 - __clz(max(ext, 1)));   // ext >> shift < 1024
+    uint32_t u[3];
+    for (int a = 0; a < 3; a++) {
+        const double g = (tri[9 * i + a] + tri[9 * i + 3 + a] + tri[9 * i + 6 + a]) * scale / 3.0;
+        const int v = min(max((int)g - box[a], 0), ext) >> shift;
+        u[a] = (uint32_t)v;
     }
-    bs[i] = make_float4(g[0], g[1], g[2], __double2float_ru(r * (1.0 + 0x1p-20)));
+    key[i] = spread10(u[0]) | (spread10(u[1]) << 1) | (spread10(u[2]) << 2);
+    val[i] = (uint32_t)i;
+}
+
+// One warp per group of 32 sorted triangles.  If the sort's bounded wait ran
+// out (*err), the triangles are taken in input order: slower searches, the
+// same results.
+__global__ void k_bnd_groups(const double* __restrict__ tri, const int32_t* __restrict__ face_of, long long n,
+                             uint32_t* __restrict__ order, const int* __restrict__ err, float4* __restrict__ ball,
+                             float4* __restrict__ nrm, float4* __restrict__ glo, float4* __restrict__ ghi) {
+    const unsigned FULL = 0xffffffffu;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const long long g = i >> 5;
+    if (32 * g >= n) return;   // warp-uniform
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (i < n) {
+        if (*err) order[i] = (uint32_t)i;
+        const long long src = order[i];
+        const double* T = tri + 9 * src;
+        float c[3];
+        for (int k = 0; k < 3; k++) {
+            c[k] = (float)((T[k] + T[3 + k] + T[6 + k]) / 3.0);
+            lo[k] = __double2float_rd(fmin(T[k], fmin(T[3 + k], T[6 + k])));
+            hi[k] = __double2float_ru(fmax(T[k], fmax(T[3 + k], T[6 + k])));
+        }
+        double r = 0.0;
+        for (int v = 0; v < 3; v++) {
+            double d2 = 0.0;
+            for (int k = 0; k < 3; k++) {
+                const double d = T[3 * v + k] - (double)c[k];
+                d2 += d * d;
+            }
+            r = fmax(r, sqrt(d2));
+        }
+        ball[i] = make_float4(c[0], c[1], c[2], __double2float_ru(r * (1.0 + 0x1p-20)));
+        // unit normal; a sliver whose normal FP64 does not fix to 2^-26 gets 0
+        // (its lower bound is then the ball's)
+        const double ux = T[3] - T[0], uy = T[4] - T[1], uz = T[5] - T[2];
+        const double vx = T[6] - T[0], vy = T[7] - T[1], vz = T[8] - T[2];
+        const double nx = uy * vz - uz * vy, ny = uz * vx - ux * vz, nz = ux * vy - uy * vx;
+        const double nn = sqrt(nx * nx + ny * ny + nz * nz);
+        const double uv = sqrt((ux * ux + uy * uy + uz * uz) * (vx * vx + vy * vy + vz * vz));
+        const double inv = nn > uv * 0x1p-24 ? 1.0 / nn : 0.0;
+        nrm[i] = make_float4((float)(nx * inv), (float)(ny * inv), (float)(nz * inv), __int_as_float(face_of[src]));
+    }
+    for (int k = 0; k < 3; k++)
+        for (int off = 16; off; off >>= 1) {
+            lo[k] = fminf(lo[k], __shfl_xor_sync(FULL, lo[k], off));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(FULL, hi[k], off));
+        }
+    if (lane == 0) {
+        glo[g] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+        ghi[g] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+    }
 }
 
 // ------------------------------------------------------------ shrinking
@@ -343,53 +408,50 @@ __device__ __forceinline__ void nearest_on_triangle(const double* T, const doubl
         for (int k = 0; k < 3; k++) q[k] = q2[k];
 }
 
-constexpr int SHRINK_THREADS = 256;
 constexpr int SHRINK_ITERS = 100;
-constexpr int SHRINK_CLUSTER = 8;   // CTAs per pin (a portable cluster size)
-
-// (distance, triangle) pairs ordered by distance, then by the lower index; a
-// pair with no triangle (-1) loses every tie.
-__device__ __forceinline__ bool closer(double d, long long k, double bd, long long bk) {
-    return d < bd || (d == bd && k >= 0 && (bk < 0 || k < bk));
-}
 
 // Sphere shrinking against all boundary triangles except the pin's own, one
-// thread-block cluster of SHRINK_CLUSTER CTAs per pin.  Each CTA scans one
-// contiguous part of the triangles for the one nearest to the current centre;
-// the parts' results meet through distributed shared memory after a cluster
-// barrier, and every CTA takes the same (distance, lowest index) minimum over
-// them in rank order, so all CTAs follow the same radii and leave the loop
-// together.  The minimum does not depend on how the triangles are split, so
-// the result equals that of a single block scanning them all.
+// warp (and block) per pin.
 //
-// Cull: a triangle whose bounding ball lies farther from the centre than the
-// current radius r cannot be the nearest one, nor tie with it: the nearest
-// one of a non-empty ball is within r, and an empty ball ends the shrinking
-// whichever triangle is nearest.  The test runs in FP32 on the rounded centre
-// with margins (2^-18 of the distance and 3 x 2^-18 of the centre's largest
-// coordinate) far above the FP32 rounding of the test, so it never culls a
-// triangle within r; only the triangles left are tested in FP64, and the
-// result is that of testing them all.  Output centre and radius (NaN for a
-// pin row without a face).
-__global__ void __cluster_dims__(SHRINK_CLUSTER, 1, 1) __launch_bounds__(SHRINK_THREADS)
-    k_shrink(const double* __restrict__ tri, const float4* __restrict__ bs, long long ntri,
-             const int32_t* __restrict__ face_of, const double* __restrict__ pins, const double* __restrict__ normals, const int32_t* __restrict__ faces,
-             double r0, const double* __restrict__ r_start, double* __restrict__ centres, double* __restrict__ radii,
-             int32_t* __restrict__ iters, int32_t* __restrict__ restarted) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ double sd[SHRINK_THREADS / 32];
-    __shared__ long long si[SHRINK_THREADS / 32];
-    __shared__ double part_d[2];        // this CTA's nearest triangle, by iteration parity
-    __shared__ long long part_k[2];
-    __shared__ double sr;
-    __shared__ int sdone, swarm;
-    const unsigned rank = cluster.block_rank();
-    const long long j = blockIdx.x / SHRINK_CLUSTER;   // the cluster's pin (uniform over the cluster)
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+// FP64 runs at 1/64 of the FP32 rate here, so a warp-wide FP64 point-triangle
+// test (a few hundred FP64 instructions) costs about two microseconds of an
+// SM whatever its number of active lanes: the work that counts is the number
+// of such warp steps.  An FP32 search over the Morton-ordered groups first
+// collects the triangles that can be the nearest one, then one step (rarely
+// more) tests them side by side in FP64.  Every FP32 test is one-sided:
+//  * a group is opened when the distance from the centre to its box, lowered
+//    by the margins below, is at most `ub`;
+//  * a triangle is collected when the lower bound
+//      sqrt(h^2 + max(0, l - rho)^2)   (h, l: the distance of the ball's
+//    centre along and across the triangle's normal, rho the ball's radius) is
+//    at most ub: across a flat patch only the triangles around the foot pass;
+//  * ub is an upper bound of what can matter: the current radius (a triangle
+//    farther than it cannot be the nearest of a non-empty ball, and an empty
+//    ball ends the shrinking whichever triangle is nearest), lowered by the
+//    distances to group boxes' far corners, to triangles' centroids and, once
+//    tested, by FP64 distances.
+// Margins: 2^-18 of the distance and 3 x 2^-18 of the centre's largest
+// coordinate (and 2^-18 rho), far above the FP32 rounding of the tests; so the
+// nearest triangle, and any tied with it, is always tested in FP64, and the
+// (distance, lowest index) minimum is that of testing them all.
+//
+// On a 125k-tet slab (28k boundary triangles, a pin on each) a scan of all
+// bounding balls by an 8-CTA cluster per pin took 152.8 ms, 24 pins 0.66 ms.
+// Output centre and radius (NaN for a pin row without a face).
+__global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, ShrinkIndex S, long long ntri,
+                                               const double* __restrict__ pins, const double* __restrict__ normals,
+                                               const int32_t* __restrict__ faces, double r0,
+                                               const double* __restrict__ r_start, double* __restrict__ centres,
+                                               double* __restrict__ radii, int32_t* __restrict__ iters,
+                                               int32_t* __restrict__ restarted) {
+    const unsigned FULL = 0xffffffffu;
+    __shared__ int list[64];      // collected triangles (sorted positions)
+    __shared__ float list_lb[64];
+    const long long j = blockIdx.x;
+    const int lane = threadIdx.x;
     const int own = faces[j];
-    if (own < 0) {   // every CTA of the cluster leaves here, before any cluster barrier
-        if (rank == 0 && tid == 0) {
+    if (own < 0) {
+        if (lane == 0) {
             for (int k = 0; k < 3; k++) centres[3 * j + k] = nan("");
             radii[j] = nan("");
             iters[j] = 0;
@@ -397,112 +459,155 @@ __global__ void __cluster_dims__(SHRINK_CLUSTER, 1, 1) __launch_bounds__(SHRINK_
         }
         return;
     }
-    const long long per = (ntri + SHRINK_CLUSTER - 1) / SHRINK_CLUSTER;
-    const long long lo = per * rank, hi = lo + per < ntri ? lo + per : ntri;
+    const long long ngroup = (ntri + 31) / 32;
     const double p[3] = {pins[3 * j], pins[3 * j + 1], pins[3 * j + 2]};
     const double n[3] = {normals[3 * j], normals[3 * j + 1], normals[3 * j + 2]};
+    // a proposed first radius (0 < r < r0) replaces r0; the first ball must
+    // then contain a surface point, otherwise it may lie below the fixed point
+    // and the shrinking starts over from r0
+    const double rs = r_start ? r_start[j] : 0.0;
+    bool warm = rs > 0.0 && rs < r0, fresh = true;
     int rs_flag = 0;
-    if (tid == 0) {
-        // a proposed first radius (0 < r < r0) replaces r0; the first ball
-        // must then contain a surface point, otherwise it may lie below the
-        // fixed point and the shrinking starts over from r0
-        const double rs = r_start ? r_start[j] : 0.0;
-        swarm = rs > 0.0 && rs < r0;
-        sr = swarm ? rs : r0;
-        sdone = 0;
-    }
-    __syncthreads();
+    double r = warm ? rs : r0;
     int it = 0;
-    for (; it < SHRINK_ITERS; it++) {
-        const double r = sr;
+    for (; it < SHRINK_ITERS; it++) {   // everything that steers the loop is uniform over the warp
         const double c[3] = {p[0] + r * n[0], p[1] + r * n[1], p[2] + r * n[2]};
-        const float cf[3] = {(float)c[0], (float)c[1], (float)c[2]};
-        const float cslack = 3.0f * 0x1p-18f * fmaxf(fabsf(cf[0]), fmaxf(fabsf(cf[1]), fabsf(cf[2])));
-        const float uf = __double2float_ru(r * (1.0 + 0x1p-20));
-        double bd = INFINITY;
-        long long bi = -1;
-        for (long long k = lo + tid; k < hi; k += SHRINK_THREADS) {
-            const float4 b = bs[k];
-            const float dx = cf[0] - b.x, dy = cf[1] - b.y, dz = cf[2] - b.z;
-            const float lb = sqrtf(dx * dx + dy * dy + dz * dz) * (1.0f - 0x1p-18f) - b.w - cslack;
-            if (lb > uf) continue;   // the whole triangle lies farther than r
-            if (face_of[k] == own) continue;
-            double q[3];
-            nearest_on_triangle(tri + 9 * k, c, q);
-            const double d = (q[0] - c[0]) * (q[0] - c[0]) + (q[1] - c[1]) * (q[1] - c[1]) + (q[2] - c[2]) * (q[2] - c[2]);
-            if (d < bd) {
-                bd = d;
-                bi = k;
+        const float cx = (float)c[0], cy = (float)c[1], cz = (float)c[2];
+        const float cslack = 3.0f * 0x1p-18f * fmaxf(fabsf(cx), fmaxf(fabsf(cy), fabsf(cz)));
+        float ub = __double2float_ru(r * (1.0 + 0x1p-20));
+        if (fresh) {   // far from the fixed point: a first bound from the groups of two or more triangles
+            float far = INFINITY;
+            for (long long g = lane; g < ngroup; g += 32) {
+                if (32 * g + 1 >= ntri) continue;   // a lone triangle may be the pin's own
+                const float4 lo = S.glo[g], hi = S.ghi[g];
+                const float fx = fmaxf(fabsf(cx - lo.x), fabsf(cx - hi.x)), fy = fmaxf(fabsf(cy - lo.y), fabsf(cy - hi.y)),
+                            fz = fmaxf(fabsf(cz - lo.z), fabsf(cz - hi.z));
+                far = fminf(far, sqrtf(fx * fx + fy * fy + fz * fz) * (1.0f + 0x1p-18f) + cslack);
+            }
+            ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(far))));
+        }
+        double bd = INFINITY, bq[3] = {0, 0, 0};
+        int bi = -1, cnt = 0;
+        // FP64 test of the last min(cnt, 32) collected triangles
+        auto flush = [&]() {
+            const int m = min(cnt, 32);
+            __syncwarp();
+            const bool on = lane < m && list_lb[cnt - m + lane] <= ub;
+            if (__any_sync(FULL, on)) {
+                float d32 = INFINITY;
+                if (on) {
+                    const int k = (int)S.order[list[cnt - m + lane]];
+                    double q[3];
+                    nearest_on_triangle(tri + 9ll * k, c, q);
+                    const double d =
+                        (q[0] - c[0]) * (q[0] - c[0]) + (q[1] - c[1]) * (q[1] - c[1]) + (q[2] - c[2]) * (q[2] - c[2]);
+                    d32 = sqrtf(__double2float_ru(d)) * (1.0f + 0x1p-20f);
+                    if (d < bd || (d == bd && k < bi)) {
+                        bd = d;
+                        bi = k;
+                        for (int z = 0; z < 3; z++) bq[z] = q[z];
+                    }
+                }
+                ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(d32))));
+            }
+            cnt -= m;
+            __syncwarp();
+        };
+        for (long long g0 = 0; g0 < ngroup; g0 += 32) {
+            float lbg = INFINITY;
+            if (g0 + lane < ngroup) {
+                const float4 lo = S.glo[g0 + lane], hi = S.ghi[g0 + lane];
+                const float dx = fmaxf(fmaxf(lo.x - cx, cx - hi.x), 0.0f), dy = fmaxf(fmaxf(lo.y - cy, cy - hi.y), 0.0f),
+                            dz = fmaxf(fmaxf(lo.z - cz, cz - hi.z), 0.0f);
+                lbg = sqrtf(dx * dx + dy * dy + dz * dz) * (1.0f - 0x1p-18f) - cslack;
+            }
+            for (unsigned open = __ballot_sync(FULL, lbg <= ub); open; open &= open - 1) {
+                const int z = __ffs(open) - 1;
+                if (__shfl_sync(FULL, lbg, z) > ub) continue;   // ub has fallen since
+                const long long k = 32 * (g0 + z) + lane;
+                float lb = INFINITY, far = INFINITY;
+                if (k < ntri) {
+                    const float4 b = S.ball[k], u = S.nrm[k];
+                    if (__float_as_int(u.w) != own) {
+                        const float vx = cx - b.x, vy = cy - b.y, vz = cz - b.z;
+                        const float v = sqrtf(vx * vx + vy * vy + vz * vz);
+                        const float m = 0x1p-18f * (v + b.w) + cslack;
+                        const float h = vx * u.x + vy * u.y + vz * u.z;
+                        const float wx = vx - h * u.x, wy = vy - h * u.y, wz = vz - h * u.z;
+                        const float l = fmaxf(sqrtf(wx * wx + wy * wy + wz * wz) - b.w - m, 0.0f);
+                        const float a = fmaxf(fabsf(h) - m, 0.0f);
+                        lb = sqrtf(a * a + l * l) * (1.0f - 0x1p-20f);
+                        far = v + m;
+                    }
+                }
+                ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(far))));
+                const unsigned in = __ballot_sync(FULL, lb <= ub);
+                if (lb <= ub) {
+                    const int at = cnt + __popc(in & ((1u << lane) - 1u));
+                    list[at] = (int)k;
+                    list_lb[at] = lb;
+                }
+                cnt += __popc(in);   // at most 31 + 32
+                if (cnt >= 32) {     // drop what ub has overtaken, test 32 if that many are left
+                    __syncwarp();
+                    const bool h1 = lane + 32 < cnt;
+                    const int k0 = list[lane], k1 = h1 ? list[lane + 32] : 0;
+                    const float l0 = list_lb[lane], l1 = h1 ? list_lb[lane + 32] : INFINITY;
+                    const unsigned m0 = __ballot_sync(FULL, l0 <= ub), m1 = __ballot_sync(FULL, l1 <= ub);
+                    const unsigned lt = (1u << lane) - 1u;
+                    __syncwarp();
+                    if (l0 <= ub) {
+                        list[__popc(m0 & lt)] = k0;
+                        list_lb[__popc(m0 & lt)] = l0;
+                    }
+                    if (l1 <= ub) {
+                        list[__popc(m0) + __popc(m1 & lt)] = k1;
+                        list_lb[__popc(m0) + __popc(m1 & lt)] = l1;
+                    }
+                    cnt = __popc(m0) + __popc(m1);
+                    if (cnt >= 32) flush();
+                }
             }
         }
+        while (cnt > 0) flush();
+        // nearest triangle over the lanes, the lowest index of a tie, and its point
+        double d = bd;
+        int k = bi;
+        int src = lane;
         for (int off = 16; off; off >>= 1) {
-            const double od = __shfl_down_sync(0xffffffffu, bd, off);
-            const long long oi = __shfl_down_sync(0xffffffffu, bi, off);
-            if (closer(od, oi, bd, bi)) {
-                bd = od;
-                bi = oi;
+            const double od = __shfl_xor_sync(FULL, d, off);
+            const int ok = __shfl_xor_sync(FULL, k, off), os = __shfl_xor_sync(FULL, src, off);
+            if (od < d || (od == d && ok >= 0 && (k < 0 || ok < k))) {
+                d = od;
+                k = ok;
+                src = os;
             }
         }
-        if (lane == 0) {
-            sd[w] = bd;
-            si[w] = bi;
-        }
-        __syncthreads();
-        const int par = it & 1;
-        if (tid == 0) {
-            double d = INFINITY;
-            long long k = -1;
-            for (int z = 0; z < SHRINK_THREADS / 32; z++)
-                if (closer(sd[z], si[z], d, k)) {
-                    d = sd[z];
-                    k = si[z];
-                }
-            part_d[par] = d;
-            part_k[par] = k;
-        }
-        // the parts of this iteration are visible cluster-wide after the
-        // barrier; a part slot is written again two iterations later, after
-        // the next barrier, which every CTA reaches only once it has read it
-        cluster.sync();
-        if (tid == 0) {
-            double d = INFINITY;
-            long long k = -1;
-            for (unsigned z = 0; z < SHRINK_CLUSTER; z++) {
-                const double* pd = cluster.map_shared_rank(&part_d[par], z);
-                const long long* pk = cluster.map_shared_rank(&part_k[par], z);
-                const double od = *pd;
-                const long long ok = *pk;
-                if (closer(od, ok, d, k)) {
-                    d = od;
-                    k = ok;
-                }
-            }
-            // empty ball (within rounding): done, unless it is a proposed one
-            if (k < 0 || sqrt(d) >= r * (1.0 - 1e-12)) {
-                if (swarm) {
-                    sr = r0;
-                    rs_flag = 1;
-                } else {
-                    sdone = 1;
-                }
+        src = __shfl_sync(FULL, src, 0);
+        fresh = false;
+        // empty ball (within rounding): done, unless it is a proposed one
+        bool stop = false;
+        if (k < 0 || sqrt(d) >= r * (1.0 - 1e-12)) {
+            if (warm) {
+                r = r0;
+                rs_flag = 1;
+                fresh = true;
             } else {
-                double q[3];
-                nearest_on_triangle(tri + 9 * k, c, q);
-                const double pq[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
-                const double dn = pq[0] * n[0] + pq[1] * n[1] + pq[2] * n[2];
-                const double rn = (pq[0] * pq[0] + pq[1] * pq[1] + pq[2] * pq[2]) / (2.0 * dn);
-                if (!(dn > 0) || !(rn < r)) sdone = 1;   // no progress possible
-                else sr = rn;
+                stop = true;
             }
-            swarm = 0;
+        } else {
+            const double q[3] = {__shfl_sync(FULL, bq[0], src), __shfl_sync(FULL, bq[1], src),
+                                 __shfl_sync(FULL, bq[2], src)};
+            const double pq[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
+            const double dn = pq[0] * n[0] + pq[1] * n[1] + pq[2] * n[2];
+            const double rn = (pq[0] * pq[0] + pq[1] * pq[1] + pq[2] * pq[2]) / (2.0 * dn);
+            if (!(dn > 0) || !(rn < r)) stop = true;   // no progress possible
+            else r = rn;
         }
-        __syncthreads();
-        if (sdone) break;
+        warm = false;
+        if (stop) break;
     }
-    // peers may still be reading this CTA's parts: leave together
-    cluster.sync();
-    if (rank == 0 && tid == 0) {
-        const double r = sr;
+    if (lane == 0) {
         for (int k = 0; k < 3; k++) centres[3 * j + k] = p[k] + r * n[k];
         radii[j] = r;
         iters[j] = it + 1;
@@ -678,23 +783,41 @@ void launch_pins(const ClipArgs& a, int kind, const int32_t* keys, const int32_t
     note_launch();
 }
 
-void launch_boundary_spheres(const double* tri, long long n, float4* bs, cudaStream_t s) {
-    if (n <= 0) return;
-    k_bnd_spheres<<<nblk(n, 256), 256, 0, s>>>(tri, n, bs);
+// The search structure of nb boundary triangles; index buffers are the
+// caller's, tmp must hold shrink_index_tmp_bytes(nb).
+size_t shrink_index_tmp_bytes(long long nb) {
+    return 2 * al256(8 * (size_t)nb) + al256(4 * (size_t)nb) + 256 + radix_tmp_bytes(nb);
+}
+
+void launch_shrink_index(const double* tri, const int32_t* face_of, long long nb, const int32_t* Xi, long long nv,
+                         double unit, const ShrinkIndex& S, void* tmp, cudaStream_t s) {
+    if (nb <= 0) return;
+    char* p = (char*)tmp;
+    uint64_t* k0 = (uint64_t*)p;
+    p += al256(8 * (size_t)nb);
+    uint64_t* k1 = (uint64_t*)p;
+    p += al256(8 * (size_t)nb);
+    uint32_t* v0 = (uint32_t*)p;
+    p += al256(4 * (size_t)nb);
+    int* box = (int*)p;
+    int* err = box + 6;
+    p += 256;
+    cudaMemsetAsync(err, 0, sizeof(int), s);
+    launch_bbox(Xi, nv, box, s);
+    k_bnd_key<<<nblk(nb, 256), 256, 0, s>>>(tri, nb, 1.0 / unit, box, k0, v0);
+    note_launch();
+    radix_sort_pairs(k0, v0, k1, S.order, nb, 30, p, err, s);
+    k_bnd_groups<<<nblk(nb, 256), 256, 0, s>>>(tri, face_of, nb, S.order, err, S.ball, S.nrm, S.glo, S.ghi);
     note_launch();
 }
 
-void launch_shrink(const double* tri, const float4* bs, long long ntri, const int32_t* face_of, const double* pins,
-                   const double* normals, const int32_t* faces, long long n, double r0, const double* r_start,
-                   double* centres, double* radii, int32_t* iters, int32_t* restarted, cudaStream_t s) {
-    // one cluster per pin, in launches of at most 2^24 pins (grid x < 2^31)
-    for (long long b = 0; b < n; b += (1ll << 24)) {
-        const long long m = n - b < (1ll << 24) ? n - b : (1ll << 24);
-        k_shrink<<<(unsigned)(m * SHRINK_CLUSTER), SHRINK_THREADS, 0, s>>>(
-            tri, bs, ntri, face_of, pins + 3 * b, normals + 3 * b, faces + b, r0, r_start ? r_start + b : nullptr,
-            centres + 3 * b, radii + b, iters + b, restarted ? restarted + b : nullptr);
-        note_launch();
-    }
+void launch_shrink(const double* tri, const ShrinkIndex& S, long long ntri, const double* pins, const double* normals,
+                   const int32_t* faces, long long n, double r0, const double* r_start, double* centres, double* radii,
+                   int32_t* iters, int32_t* restarted, cudaStream_t s) {
+    if (n <= 0) return;
+    k_shrink<<<(unsigned)n, 32, 0, s>>>(tri, S, ntri, pins, normals, faces, r0, r_start, centres, radii, iters,
+                                        restarted);
+    note_launch();
 }
 
 // ----------------------------------------------------- proposer features
