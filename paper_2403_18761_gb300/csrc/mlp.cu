@@ -10,12 +10,13 @@
 // D[128 x N] (TMEM, FP32) += A[128 x K] B[N x K]^T with both operands BF16 in
 // shared memory, issued by one thread as tcgen05.mma kind::f16 (M = 128,
 // K = 16 per instruction), completion signalled through an mbarrier by
-// tcgen05.commit, the accumulator read back by tcgen05.ld for a fused
-// epilogue (bias + ReLU, ReLU mask, or FP32 atomic accumulation).  The
-// operands are staged by the CTA's threads (transposed where the layer needs
-// it) into the canonical no-swizzle K-major layout: 8 rows x 16 bytes per
-// core matrix, core matrices consecutive along K (leading byte offset 128)
-// and rows of core matrices K * 2 bytes x 8 apart (stride byte offset).
+// tcgen05.commit, the accumulator read back by tcgen05.ld.  Operands are in
+// the canonical no-swizzle K-major layout: 8 rows x 16 bytes per core matrix,
+// core matrices consecutive along K (leading byte offset 128) and rows of core
+// matrices K * 2 bytes x 8 apart (stride byte offset).
+//
+// One kernel (k_mlp_step) takes a 128-row tile through the whole network,
+// forward and backward, without leaving the SM: see its comment.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <cuda_bf16.h>
@@ -32,7 +33,8 @@ namespace {
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 constexpr int TM = 128;                 // rows of a tile (tcgen05 M)
-constexpr int MLP_THREADS = 128;        // 4 warps: one per 32 TMEM lanes
+constexpr int STEP_THREADS = 256;       // 8 warps: two per 32 TMEM lanes, each takes half of the columns
+constexpr int MAX_CTAS = 152;           // one per SM
 constexpr long long MBAR_SPIN_LIMIT = 1ll << 24;
 
 // ----------------------------------------------------------- PTX helpers
@@ -131,281 +133,414 @@ __device__ __forceinline__ uint32_t tile_off(int row, int k, int kdim) {
     return (uint32_t)((((row >> 3) * (kdim >> 3) + (k >> 3)) << 7) + ((row & 7) << 4) + ((k & 7) << 1));
 }
 
-// -------------------------------------------------------------- tile GEMM
-// Shared memory of one tile: A (128 x K), B (N x K), the barrier and the
-// TMEM base address.  K, N <= 128.
-struct TileSmem {
-    __nv_bfloat16 a[TM * 128];
-    __nv_bfloat16 b[128 * 128];
-    uint64_t bar;
-    uint32_t tmem;
-    int err;
-};
-
-// Issue the K / 16 MMAs of the staged tile from one thread and wait for
-// their completion (every thread waits).  False if the bounded wait ran out.
-__device__ __forceinline__ bool tile_mma(TileSmem& S, int K, int N, uint32_t phase) {
-    fence_proxy_async();   // staged operands visible to the tensor cores
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    if (threadIdx.x == 0) {
-        const uint32_t idesc = instr_desc(TM, N);
-        const uint32_t a0 = smem_u32(S.a), b0 = smem_u32(S.b);
-        for (int j = 0; j < K / 16; j++)
-            mma_bf16(S.tmem, smem_desc(a0 + 256u * j, 128u, 16u * K), smem_desc(b0 + 256u * j, 128u, 16u * K),
-                     idesc, j > 0);
-        mma_commit(&S.bar);
-    }
-    const bool ok = mbar_wait(&S.bar, phase);
-    fence_after_sync();
-    return ok;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
-
-__device__ __forceinline__ void tile_begin(TileSmem& S, int ncols) {
-    if (threadIdx.x < 32) tmem_alloc(&S.tmem, ncols);
-    if (threadIdx.x == 0) {
-        mbar_init(&S.bar, 1);
-        S.err = 0;
-    }
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-
-__device__ __forceinline__ void tile_end(TileSmem& S, int ncols, bool ok, int* err) {
-    if (!ok && threadIdx.x == 0) atomicCAS(err, 0, (int)RPD_E_TIMEOUT);
-    fence_before_sync();
-    __syncthreads();
-    if (threadIdx.x < 32) tmem_dealloc(S.tmem, ncols);
-}
-
-// Stage rows [r0, r0 + 128) x [0, K) of a row-major bf16 matrix (ld columns)
-// as an A or B operand (K-major); rows past nrows are zero.
-__device__ __forceinline__ void stage_rows(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, long long r0,
-                                           long long nrows, int nr, int K, int ld) {
-    const int chunks = nr * (K / 8);
-    for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-        const int row = c / (K / 8), kc = (c % (K / 8)) * 8;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (r0 + row < nrows) v = *reinterpret_cast<const uint4*>(src + (r0 + row) * ld + kc);
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(dst) + tile_off(row, kc, K)) = v;
-    }
-}
-
-// Stage the transpose: operand row i, column j = src[(c0 + j) * ld + i] for
-// i < nr (operand rows) and j < K (src rows c0.., zero past nsrc).
-__device__ __forceinline__ void stage_cols(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, long long c0,
-                                           long long nsrc, int nr, int K, int ld) {
-    const int chunks = nr * (K / 8);
-    for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-        const int row = c % nr, kc = (c / nr) * 8;
-        __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            const long long sr = c0 + kc + q;
-            v[q] = sr < nsrc ? src[sr * ld + row] : __float2bfloat16(0.0f);
-        }
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(dst) + tile_off(row, kc, K)) = *reinterpret_cast<uint4*>(v);
-    }
-}
-
-// Forward: Y[m][n] = relu(sum_k X[m][k] W[n][k] + b[n]) for the CTA's 128 rows.
-__global__ void __launch_bounds__(MLP_THREADS) k_mlp_fwd(const __nv_bfloat16* __restrict__ X, long long M, int K,
-                                                         const __nv_bfloat16* __restrict__ W,
-                                                         const float* __restrict__ bias, int N,
-                                                         __nv_bfloat16* __restrict__ Y, int* err) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    TileSmem& S = *reinterpret_cast<TileSmem*>(smem_raw);
-    const long long m0 = (long long)blockIdx.x * TM;
-    tile_begin(S, 128);
-    stage_rows(S.a, X, m0, M, TM, K, K);
-    stage_rows(S.b, W, 0, N, N, K, K);
-    const bool ok = tile_mma(S, K, N, 0);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long m = m0 + 32 * w + lane;
-    for (int c0 = 0; c0 < N; c0 += 32) {
-        float v[32];
-        tmem_ld32(S.tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, v);
-        if (ok && m < M) {
-            __align__(16) __nv_bfloat16 o[32];
-#pragma unroll
-            for (int k = 0; k < 32; k++) o[k] = __float2bfloat16(fmaxf(v[k] + bias[c0 + k], 0.0f));
-#pragma unroll
-            for (int q = 0; q < 4; q++)
-                reinterpret_cast<uint4*>(Y + m * N + c0)[q] = reinterpret_cast<const uint4*>(o)[q];
-        }
-    }
-    tile_end(S, 128, ok, err);
-}
-
-// Input gradient: dZprev[m][k] = (sum_n dZ[m][n] W[n][k]) * (H[m][k] > 0).
-__global__ void __launch_bounds__(MLP_THREADS) k_mlp_dx(const __nv_bfloat16* __restrict__ dZ, long long M, int N,
-                                                        const __nv_bfloat16* __restrict__ W, int K,
-                                                        const __nv_bfloat16* __restrict__ H,
-                                                        __nv_bfloat16* __restrict__ dZprev, int* err) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    TileSmem& S = *reinterpret_cast<TileSmem*>(smem_raw);
-    const long long m0 = (long long)blockIdx.x * TM;
-    tile_begin(S, 128);
-    stage_rows(S.a, dZ, m0, M, TM, N, N);    // A: 128 x N (reduction over n)
-    stage_cols(S.b, W, 0, N, K, N, K);       // B: K rows x N (B[k][n] = W[n][k])
-    const bool ok = tile_mma(S, N, K, 0);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long m = m0 + 32 * w + lane;
-    for (int c0 = 0; c0 < K; c0 += 32) {
-        float v[32];
-        tmem_ld32(S.tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, v);
-        if (ok && m < M) {
-            __align__(16) __nv_bfloat16 h[32], o[32];
-#pragma unroll
-            for (int q = 0; q < 4; q++) reinterpret_cast<uint4*>(h)[q] = reinterpret_cast<const uint4*>(H + m * K + c0)[q];
-#pragma unroll
-            for (int k = 0; k < 32; k++) o[k] = __float2bfloat16(__bfloat162float(h[k]) > 0.0f ? v[k] : 0.0f);
-#pragma unroll
-            for (int q = 0; q < 4; q++)
-                reinterpret_cast<uint4*>(dZprev + m * K + c0)[q] = reinterpret_cast<const uint4*>(o)[q];
-        }
-    }
-    tile_end(S, 128, ok, err);
-}
-
-// Weight gradient of the CTA's 128 rows: dW[n][k] += sum_m dZ[m][n] H[m][k].
-__global__ void __launch_bounds__(MLP_THREADS) k_mlp_dw(const __nv_bfloat16* __restrict__ dZ, long long M, int N,
-                                                        const __nv_bfloat16* __restrict__ H, int K,
-                                                        float* __restrict__ dW, int* err) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    TileSmem& S = *reinterpret_cast<TileSmem*>(smem_raw);
-    const long long m0 = (long long)blockIdx.x * TM;
-    tile_begin(S, 128);
-    stage_cols(S.a, dZ, m0, M, N, TM, N);    // A: N rows (n) x 128 (m)
-    stage_cols(S.b, H, m0, M, K, TM, K);     // B: K rows (k) x 128 (m)
-    const bool ok = tile_mma(S, TM, K, 0);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = 32 * w + lane;
-    for (int c0 = 0; c0 < K; c0 += 32) {
-        float v[32];
-        tmem_ld32(S.tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, v);
-        if (ok && n < N)
-#pragma unroll
-            for (int k = 0; k < 32; k++) atomicAdd(&dW[n * K + c0 + k], v[k]);
-    }
-    tile_end(S, 128, ok, err);
-}
-
-}  // namespace
-
-// ------------------------------------------------------- CUDA-core parts
-namespace {
 
 constexpr int HID = 128;   // hidden width
 constexpr int NIN = 32;    // padded input width
 // parameter offsets in the FP32 master vector
 constexpr long long OW0 = 0, OB0 = OW0 + HID * NIN, OW1 = OB0 + HID, OB1 = OW1 + HID * HID, OW2 = OB1 + HID,
                     OB2 = OW2 + HID * HID, OW3 = OB2 + HID, OB3 = OW3 + HID, NPARAM = OB3 + 1;
+constexpr int PSTRIDE = 37440;   // floats of one CTA's partial gradient: NPARAM, the loss at NPARAM, padding
+// BF16 copies of the weights as tile images (K-major, no swizzle): W0 [n][k],
+// W1, W2 [n][k], and W1, W2 transposed [k][n] for the input gradients
+constexpr int IW0 = 0, IW1 = IW0 + HID * NIN, IW2 = IW1 + HID * HID, IW1T = IW2 + HID * HID, IW2T = IW1T + HID * HID,
+              NIMG = IW2T + HID * HID;
 
-// fp32 rows [n][n_in] -> bf16 rows [cap][NIN], zero padded.
-__global__ void k_to_bf16(const float* __restrict__ x, long long n, int n_in, long long cap,
-                          __nv_bfloat16* __restrict__ X) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap * NIN) return;
-    const long long r = i / NIN;
-    const int c = (int)(i % NIN);
-    X[i] = __float2bfloat16(r < n && c < n_in ? x[r * n_in + c] : 0.0f);
+// Shared memory of one CTA (one per SM): 220 KB.
+struct StepSmem {
+    __nv_bfloat16 x[TM * NIN], xt[NIN * TM];   // the tile's inputs, by row and transposed
+    __nv_bfloat16 w0[HID * NIN];
+    __nv_bfloat16 wa[HID * HID], wb[HID * HID];   // W1 then W2^T; W2 then W1^T
+    __nv_bfloat16 row[TM * HID];                  // the A operand: H0, H1, dZ2, dZ1 by row
+    __nv_bfloat16 h0t[HID * TM], h1t[HID * TM];   // transposed activations (weight gradients' B operand)
+    __nv_bfloat16 zt[HID * TM];                   // H2, then dZ2, dZ1, dZ0, transposed (their A operand)
+    float bias[3][HID], w3[HID], ypart[2][TM], dy[TM], red[HID], lred[4];
+    uint64_t bar;
+    uint32_t tmem;
+};
+
+// 16-byte chunks of a tile image into shared memory (its own commit group).
+__device__ __forceinline__ void load_image(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int n) {
+    for (int c = threadIdx.x; c < n / 8; c += STEP_THREADS) cp_async16(dst + 8 * c, src + 8 * c);
+    cp_async_commit();
 }
 
-// Training batch: row r of the batch is row (cur[0] + r) mod n_total of the
-// data (cur on the device, so every step is the same launch sequence).
-__global__ void k_to_bf16_batch(const float* __restrict__ x, long long n_total, int n_in, long long b, long long cap,
-                                const long long* __restrict__ cur, __nv_bfloat16* __restrict__ X) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap * NIN) return;
-    const long long r = i / NIN;
-    const int c = (int)(i % NIN);
-    const long long src = (cur[0] + r) % n_total;
-    X[i] = __float2bfloat16(r < b && c < n_in ? x[src * n_in + c] : 0.0f);
+__device__ __forceinline__ char* at(__nv_bfloat16* base, int row, int k, int kdim) {
+    return reinterpret_cast<char*>(base) + tile_off(row, k, kdim);
 }
 
-// After a step: the next batch starts b rows later; one more Adam step.
-__global__ void k_cursor_advance(long long* cur, long long b, long long n_total) {
-    cur[0] = (cur[0] + b) % n_total;
-    cur[1] += 1;
-}
-
-__global__ void k_cast_weights(const float* __restrict__ p, __nv_bfloat16* __restrict__ W0,
-                               __nv_bfloat16* __restrict__ W1, __nv_bfloat16* __restrict__ W2) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < HID * NIN) W0[i] = __float2bfloat16(p[OW0 + i]);
-    if (i < HID * HID) {
-        W1[i] = __float2bfloat16(p[OW1 + i]);
-        W2[i] = __float2bfloat16(p[OW2 + i]);
+// 32 values of one tile row m, columns c0..c0+31, as BF16: by row (when row
+// is not NULL) and transposed.  The transposed stores pair the lanes of two
+// neighbouring rows into 32-bit words.
+__device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, int m, int c0,
+                                         const __nv_bfloat16 (&o)[32]) {
+    if (row) {
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            *reinterpret_cast<uint4*>(at(row, m, c0 + 8 * q, HID)) = reinterpret_cast<const uint4*>(o)[q];
+    }
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(o);
+    const int odd = m & 1;
+#pragma unroll
+    for (int q = 0; q < 16; q++) {   // columns c0 + 2q (even lane's) and c0 + 2q + 1 (odd lane's)
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, w[q], 1);
+        const uint32_t v = odd ? __byte_perm(w[q], other, 0x3276) : __byte_perm(w[q], other, 0x5410);
+        *reinterpret_cast<uint32_t*>(at(tr, c0 + 2 * q + odd, m & ~1, TM)) = v;
     }
 }
 
-// Output layer on the CUDA cores (one warp per row): y = H2 . w3 + b3; with
-// targets, also the mean-squared-error gradient: dy = 2 (y - t) / n,
-// dZ2 = bf16(dy w3 (H2 > 0)), and the head's weight and bias gradients.
-__global__ void k_head(const __nv_bfloat16* __restrict__ H2, long long n, const float* __restrict__ p,
-                       float* __restrict__ y, const float* __restrict__ t, __nv_bfloat16* __restrict__ dZ2,
-                       float* __restrict__ g, float* __restrict__ loss, const long long* __restrict__ cur,
-                       long long n_total) {
-    __shared__ float sw[HID + 1];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = threadIdx.x; k <= HID; k += blockDim.x) sw[k] = 0.0f;
-    __syncthreads();
-    float w3[4], h[4];
-    for (int q = 0; q < 4; q++) w3[q] = p[OW3 + 4 * lane + q];
+// The network on 128-row tiles, one CTA of 8 warps per SM, tiles strided over
+// the grid.  Forward: three GEMMs, each followed by an epilogue that adds the
+// bias, applies ReLU and writes the BF16 activations back to shared memory,
+// by row (the next GEMM's A operand) and, with GRAD, transposed (the weight
+// gradient's B operand).  The head (w3, b3) runs on the CUDA cores.  Backward:
+// dZ2 from the head's gradient and the ReLU mask; then per layer one batch of
+// MMAs computes the weight gradient, accumulated in TMEM over all of the CTA's
+// tiles, and the input gradient, whose epilogue masks it into the next dZ.
+// At the end every CTA writes its own partial gradient, which k_adam sums in
+// order: no atomics.
+//
+// What bounds it: latency.  A training batch of 8192 rows is 64 tiles, one per
+// SM: eight dependent MMA batches of about 0.1 us each and as many epilogues
+// through shared memory.  The form before this one ran a kernel per layer and
+// direction with global round trips in between and one FP32 atomic per weight
+// and tile: 206 us per step of 8192 rows, 17 launches; now 2 launches.
+//
+// Rows past n (the last tile's) have zero activations and dy = 0.
+// x rows: row r of the pass is row (cur[0] + r) mod n_total of the data when
+// cur is given, else row r.
+template <bool GRAD>
+__global__ void __launch_bounds__(STEP_THREADS, 1)
+    k_mlp_step(const float* __restrict__ x, const float* __restrict__ t, long long n, int n_in, long long n_total,
+               long long* __restrict__ cur, const float* __restrict__ p, const __nv_bfloat16* __restrict__ img,
+               float* __restrict__ y, float* __restrict__ part, int* __restrict__ err) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int quad = warp & 3, half = warp >> 2;   // TMEM lanes 32 quad.., columns 64 half..
+    const int m = 32 * quad + lane;                // this thread's row of the tile
+    const uint32_t D = 0, DW2 = 128, DW1 = 256, DW0 = 384;   // TMEM columns
+    const uint32_t tlane = (uint32_t)(32 * quad) << 16;
+    const long long base = cur ? cur[0] : 0;
+    if (warp == 0) tmem_alloc(&S.tmem, 512);
+    if (tid == 0) mbar_init(&S.bar, 1);
+    load_image(S.w0, img + IW0, HID * NIN);
+    for (int k = tid; k < HID; k += STEP_THREADS) {
+        S.bias[0][k] = p[OB0 + k];
+        S.bias[1][k] = p[OB1 + k];
+        S.bias[2][k] = p[OB2 + k];
+        S.w3[k] = p[OW3 + k];
+    }
     const float b3 = p[OB3];
-    float lsum = 0.0f;
-    for (long long r = (long long)blockIdx.x * nw + warp; r < n; r += (long long)gridDim.x * nw) {
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t T0 = S.tmem;
+    uint32_t phase = 0;
+    bool ok = true;
+    // staged operands visible to the tensor cores, then one thread issues
+    auto begin_mma = [&]() {
+        fence_proxy_async();
+        fence_before_sync();
+        __syncthreads();
+        fence_after_sync();
+    };
+    auto issue = [&](uint32_t d, __nv_bfloat16* a, __nv_bfloat16* b, int K, int N, bool acc) {
+        const uint32_t idesc = instr_desc(TM, N), a0 = smem_u32(a), b0 = smem_u32(b);
+        for (int j = 0; j < K / 16; j++)
+            mma_bf16(T0 + d, smem_desc(a0 + 256u * j, 128u, 16u * K), smem_desc(b0 + 256u * j, 128u, 16u * K), idesc,
+                     acc || j > 0);
+    };
+    auto end_mma = [&]() {   // every thread waits for the committed MMAs; uniform over the CTA
+        const bool done = mbar_wait(&S.bar, phase);
+        phase ^= 1;
+        ok = __syncthreads_and(done) && ok;
+        fence_after_sync();
+    };
+    float gw3 = 0.0f, gb[3] = {0.0f, 0.0f, 0.0f}, gb3 = 0.0f, lsum = 0.0f;   // column sums of this thread's half rows
+    // sum over 64 rows (this half's) of row `col` of zt, optionally weighted by dy
+    auto col_sum = [&](bool weighted) {
+        const int col = tid & 127, r0 = 64 * (tid >> 7);
         float s = 0.0f;
-        for (int q = 0; q < 4; q++) {
-            h[q] = __bfloat162float(H2[r * HID + 4 * lane + q]);
-            s += h[q] * w3[q];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const uint4 v = *reinterpret_cast<const uint4*>(at(S.zt, col, r0 + 8 * q, TM));
+            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+            for (int z = 0; z < 4; z++) {
+                const float2 f = __bfloat1622float2(h[z]);
+                if (weighted) s += f.x * S.dy[r0 + 8 * q + 2 * z] + f.y * S.dy[r0 + 8 * q + 2 * z + 1];
+                else s += f.x + f.y;
+            }
         }
-        for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        const float yr = s + b3;
-        if (lane == 0 && y) y[r] = yr;
-        if (!t) continue;
-        const float e = yr - t[cur ? (cur[0] + r) % n_total : r];
-        const float dy = 2.0f * e / (float)n;
-        if (lane == 0) {
-            lsum += e * e;
-            atomicAdd(&sw[HID], dy);
+        return s;
+    };
+    const long long ntile = (n + TM - 1) / TM;
+    bool first = true;
+    for (long long tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x) {
+        const long long m0 = tile * TM;
+        load_image(S.wa, img + IW1, HID * HID);
+        load_image(S.wb, img + IW2, HID * HID);
+        // inputs: two threads per row, 16 columns each
+        {
+            const int r = tid >> 1, c0 = 16 * (tid & 1);
+            const bool in = m0 + r < n;
+            long long src = m0 + r;
+            if (cur && in) src = (base + src) % n_total;
+            __align__(16) __nv_bfloat16 o[16];
+#pragma unroll
+            for (int k = 0; k < 16; k++)
+                o[k] = __float2bfloat16(in && c0 + k < n_in ? x[src * n_in + c0 + k] : 0.0f);
+#pragma unroll
+            for (int q = 0; q < 2; q++)
+                *reinterpret_cast<uint4*>(at(S.x, r, c0 + 8 * q, NIN)) = reinterpret_cast<const uint4*>(o)[q];
+            if (GRAD)
+#pragma unroll
+                for (int k = 0; k < 16; k++) *reinterpret_cast<__nv_bfloat16*>(at(S.xt, c0 + k, r, TM)) = o[k];
         }
-        for (int q = 0; q < 4; q++) {
-            dZ2[r * HID + 4 * lane + q] = __float2bfloat16(h[q] > 0.0f ? dy * w3[q] : 0.0f);
-            atomicAdd(&sw[4 * lane + q], dy * h[q]);
+        const bool live = m0 + m < n;
+        cp_async_wait<2>();   // W0 (first tile)
+        begin_mma();
+        if (tid == 0) {
+            issue(D, S.x, S.w0, NIN, HID, false);
+            mma_commit(&S.bar);
+        }
+        end_mma();
+        // hidden layers 0 and 1: bias, ReLU, BF16; the ReLU masks stay in registers
+        uint32_t mask[3][2];
+#pragma unroll
+        for (int layer = 0; layer < 2; layer++) {
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                const int c0 = 64 * half + 32 * c;
+                float v[32];
+                tmem_ld32(T0 + D + tlane + (uint32_t)c0, v);
+                __align__(16) __nv_bfloat16 o[32];
+                uint32_t mk = 0;
+#pragma unroll
+                for (int k = 0; k < 32; k++) {
+                    o[k] = __float2bfloat16(live ? fmaxf(v[k] + S.bias[layer][c0 + k], 0.0f) : 0.0f);
+                    mk |= (__bfloat162float(o[k]) > 0.0f ? 1u : 0u) << k;
+                }
+                mask[layer][c] = mk;
+                if (GRAD) {
+                    put_tile(S.row, layer == 0 ? S.h0t : S.h1t, m, c0, o);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        *reinterpret_cast<uint4*>(at(S.row, m, c0 + 8 * q, HID)) = reinterpret_cast<const uint4*>(o)[q];
+                }
+            }
+            if (layer == 0) cp_async_wait<1>();   // W1
+            else cp_async_wait<0>();              // W2 (and whatever was loaded behind it)
+            begin_mma();
+            if (tid == 0) {
+                issue(D, S.row, layer == 0 ? S.wa : S.wb, HID, HID, false);
+                mma_commit(&S.bar);
+            }
+            end_mma();
+        }
+        if (GRAD) load_image(S.wa, img + IW2T, HID * HID);   // W1 has been consumed
+        // layer 2 and the head
+        float ys = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const int c0 = 64 * half + 32 * c;
+            float v[32];
+            tmem_ld32(T0 + D + tlane + (uint32_t)c0, v);
+            __align__(16) __nv_bfloat16 o[32];
+            uint32_t mk = 0;
+#pragma unroll
+            for (int k = 0; k < 32; k++) {
+                o[k] = __float2bfloat16(live ? fmaxf(v[k] + S.bias[2][c0 + k], 0.0f) : 0.0f);
+                const float h = __bfloat162float(o[k]);
+                mk |= (h > 0.0f ? 1u : 0u) << k;
+                ys += h * S.w3[c0 + k];
+            }
+            mask[2][c] = mk;
+            if (GRAD) put_tile(nullptr, S.zt, m, c0, o);
+        }
+        S.ypart[half][m] = ys;
+        if (GRAD) load_image(S.wb, img + IW1T, HID * HID);   // W2 has been consumed
+        __syncthreads();
+        if (half == 0) {
+            const float yr = S.ypart[0][m] + S.ypart[1][m] + b3;
+            if (y && live) y[m0 + m] = yr;
+            if (GRAD) {
+                long long src = m0 + m;
+                if (cur && live) src = (base + src) % n_total;
+                const float e = live ? yr - t[src] : 0.0f;
+                const float d = 2.0f * e / (float)n;
+                S.dy[m] = d;
+                gb3 += d;
+                lsum += e * e;
+            }
+        }
+        if (!GRAD) {
+            __syncthreads();   // ypart and the operands are rewritten by the next tile
+            continue;
+        }
+        __syncthreads();
+        gw3 += col_sum(true);
+        const float dy = S.dy[m];
+        __syncthreads();   // H2 has been read
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const int c0 = 64 * half + 32 * c;
+            __align__(16) __nv_bfloat16 o[32];
+#pragma unroll
+            for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mask[2][c] >> k) & 1u ? dy * S.w3[c0 + k] : 0.0f);
+            put_tile(S.row, S.zt, m, c0, o);
+        }
+        // layers 2 and 1: weight gradient and input gradient in one batch
+#pragma unroll
+        for (int layer = 2; layer >= 1; layer--) {
+            if (layer == 2) cp_async_wait<1>();   // W2^T
+            else cp_async_wait<0>();              // W1^T
+            begin_mma();
+            if (tid == 0) {
+                issue(D, S.row, layer == 2 ? S.wa : S.wb, HID, HID, false);
+                issue(layer == 2 ? DW2 : DW1, S.zt, layer == 2 ? S.h1t : S.h0t, TM, HID, !first);
+                mma_commit(&S.bar);
+            }
+            gb[layer] += col_sum(false);   // beside the MMAs: both only read zt
+            end_mma();
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                const int c0 = 64 * half + 32 * c;
+                float v[32];
+                tmem_ld32(T0 + D + tlane + (uint32_t)c0, v);
+                __align__(16) __nv_bfloat16 o[32];
+#pragma unroll
+                for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mask[layer - 1][c] >> k) & 1u ? v[k] : 0.0f);
+                put_tile(layer == 2 ? S.row : nullptr, S.zt, m, c0, o);
+            }
+        }
+        begin_mma();
+        if (tid == 0) {
+            issue(DW0, S.zt, S.xt, TM, NIN, !first);
+            mma_commit(&S.bar);
+        }
+        gb[0] += col_sum(false);
+        end_mma();
+        first = false;
+    }
+    cp_async_wait<0>();
+    if (GRAD) {
+        // this CTA's partial gradient: the accumulators, then the column sums
+        float* g = part + (long long)blockIdx.x * PSTRIDE;
+        if (ok) {
+            for (int layer = 0; layer < 3; layer++) {
+                const int K = layer == 0 ? NIN : HID;
+                const uint32_t d = layer == 0 ? DW0 : (layer == 1 ? DW1 : DW2);
+                float* gw = g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2)) + (long long)m * K;
+                for (int c = 0; c < 2; c++) {
+                    const int c0 = K == HID ? 64 * half + 32 * c : 0;
+                    if (K == NIN && (half || c)) continue;   // warp-uniform
+                    float v[32];
+                    tmem_ld32(T0 + d + tlane + (uint32_t)c0, v);
+#pragma unroll
+                    for (int q = 0; q < 8; q++)
+                        reinterpret_cast<float4*>(gw + c0)[q] =
+                            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                }
+            }
+        }
+        const int col = tid & 127;
+        const float sums[4] = {gb[0], gb[1], gb[2], gw3};
+        const long long to[4] = {OB0, OB1, OB2, OW3};
+        for (int k = 0; k < 4; k++) {
+            __syncthreads();
+            if (tid >= 128) S.red[col] = sums[k];
+            __syncthreads();
+            if (tid < 128) g[to[k] + col] = sums[k] + S.red[col];
+        }
+        for (int off = 16; off; off >>= 1) {
+            gb3 += __shfl_xor_sync(0xffffffffu, gb3, off);
+            lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+        }
+        __syncthreads();
+        if (half == 0 && lane == 0) {
+            S.red[quad] = gb3;
+            S.lred[quad] = lsum;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            g[OB3] = S.red[0] + S.red[1] + S.red[2] + S.red[3];
+            g[NPARAM] = (S.lred[0] + S.lred[1] + S.lred[2] + S.lred[3]) / (float)n;
+            // one more Adam step: read by k_adam only
+            if (cur && blockIdx.x == 0) cur[1] += 1;
         }
     }
+    if (!ok && tid == 0) atomicCAS(err, 0, (int)RPD_E_TIMEOUT);
+    fence_before_sync();
     __syncthreads();
-    if (!t) return;
-    for (int k = threadIdx.x; k < HID; k += blockDim.x) atomicAdd(&g[OW3 + k], sw[k]);
-    if (threadIdx.x == 0) atomicAdd(&g[OB3], sw[HID]);
-    if (lane == 0 && lsum != 0.0f) atomicAdd(loss, lsum / (float)n);
+    if (warp == 0) tmem_dealloc(T0, 512);
 }
 
-// Bias gradient: column sums of dZ [n][HID] into g[off .. off + HID).
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ dZ, long long n, float* __restrict__ g, long long off) {
-    const int c = threadIdx.x;   // blockDim.x == HID
-    float s = 0.0f;
-    for (long long r = blockIdx.x; r < n; r += gridDim.x) s += __bfloat162float(dZ[r * HID + c]);
-    atomicAdd(&g[off + c], s);
+// BF16 value of weight i of the master vector into its tile images.
+__device__ __forceinline__ void put_weight(__nv_bfloat16* img, long long i, float w) {
+    const __nv_bfloat16 b = __float2bfloat16(w);
+    if (i < OB0) {
+        *reinterpret_cast<__nv_bfloat16*>(at(img + IW0, (int)(i / NIN), (int)(i % NIN), NIN)) = b;
+    } else if (i >= OW1 && i < OB1) {
+        const int r = (int)((i - OW1) / HID), c = (int)((i - OW1) % HID);
+        *reinterpret_cast<__nv_bfloat16*>(at(img + IW1, r, c, HID)) = b;
+        *reinterpret_cast<__nv_bfloat16*>(at(img + IW1T, c, r, HID)) = b;
+    } else if (i >= OW2 && i < OB2) {
+        const int r = (int)((i - OW2) / HID), c = (int)((i - OW2) % HID);
+        *reinterpret_cast<__nv_bfloat16*>(at(img + IW2, r, c, HID)) = b;
+        *reinterpret_cast<__nv_bfloat16*>(at(img + IW2T, c, r, HID)) = b;
+    }
 }
 
-// Adam step on the FP32 master parameters; step number cur[1] + 1 (bias
-// corrections 1 - b^step).
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       long long n, float lr, float b1, float b2, float eps, const long long* __restrict__ cur) {
+__global__ void k_cast_weights(const float* __restrict__ p, __nv_bfloat16* __restrict__ img) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float step = (float)(cur[1] + 1);
+    if (i < NPARAM) put_weight(img, i, p[i]);
+}
+
+// Sum of the CTAs' partial gradients, in CTA order, into g; loss at NPARAM.
+__device__ __forceinline__ float part_sum(const float* __restrict__ part, int np, long long i) {
+    float s = 0.0f;
+#pragma unroll 8
+    for (int c = 0; c < np; c++) s += part[(long long)c * PSTRIDE + i];
+    return s;
+}
+
+__global__ void k_grad_sum(const float* __restrict__ part, int np, float* __restrict__ g, float* __restrict__ loss) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < NPARAM) g[i] = part_sum(part, np, i);
+    if (i == NPARAM) *loss = part_sum(part, np, i);
+}
+
+// Adam step on the FP32 master parameters: the gradient summed from the
+// partials, step number cur[1] (bias corrections 1 - b^step), the BF16 tile
+// images of the new weights, and the next batch's first row.
+__global__ void k_adam(float* __restrict__ p, const float* __restrict__ part, int np, float* __restrict__ g,
+                       float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ img,
+                       float* __restrict__ loss, float lr, float b1, float b2, float eps, long long* __restrict__ cur,
+                       long long b, long long n_total) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) cur[0] = (cur[0] + b) % n_total;   // read by k_mlp_step only
+    if (i == NPARAM) *loss = part_sum(part, np, i);
+    if (i >= NPARAM) return;
+    const float gi = part_sum(part, np, i);
+    const float step = (float)cur[1];
     const float c1 = 1.0f - powf(b1, step), c2 = 1.0f - powf(b2, step);
-    const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi, vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    g[i] = gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = w;
+    put_weight(img, i, w);
 }
 
 }  // namespace
@@ -420,48 +555,39 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 struct rpd_mlp {
     cudaStream_t stream = nullptr;
     int n_in = 0;
+    char* mem = nullptr;  // one allocation for everything below
     float* p = nullptr;   // FP32 master parameters
     float* g = nullptr;   // gradient
     float* m = nullptr;   // Adam moments
     float* v = nullptr;
-    __nv_bfloat16* Wb = nullptr;   // BF16 copies of the three hidden layers
+    __nv_bfloat16* img = nullptr;   // BF16 tile images of the hidden layers' weights
     int* err = nullptr;
     float* loss = nullptr;
     long long step = 0;
-    long long* cur = nullptr;          // device: [next batch row, Adam steps taken]
-    cudaStream_t tstream = nullptr;    // private stream the training steps are captured on
-    cudaEvent_t tev[2] = {nullptr, nullptr};
-    long long cap = 0;    // rows of the activation buffers (multiple of 128)
-    __nv_bfloat16 *X = nullptr, *H0 = nullptr, *H1 = nullptr, *H2 = nullptr, *D2 = nullptr, *D1 = nullptr,
-                  *D0 = nullptr;
-    __nv_bfloat16* W0() const { return Wb; }
-    __nv_bfloat16* W1() const { return Wb + HID * NIN; }
-    __nv_bfloat16* W2() const { return Wb + HID * NIN + HID * HID; }
+    long long* cur = nullptr;       // device: [next batch row, Adam steps taken]
+    float* part = nullptr;          // partial gradients, one row per CTA
+    int part_rows = 0;
 };
 
 namespace {
 
-size_t tile_smem() { return sizeof(TileSmem) + 1024; }
+size_t step_smem() { return sizeof(StepSmem) + 1024; }
 
-void free_acts(rpd_mlp* q) {
-    for (__nv_bfloat16* b : {q->X, q->H0, q->H1, q->H2, q->D2, q->D1, q->D0})
-        if (b) cudaFree(b);
-    q->X = q->H0 = q->H1 = q->H2 = q->D2 = q->D1 = q->D0 = nullptr;
-    q->cap = 0;
-}
+int step_ctas(long long n) { return (int)std::min<long long>((n + TM - 1) / TM, MAX_CTAS); }
 
-rpd_status ensure_acts(rpd_mlp* q, long long n) {
-    const long long need = ((n + TM - 1) / TM) * TM;
-    if (need <= q->cap) return RPD_OK;
-    free_acts(q);
-    __nv_bfloat16** bufs[7] = {&q->X, &q->H0, &q->H1, &q->H2, &q->D2, &q->D1, &q->D0};
-    for (int k = 0; k < 7; k++)
-        if (cudaMalloc(bufs[k], sizeof(__nv_bfloat16) * need * (k == 0 ? NIN : HID)) != cudaSuccess) {
-            cudaGetLastError();
-            free_acts(q);
-            return RPD_E_OOM;
-        }
-    q->cap = need;
+rpd_status ensure_part(rpd_mlp* q, long long n) {
+    const int need = step_ctas(n);
+    if (need <= q->part_rows) return RPD_OK;
+    if (q->part) cudaFreeAsync(q->part, q->stream);
+    q->part = nullptr;
+    q->part_rows = 0;
+    if (cudaMallocFromPoolAsync((void**)&q->part, sizeof(float) * PSTRIDE * need, library_pool(), q->stream) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        q->part = nullptr;
+        return RPD_E_OOM;
+    }
+    q->part_rows = need;
     return RPD_OK;
 }
 
@@ -476,50 +602,23 @@ rpd_status launch_check(rpd_mlp* q) {
     return e ? (rpd_status)e : RPD_OK;
 }
 
-// Forward through the three hidden layers (tensor cores) and the head.  With
-// n_total > 0 the n rows are the training batch that starts at the device
-// cursor's row of the n_total data rows (x and t are the whole data).
-void forward(rpd_mlp* q, const float* x, long long n, float* y, const float* t, long long n_total = 0) {
-    cudaStream_t s = q->stream;
-    const unsigned tiles = (unsigned)((n + TM - 1) / TM);
-    const size_t sm = tile_smem();
-    if (n_total > 0)
-        k_to_bf16_batch<<<nblk(q->cap * NIN, 256), 256, 0, s>>>(x, n_total, q->n_in, n, q->cap, q->cur, q->X);
+// Forward, and with t backward into the partial gradients.  With n_total > 0
+// the n rows are the training batch that starts at the device cursor's row of
+// the n_total data rows (x and t are the whole data).
+void run_step(rpd_mlp* q, const float* x, const float* t, long long n, float* y, long long n_total = 0) {
+    const int ctas = step_ctas(n);
+    long long* cur = n_total > 0 ? q->cur : nullptr;
+    if (t)
+        k_mlp_step<true><<<ctas, STEP_THREADS, step_smem(), q->stream>>>(x, t, n, q->n_in, n_total, cur, q->p, q->img,
+                                                                          y, q->part, q->err);
     else
-        k_to_bf16<<<nblk(q->cap * NIN, 256), 256, 0, s>>>(x, n, q->n_in, q->cap, q->X);
+        k_mlp_step<false><<<ctas, STEP_THREADS, step_smem(), q->stream>>>(x, t, n, q->n_in, n_total, cur, q->p, q->img,
+                                                                           y, q->part, q->err);
     note_launch();
-    k_mlp_fwd<<<tiles, MLP_THREADS, sm, s>>>(q->X, n, NIN, q->W0(), q->p + OB0, HID, q->H0, q->err);
-    k_mlp_fwd<<<tiles, MLP_THREADS, sm, s>>>(q->H0, n, HID, q->W1(), q->p + OB1, HID, q->H1, q->err);
-    k_mlp_fwd<<<tiles, MLP_THREADS, sm, s>>>(q->H1, n, HID, q->W2(), q->p + OB2, HID, q->H2, q->err);
-    for (int k = 0; k < 3; k++) note_launch();
-    if (t) {
-        cudaMemsetAsync(q->g, 0, sizeof(float) * NPARAM, s);
-        cudaMemsetAsync(q->loss, 0, sizeof(float), s);
-    }
-    k_head<<<152 * 4, 256, 0, s>>>(q->H2, n, q->p, y, t, q->D2, q->g, q->loss, n_total > 0 ? q->cur : nullptr,
-                                   n_total);
-    note_launch();
-}
-
-// Backward from dZ2 (written by the head): every gradient into q->g.
-void backward(rpd_mlp* q, long long n) {
-    cudaStream_t s = q->stream;
-    const unsigned tiles = (unsigned)((n + TM - 1) / TM);
-    const size_t sm = tile_smem();
-    const unsigned bg = (unsigned)std::min<long long>(n, 152 * 8);
-    k_mlp_dw<<<tiles, MLP_THREADS, sm, s>>>(q->D2, n, HID, q->H1, HID, q->g + OW2, q->err);
-    k_bias_grad<<<bg, HID, 0, s>>>(q->D2, n, q->g, OB2);
-    k_mlp_dx<<<tiles, MLP_THREADS, sm, s>>>(q->D2, n, HID, q->W2(), HID, q->H1, q->D1, q->err);
-    k_mlp_dw<<<tiles, MLP_THREADS, sm, s>>>(q->D1, n, HID, q->H0, HID, q->g + OW1, q->err);
-    k_bias_grad<<<bg, HID, 0, s>>>(q->D1, n, q->g, OB1);
-    k_mlp_dx<<<tiles, MLP_THREADS, sm, s>>>(q->D1, n, HID, q->W1(), HID, q->H0, q->D0, q->err);
-    k_mlp_dw<<<tiles, MLP_THREADS, sm, s>>>(q->D0, n, HID, q->X, NIN, q->g + OW0, q->err);
-    k_bias_grad<<<bg, HID, 0, s>>>(q->D0, n, q->g, OB0);
-    for (int k = 0; k < 8; k++) note_launch();
 }
 
 void cast_weights(rpd_mlp* q) {
-    k_cast_weights<<<nblk(HID * HID, 256), 256, 0, q->stream>>>(q->p, q->W0(), q->W1(), q->W2());
+    k_cast_weights<<<nblk(NPARAM, 256), 256, 0, q->stream>>>(q->p, q->img);
     note_launch();
 }
 
@@ -534,25 +633,30 @@ rpd_status rpd_mlp_create(int32_t n_in, uint64_t seed, void* cuda_stream, rpd_ml
     rpd_mlp* q = new rpd_mlp();
     q->stream = (cudaStream_t)cuda_stream;
     q->n_in = n_in;
-    const size_t sm = tile_smem();
-    bool ok = cudaFuncSetAttribute(k_mlp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
-              cudaFuncSetAttribute(k_mlp_dx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
-              cudaFuncSetAttribute(k_mlp_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
-    ok = ok && cudaMalloc(&q->p, sizeof(float) * NPARAM) == cudaSuccess &&
-         cudaMalloc(&q->g, sizeof(float) * NPARAM) == cudaSuccess &&
-         cudaMalloc(&q->m, sizeof(float) * NPARAM) == cudaSuccess &&
-         cudaMalloc(&q->v, sizeof(float) * NPARAM) == cudaSuccess &&
-         cudaMalloc(&q->Wb, sizeof(__nv_bfloat16) * (HID * NIN + 2 * HID * HID)) == cudaSuccess &&
-         cudaMalloc(&q->err, sizeof(int)) == cudaSuccess && cudaMalloc(&q->loss, sizeof(float)) == cudaSuccess &&
-         cudaMalloc(&q->cur, 2 * sizeof(long long)) == cudaSuccess &&
-         cudaStreamCreateWithFlags(&q->tstream, cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&q->tev[0], cudaEventDisableTiming) == cudaSuccess &&
-         cudaEventCreateWithFlags(&q->tev[1], cudaEventDisableTiming) == cudaSuccess;
+    const int sm = (int)step_smem();
+    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t fb = al(sizeof(float) * NPARAM), ib = al(sizeof(__nv_bfloat16) * NIMG);
+    cudaMemPool_t pool = library_pool();
+    const bool ok =
+        pool && cudaFuncSetAttribute(k_mlp_step<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) == cudaSuccess &&
+        cudaFuncSetAttribute(k_mlp_step<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) == cudaSuccess &&
+        cudaMallocFromPoolAsync((void**)&q->mem, 4 * fb + ib + 3 * 256, pool, q->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
+        q->mem = nullptr;
         rpd_mlp_destroy(q);
         return RPD_E_OOM;
     }
+    char* at = q->mem;
+    for (float** b : {&q->p, &q->g, &q->m, &q->v}) {
+        *b = (float*)at;
+        at += fb;
+    }
+    q->img = (__nv_bfloat16*)at;
+    at += ib;
+    q->err = (int*)at;
+    q->loss = (float*)(at + 256);
+    q->cur = (long long*)(at + 512);
     // He-uniform weights from a 64-bit xorshift stream of the seed; zero biases
     std::vector<float> h(NPARAM, 0.0f);
     unsigned long long st = seed * 0x9E3779B97F4A7C15ull + 0xD1B54A32D192ED03ull;
@@ -571,7 +675,7 @@ rpd_status rpd_mlp_create(int32_t n_in, uint64_t seed, void* cuda_stream, rpd_ml
     cudaMemcpyAsync(q->p, h.data(), sizeof(float) * NPARAM, cudaMemcpyHostToDevice, q->stream);
     cudaMemsetAsync(q->m, 0, sizeof(float) * NPARAM, q->stream);
     cudaMemsetAsync(q->v, 0, sizeof(float) * NPARAM, q->stream);
-    cudaMemsetAsync(q->err, 0, sizeof(int), q->stream);
+    cudaMemsetAsync(q->err, 0, 3 * 256, q->stream);   // err, loss, cur
     cast_weights(q);
     const rpd_status s = launch_check(q);
     if (s != RPD_OK) {
@@ -601,16 +705,16 @@ rpd_status rpd_mlp_set_params(rpd_mlp* q, const float* d_in, int64_t n) {
 rpd_status rpd_mlp_forward(rpd_mlp* q, const float* d_x, int64_t n, float* d_y) {
     if (!q || n < 0 || (n > 0 && (!d_x || !d_y))) return RPD_E_INVALID;
     if (n == 0) return RPD_OK;
-    TRY_M(ensure_acts(q, n));
-    forward(q, d_x, n, d_y, nullptr);
+    run_step(q, d_x, nullptr, n, d_y);
     return launch_check(q);
 }
 
 rpd_status rpd_mlp_grad(rpd_mlp* q, const float* d_x, const float* d_t, int64_t n, float* d_grad, float* h_loss) {
     if (!q || n < 1 || !d_x || !d_t) return RPD_E_INVALID;
-    TRY_M(ensure_acts(q, n));
-    forward(q, d_x, n, nullptr, d_t);
-    backward(q, n);
+    TRY_M(ensure_part(q, n));
+    run_step(q, d_x, d_t, n, nullptr);
+    k_grad_sum<<<nblk(NPARAM + 1, 256), 256, 0, q->stream>>>(q->part, step_ctas(n), q->g, q->loss);
+    note_launch();
     if (d_grad) cudaMemcpyAsync(d_grad, q->g, sizeof(float) * NPARAM, cudaMemcpyDeviceToDevice, q->stream);
     if (h_loss) cudaMemcpyAsync(h_loss, q->loss, sizeof(float), cudaMemcpyDeviceToHost, q->stream);
     return launch_check(q);
@@ -620,46 +724,18 @@ rpd_status rpd_mlp_train(rpd_mlp* q, const float* d_x, const float* d_t, int64_t
                          float lr, float* h_loss) {
     if (!q || n < 1 || !d_x || !d_t || steps < 0 || batch < 1 || !(lr > 0)) return RPD_E_INVALID;
     const long long b = std::min<long long>(batch, n);
-    TRY_M(ensure_acts(q, b));
     if (steps > 0) {
+        TRY_M(ensure_part(q, b));
         // consecutive batches of the (caller-shuffled) data, wrapping around:
-        // batch rows chosen on the device from the cursor, so one step's
-        // launches are captured once as a CUDA graph and replayed
+        // the batch's rows come from the device cursor.  Two launches a step,
+        // issued well ahead of the device (a step takes longer than they do).
         const long long c0[2] = {0, q->step};
         cudaMemcpyAsync(q->cur, c0, sizeof(c0), cudaMemcpyHostToDevice, q->stream);
-        cudaEventRecord(q->tev[0], q->stream);
-        cudaStreamWaitEvent(q->tstream, q->tev[0], 0);
-        cudaStream_t user = q->stream;
-        q->stream = q->tstream;
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
-        const long long l0 = rpd_launch_count();
-        bool ok = cudaStreamBeginCapture(q->tstream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) {
-            forward(q, d_x, b, nullptr, d_t, n);
-            backward(q, b);
-            k_adam<<<nblk(NPARAM, 256), 256, 0, q->tstream>>>(q->p, q->g, q->m, q->v, NPARAM, lr, 0.9f, 0.999f, 1e-8f,
-                                                               q->cur);
+        for (int it = 0; it < steps; it++) {
+            run_step(q, d_x, d_t, b, nullptr, n);
+            k_adam<<<nblk(NPARAM + 1, 256), 256, 0, q->stream>>>(q->p, q->part, step_ctas(b), q->g, q->m, q->v, q->img,
+                                                                  q->loss, lr, 0.9f, 0.999f, 1e-8f, q->cur, b, n);
             note_launch();
-            cast_weights(q);
-            k_cursor_advance<<<1, 1, 0, q->tstream>>>(q->cur, b, n);
-            note_launch();
-            ok = cudaStreamEndCapture(q->tstream, &graph) == cudaSuccess && graph;
-        }
-        const long long per_step = rpd_launch_count() - l0;
-        ok = ok && cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
-        for (int it = 0; ok && it < steps; it++) ok = cudaGraphLaunch(exec, q->tstream) == cudaSuccess;
-        if (ok)   // the captured launches ran `steps` times, not once
-            for (long long k = 0; k < per_step * (steps - 1); k++) note_launch();
-        cudaEventRecord(q->tev[1], q->tstream);
-        q->stream = user;
-        cudaStreamWaitEvent(q->stream, q->tev[1], 0);
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        if (!ok) {
-            cudaGetLastError();
-            cudaStreamSynchronize(q->tstream);
-            return RPD_E_CUDA;
         }
         q->step += steps;
     }
@@ -669,15 +745,9 @@ rpd_status rpd_mlp_train(rpd_mlp* q, const float* d_x, const float* d_t, int64_t
 
 void rpd_mlp_destroy(rpd_mlp* q) {
     if (!q) return;
-    if (q->stream) cudaStreamSynchronize(q->stream);
-    free_acts(q);
-    if (q->tstream) cudaStreamSynchronize(q->tstream);
-    for (void* b : {(void*)q->p, (void*)q->g, (void*)q->m, (void*)q->v, (void*)q->Wb, (void*)q->err, (void*)q->loss,
-                    (void*)q->cur})
-        if (b) cudaFree(b);
-    for (cudaEvent_t e : q->tev)
-        if (e) cudaEventDestroy(e);
-    if (q->tstream) cudaStreamDestroy(q->tstream);
+    if (q->part) cudaFreeAsync(q->part, q->stream);
+    if (q->mem) cudaFreeAsync(q->mem, q->stream);
+    cudaStreamSynchronize(q->stream);
     cudaGetLastError();
     delete q;
 }
