@@ -27,10 +27,9 @@
 //    distance is then v.(s - c_1) - r_1.
 //
 // FP32 arithmetic on coordinates relative to mesh vertex 0 (the distances
-// only decide a threshold); one thread per sample, the samples in Morton
-// order, the Morton-sorted primitives staged through shared memory in tiles,
-// scanned outwards from the block's position and skipped when their bounding
-// ball is already farther than every sample's best distance.
+// only decide a threshold); one lane per sample, the samples and the
+// primitives in Morton order; a warp culls tiles of 32 primitives, then single
+// primitives, by bounding balls (see k_env_dist).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -41,8 +40,9 @@ namespace {
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-constexpr int ENV_THREADS = 256;
-constexpr int ENV_TILE = 64;    // primitives per shared-memory tile (64 measured fastest of 64, 128, 256)
+constexpr int ENV_THREADS = 128;
+constexpr int ENV_TILE = 64;    // primitives per tile of the tie order (k_env_dist)
+constexpr int ENV_BLOCK = 256;  // samples that share a start of the tie order
 
 // A primitive: up to three spheres (x, y, z, r) and its kind (1, 2, 3).
 struct Prim {
@@ -190,132 +190,215 @@ __global__ void k_env_sample_keys(const double* __restrict__ samples, long long 
     idx[i] = (uint32_t)i;
 }
 
+// Primitives in Morton order, each with a bounding ball of its spheres (every
+// point of its envelope is within the radius of the centre), and the bounding
+// ball of each 32 of them (one warp).
 __global__ void k_env_gather(const Prim* __restrict__ in, const uint32_t* __restrict__ order, long long n,
-                             Prim* __restrict__ out) {
+                             Prim* __restrict__ out, float4* __restrict__ balls, float4* __restrict__ tiles) {
+    const unsigned FULL = 0xffffffffu;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = in[order[i]];
+    if ((i & ~31ll) >= n) return;   // warp-uniform
+    float4 b = make_float4(0, 0, 0, -INFINITY);
+    if (i < n) {
+        const Prim q = in[order[i]];
+        out[i] = q;
+        for (int z = 0; z < q.kind; z++) {
+            b.x += q.s[z].x;
+            b.y += q.s[z].y;
+            b.z += q.s[z].z;
+        }
+        const float w = 1.0f / (float)q.kind;
+        b.x *= w;
+        b.y *= w;
+        b.z *= w;
+        for (int z = 0; z < q.kind; z++) {
+            const float dx = q.s[z].x - b.x, dy = q.s[z].y - b.y, dz = q.s[z].z - b.z;
+            b.w = fmaxf(b.w, sqrtf(dx * dx + dy * dy + dz * dz) + q.s[z].w);
+        }
+        b.w *= 1.0f + 0x1p-18f;
+        balls[i] = b;
+    }
+    const int m = (int)(n - (i & ~31ll) < 32 ? n - (i & ~31ll) : 32);
+    float sx = b.x, sy = b.y, sz = b.z;
+    for (int off = 16; off; off >>= 1) {
+        sx += __shfl_xor_sync(FULL, sx, off);
+        sy += __shfl_xor_sync(FULL, sy, off);
+        sz += __shfl_xor_sync(FULL, sz, off);
+    }
+    const float cx = sx / (float)m, cy = sy / (float)m, cz = sz / (float)m;
+    const float dx = b.x - cx, dy = b.y - cy, dz = b.z - cz;
+    float r = sqrtf(dx * dx + dy * dy + dz * dz) + b.w;   // -inf past the end
+    for (int off = 16; off; off >>= 1) r = fmaxf(r, __shfl_xor_sync(FULL, r, off));
+    if ((i & 31) == 0) tiles[i >> 5] = make_float4(cx, cy, cz, r * (1.0f + 0x1p-18f));
 }
 
-// Bounding ball (centre, radius) of each tile of sorted primitives: every
-// point of a primitive's envelope lies within (distance to the ball centre
-// + the sphere radius) of it.
-__global__ void k_env_tiles(const Prim* __restrict__ p, long long n, float4* __restrict__ tiles) {
-    const long long t = blockIdx.x;
-    const long long b = t * ENV_TILE, e = b + ENV_TILE < n ? b + ENV_TILE : n;
-    __shared__ float sx, sy, sz;
-    if (threadIdx.x == 0) {
-        double ax = 0, ay = 0, az = 0;
-        for (long long i = b; i < e; i++) {
-            ax += p[i].s[0].x;
-            ay += p[i].s[0].y;
-            az += p[i].s[0].z;
-        }
-        const double m = (double)(e - b);
-        sx = (float)(ax / m);
-        sy = (float)(ay / m);
-        sz = (float)(az / m);
+// First position whose key is >= key (n if there is none); the whole warp,
+// 32 probes a step.
+__device__ __forceinline__ long long warp_lower_bound(const uint64_t* __restrict__ keys, long long n, uint64_t key) {
+    const int lane = threadIdx.x & 31;
+    long long lo = 0, hi = n;   // the answer is in [lo, hi]
+    while (lo < hi) {
+        const long long pos = lo + (hi - lo) * lane / 32;   // < hi, ascending over the lanes
+        const int below = __popc(__ballot_sync(0xffffffffu, keys[pos] < key));
+        const long long at = __shfl_sync(0xffffffffu, pos, below > 0 ? below - 1 : 0);
+        const long long up = __shfl_sync(0xffffffffu, pos, below < 32 ? below : 31);
+        if (below < 32) hi = up;
+        if (below > 0) lo = at + 1;
     }
-    __syncthreads();
-    float r = 0;
-    for (long long i = b + threadIdx.x; i < e; i += blockDim.x)
-        for (int z = 0; z < p[i].kind; z++) {
-            const float4 c = p[i].s[z];
-            const float dx = c.x - sx, dy = c.y - sy, dz = c.z - sz;
-            r = fmaxf(r, sqrtf(dx * dx + dy * dy + dz * dz) + c.w);
-        }
-    for (int off = 16; off; off >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, off));
-    __shared__ float wr[32];
-    if ((threadIdx.x & 31) == 0) wr[threadIdx.x >> 5] = r;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); k++) m = fmaxf(m, wr[k]);
-        tiles[t] = make_float4(sx, sy, sz, m * 1.0001f + 1e-6f);
-    }
+    return lo;
 }
 
-// One thread per sample, the samples taken in Morton order (sorder) so that a
-// block's samples are close together; the block starts at the tile of
-// primitives whose Morton codes follow its first sample's and alternates
-// outwards (t0, t0 + 1, t0 - 1, ...), so the best distances shrink early and
-// far tiles fail the ball test.
+// Order of floats as unsigned integers (no NaN).
+__device__ __forceinline__ unsigned float_key(float f) {
+    const unsigned u = __float_as_uint(f);
+    return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float key_float(unsigned k) {
+    return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
+}
+
+// One block per 32 samples in Morton order: a lane is a sample in each of the
+// block's warps, and the warps share out the tiles of 32 primitives.  Tiles
+// are tested 32 at a time (one per lane) against the box of the samples and
+// the largest of their best distances, R, then against each sample's own best
+// distance; the primitives of an open tile likewise, and each that is left is
+// evaluated by all lanes.  Groups of 32 tiles are taken outwards from the
+// block's own place in the Morton order, so the distances fall early; the warps
+// share them through shared memory.
+//
+// What bounds it: latency and issue on the primitives that a ball cannot
+// reject (those whose envelope nearly touches a sample); the samples alone are
+// too few warps to hide it, hence several per packet.  Culling by blocks of
+// 256 samples and tiles of 64 primitives, with three block barriers per tile,
+// evaluated every primitive of a tile for all 256: 5.8 ms for 58 k samples
+// and 45 k primitives.
+//
+// Equal distances go to the primitive that comes first in an order fixed by
+// the sample's place: tiles of 64 outwards (t0, t0 + 1, t0 - 1, ...) from t0, the
+// tile where the codes reach that of the first of the sample's 256.
 __global__ void __launch_bounds__(ENV_THREADS) k_env_dist(const double* __restrict__ samples, long long ns, double3 o,
                                                           const Prim* __restrict__ prims, long long np,
+                                                          const float4* __restrict__ balls,
                                                           const float4* __restrict__ tiles,
                                                           const uint64_t* __restrict__ pkeys,
+                                                          const uint32_t* __restrict__ porder,
                                                           const uint64_t* __restrict__ skeys,
                                                           const uint32_t* __restrict__ sorder, float* __restrict__ dist,
                                                           int32_t* __restrict__ arg) {
-    __shared__ Prim tile[ENV_TILE];
-    __shared__ int skip;
-    __shared__ long long t0s;
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = q < ns;
-    const long long i = live ? (long long)sorder[q] : 0;
-    const float3 p = live ? make_float3((float)(samples[3 * i] - o.x), (float)(samples[3 * i + 1] - o.y),
-                                        (float)(samples[3 * i + 2] - o.z))
-                          : make_float3(0, 0, 0);
-    float best = INFINITY;
-    int bi = -1;
-    const long long ntile = (np + ENV_TILE - 1) / ENV_TILE;
-    if (threadIdx.x == 0) {   // first primitive whose code is >= the block's first sample's
-        const uint64_t key = skeys[(long long)blockIdx.x * blockDim.x];
-        long long lo = 0, hi = np;
-        while (lo < hi) {
-            const long long mid = (lo + hi) >> 1;
-            if (pkeys[mid] < key) lo = mid + 1;
-            else hi = mid;
+    const unsigned FULL = 0xffffffffu;
+    constexpr int NW = ENV_THREADS / 32;
+    __shared__ unsigned sbest[32];        // the samples' best distances so far (float_key)
+    __shared__ float fd[NW][32];          // the warps' results
+    __shared__ long long fr[NW][32];
+    __shared__ int fi[NW][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long q0 = 32ll * blockIdx.x;
+    const bool live = q0 + lane < ns;
+    const long long i = (long long)sorder[live ? q0 + lane : q0];
+    const float3 p = make_float3((float)(samples[3 * i] - o.x), (float)(samples[3 * i + 1] - o.y),
+                                 (float)(samples[3 * i + 2] - o.z));
+    if (warp == 0) sbest[lane] = float_key(INFINITY);
+    float lo[3] = {p.x, p.y, p.z}, hi[3] = {p.x, p.y, p.z};
+    for (int a = 0; a < 3; a++)
+        for (int off = 16; off; off >>= 1) {
+            lo[a] = fminf(lo[a], __shfl_xor_sync(FULL, lo[a], off));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(FULL, hi[a], off));
         }
-        t0s = lo < np ? lo / ENV_TILE : ntile - 1;
-    }
-    __syncthreads();
-    const long long t0 = t0s;
-    for (long long j = 0; j < 2 * ntile; j++) {
-        const long long t = (j & 1) ? t0 + (j + 1) / 2 : t0 - j / 2;   // t0, t0 + 1, t0 - 1, t0 + 2, ...
-        if (t < 0 || t >= ntile) continue;   // uniform over the block
-        // the block skips a tile whose bounding ball is farther from every
-        // live sample than that sample's best distance
-        const float4 tb = tiles[t];
-        const float dx = p.x - tb.x, dy = p.y - tb.y, dz = p.z - tb.z;
-        const bool need = live && (sqrtf(dx * dx + dy * dy + dz * dz) - tb.w < best);
-        if (threadIdx.x == 0) skip = 1;
-        __syncthreads();
-        if (need) skip = 0;
-        __syncthreads();
-        if (skip) continue;
-        const long long b = t * ENV_TILE;
-        const int m = (int)(np - b < ENV_TILE ? np - b : ENV_TILE);
-        for (int k = threadIdx.x; k < m; k += blockDim.x) tile[k] = prims[b + k];
-        __syncthreads();
-        if (need)
-            for (int k = 0; k < m; k++) {
-                const float d = prim_d(p, tile[k]);
-                if (d < best) {
-                    best = d;
-                    bi = (int)(b + k);
-                }
+    // margin of the ball tests, far above their FP32 rounding
+    float slack = 0.0f;
+    for (int a = 0; a < 3; a++) slack = fmaxf(slack, fmaxf(fabsf(lo[a]), fabsf(hi[a])));
+    slack *= 0x1p-18f;
+    // distance from the samples' box, or from this sample, to a ball, from below
+    auto gap = [&](float4 b) {
+        const float dx = fmaxf(fmaxf(lo[0] - b.x, b.x - hi[0]), 0.0f), dy = fmaxf(fmaxf(lo[1] - b.y, b.y - hi[1]), 0.0f),
+                    dz = fmaxf(fmaxf(lo[2] - b.z, b.z - hi[2]), 0.0f);
+        return sqrtf(dx * dx + dy * dy + dz * dz) * (1.0f - 0x1p-18f) - b.w - slack;
+    };
+    auto own_gap = [&](float4 b) {
+        const float dx = p.x - b.x, dy = p.y - b.y, dz = p.z - b.z;
+        return sqrtf(dx * dx + dy * dy + dz * dz) * (1.0f - 0x1p-18f) - b.w - slack;
+    };
+    const long long ntile64 = (np + ENV_TILE - 1) / ENV_TILE;
+    const long long l0 = warp_lower_bound(pkeys, np, skeys[q0 / ENV_BLOCK * ENV_BLOCK]);
+    const long long t0 = l0 < np ? l0 / ENV_TILE : ntile64 - 1;
+    float best = INFINITY;   // this warp's
+    long long brank = 0;
+    int bi = -1;
+    float bound = INFINITY, R = INFINITY;   // best of all the warps', and its largest over the samples
+    auto refresh = [&]() {
+        __syncwarp();
+        bound = key_float(*(volatile unsigned*)&sbest[lane]);
+        R = live ? bound : -INFINITY;
+        for (int off = 16; off; off >>= 1) R = fmaxf(R, __shfl_xor_sync(FULL, R, off));
+    };
+    auto tile = [&](long long t) {   // the 32 primitives of tile t
+        const long long k = 32 * t + lane;
+        unsigned open = __ballot_sync(FULL, k < np && !(gap(balls[k < np ? k : np - 1]) > R));
+        const long long t64 = t >> 1, j = t64 > t0 ? 2 * (t64 - t0) - 1 : 2 * (t0 - t64);
+        for (; open; open &= open - 1) {
+            const int b = __ffs(open) - 1;
+            if (!__any_sync(FULL, live && !(own_gap(balls[32 * t + b]) > fminf(bound, best)))) continue;
+            const float d = prim_d(p, prims[32 * t + b]);
+            const long long rank = j * ENV_TILE + 32 * (t & 1) + b;
+            if (live && (d < best || (d == best && rank < brank))) {
+                best = d;
+                bi = (int)(32 * t + b);
+                brank = rank;
             }
-        __syncthreads();
+        }
+        if (best < bound) atomicMin(&sbest[lane], float_key(best));
+        refresh();
+    };
+    const long long ntile = (np + 31) / 32, ngroup = (ntile + 31) / 32;
+    long long start = warp_lower_bound(pkeys, np, skeys[q0]) / 32;
+    if (start >= ntile) start = ntile - 1;
+    __syncthreads();   // sbest
+    // the tiles around the samples first, one per warp
+    const long long s0 = start - NW / 2 + warp;
+    if (s0 >= 0 && s0 < ntile) tile(s0);
+    __syncthreads();
+    refresh();
+    const long long g0 = start / 32;
+    for (long long jg = 0; jg < 2 * ngroup; jg++) {
+        const long long g = (jg & 1) ? g0 + (jg + 1) / 2 : g0 - jg / 2;
+        if (g < 0 || g >= ngroup) continue;
+        const long long t = 32 * g + lane;
+        const float gp = t < ntile ? gap(tiles[t]) : INFINITY;
+        // this warp's tiles of the group: every NW-th
+        for (unsigned open = __ballot_sync(FULL, t < ntile && !(gp > R) && (lane & (NW - 1)) == warp); open;
+             open &= open - 1) {
+            const int b = __ffs(open) - 1;
+            if (__shfl_sync(FULL, gp, b) > R) continue;   // R has fallen since
+            if (!__any_sync(FULL, live && !(own_gap(tiles[32 * g + b]) > fminf(bound, best)))) continue;
+            tile(32 * g + b);
+        }
     }
-    if (live) {
+    fd[warp][lane] = best;
+    fr[warp][lane] = brank;
+    fi[warp][lane] = bi;
+    __syncthreads();
+    if (warp == 0 && live) {
+        for (int w = 1; w < NW; w++)
+            if (fi[w][lane] >= 0 &&
+                (bi < 0 || fd[w][lane] < best || (fd[w][lane] == best && fr[w][lane] < brank))) {
+                best = fd[w][lane];
+                brank = fr[w][lane];
+                bi = fi[w][lane];
+            }
         dist[i] = best;
-        arg[i] = bi;
+        arg[i] = bi < 0 ? -1 : (int32_t)porder[bi];   // sorted position -> table row
     }
-}
-
-__global__ void k_env_unsort(int32_t* __restrict__ arg, long long n, const uint32_t* __restrict__ order) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && arg[i] >= 0) arg[i] = (int32_t)order[arg[i]];
 }
 
 }  // namespace
 
 size_t envelope_tmp_bytes(long long np, long long nsamp) {
     const size_t a = ((size_t)np * sizeof(Prim) + 255) & ~(size_t)255;
-    const size_t t = (((size_t)(np + ENV_TILE - 1) / ENV_TILE + 1) * sizeof(float4) + 255) & ~(size_t)255;
+    const size_t t = (((size_t)(np + 31) / 32 + 1) * sizeof(float4) + 255) & ~(size_t)255;
+    const size_t bl = ((size_t)np * sizeof(float4) + 255) & ~(size_t)255;
     const size_t k = ((size_t)(np + 1) * 8 + 255) & ~(size_t)255, v = ((size_t)(np + 1) * 4 + 255) & ~(size_t)255;
     const size_t ks = ((size_t)(nsamp + 1) * 8 + 255) & ~(size_t)255, vs = ((size_t)(nsamp + 1) * 4 + 255) & ~(size_t)255;
-    return 2 * a + t + 2 * k + 2 * v + 2 * ks + 2 * vs + radix_tmp_bytes(np > nsamp ? np : nsamp);
+    return 2 * a + t + bl + 2 * k + 2 * v + 2 * ks + 2 * vs + radix_tmp_bytes(np > nsamp ? np : nsamp);
 }
 
 // Primitive table sorted by the Morton code of the primitive's mean centre,
@@ -327,7 +410,8 @@ void launch_envelope(const int32_t* k1, long long n1, const int32_t* k2, long lo
     const long long np = n1 + n2 + n3;
     if (np <= 0 || nsamp <= 0) return;
     const size_t a = ((size_t)np * sizeof(Prim) + 255) & ~(size_t)255;
-    const size_t t = (((size_t)(np + ENV_TILE - 1) / ENV_TILE + 1) * sizeof(float4) + 255) & ~(size_t)255;
+    const size_t t = (((size_t)(np + 31) / 32 + 1) * sizeof(float4) + 255) & ~(size_t)255;
+    const size_t bl = ((size_t)np * sizeof(float4) + 255) & ~(size_t)255;
     const size_t k = ((size_t)(np + 1) * 8 + 255) & ~(size_t)255, v = ((size_t)(np + 1) * 4 + 255) & ~(size_t)255;
     char* p = (char*)tmp;
     Prim* raw = (Prim*)p;
@@ -336,6 +420,8 @@ void launch_envelope(const int32_t* k1, long long n1, const int32_t* k2, long lo
     p += a;
     float4* tiles = (float4*)p;
     p += t;
+    float4* balls = (float4*)p;
+    p += bl;
     uint64_t* m0 = (uint64_t*)p;
     p += k;
     uint64_t* m1 = (uint64_t*)p;
@@ -360,17 +446,12 @@ void launch_envelope(const int32_t* k1, long long n1, const int32_t* k2, long lo
                                                make_int3(g0, g0, g0), 1);
     note_launch();
     radix_sort_pairs(m0, i0, m1, i1, np, 63, p, d_err, s);
-    k_env_gather<<<nblk(np, 256), 256, 0, s>>>(raw, i1, np, sorted);
-    note_launch();
-    const long long ntile = (np + ENV_TILE - 1) / ENV_TILE;
-    k_env_tiles<<<(unsigned)ntile, 128, 0, s>>>(sorted, np, tiles);
+    k_env_gather<<<nblk(np, 256), 256, 0, s>>>(raw, i1, np, sorted, balls, tiles);
     note_launch();
     k_env_sample_keys<<<nblk(nsamp, 256), 256, 0, s>>>(samples, nsamp, 1.0 / unit, make_int3(g0, g0, g0), 1, sk0, so0);
     note_launch();
     radix_sort_pairs(sk0, so0, sk1, so1, nsamp, 63, p, d_err, s);
-    k_env_dist<<<nblk(nsamp, ENV_THREADS), ENV_THREADS, 0, s>>>(samples, nsamp, o, sorted, np, tiles, m1, sk1, so1, dist,
-                                                                  prim_id);
-    note_launch();
-    k_env_unsort<<<nblk(nsamp, 256), 256, 0, s>>>(prim_id, nsamp, i1);   // sorted positions -> table rows
+    k_env_dist<<<nblk(nsamp, 32), ENV_THREADS, 0, s>>>(samples, nsamp, o, sorted, np, balls, tiles, m1, i1,
+                                                                sk1, so1, dist, prim_id);
     note_launch();
 }
