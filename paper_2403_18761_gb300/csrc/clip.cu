@@ -195,86 +195,122 @@ __device__ __forceinline__ Real dot_bound(int m, const Real C[4]) {
 }
 
 // ------------------------------------------------------------- slow paths
+// What a slow predicate needs to compute its exact rows again: a few pointers
+// and indices, so that a call keeps few of the clip kernel's registers alive.
 struct Slow {
-    const int32_t* Ci;
+    const int32_t *X0, *tet, *Ci, *cand;   // grid vertices, the tet's vertex ids, sphere centres, the tet's candidates
     const long long* W;
-    DevState* st;
+    int i;   // the piece's sphere
 };
 
-struct Row4 {
-    long long v[4];
-};
+__device__ __forceinline__ void slow_row(const Slow& S, int slot, long long F[4]) {
+    const int j = S.cand[slot];
+    const int3 ci = ld_int3(S.Ci, S.i), cj = ld_int3(S.Ci, j);
+    const long long wi = S.W[S.i], wj = S.W[j];
+    for (int k = 0; k < 4; k++) {
+        const int3 x = ld_int3(S.X0, S.tet[k]);
+        F[k] = pd_exact(x, ci, wi) - pd_exact(x, cj, wj);
+    }
+}
 
 // Exact-or-FP64 sign of (F_u . C) * sign(sum C) for the vertex on planes
-// (a,b,c); has_u == false asks for sign(sum C) alone.  Returns 0 only when
-// the exact value is zero (degenerate input).  Arguments are passed by value
-// so that the caller's lane state stays in registers.
-__device__ __noinline__ int slow_sign_impl(Lane L, Slow S, int a, int b, int c, Row4 U, bool has_u, bool try_fp64,
-                                           unsigned* cnt) {
-    const long long* Fu = has_u ? U.v : nullptr;
-    unsigned& n64 = cnt[0];
-    unsigned& nex = cnt[1];
+// (a,b,c), u the candidate slot of the plane; u < 0 asks for sign(sum C)
+// alone.  Returns 0 only when the exact value is zero (degenerate input), in
+// bits 0..1 as sign + 1; bit 2 is set when FP64 decided.
+__device__ __noinline__ unsigned slow_sign_impl(Slow S, int a, int b, int c, int u, bool try_fp64) {
     int fc[4], bis[3];
     int m = split_planes(a, b, c, fc, bis);
-    long long R[3][4];
-    for (int k = 0; k < m; k++) row_i64(L, S.Ci, S.W, bis[k] - 4, R[k]);
+    long long R[3][4], Fu[4] = {0, 0, 0, 0};
+    for (int k = 0; k < m; k++) slow_row(S, bis[k] - 4, R[k]);
+    if (u >= 0) slow_row(S, u, Fu);
     if (try_fp64) {
         double Rd[3][4], Cd[4], Fd[4];
         for (int k = 0; k < m; k++) scale_row<double>(R[k], Rd[k]);
         cof_real<double>(m, Rd, fc, Cd);
-        const double u = 0x1p-53, em = cof_err<double>(m);
+        const double ur = 0x1p-53, em = cof_err<double>(m);
         double sum = Cd[0] + Cd[1] + Cd[2] + Cd[3];
         double sa = fabs(Cd[0]) + fabs(Cd[1]) + fabs(Cd[2]) + fabs(Cd[3]);
-        double bs = ((m + 1) * em + 4 * u * sa) * (1 + 8 * u);
+        double bs = ((m + 1) * em + 4 * ur * sa) * (1 + 8 * ur);
         if (fabs(sum) > bs) {
             int ss = sum > 0 ? 1 : -1;
-            if (!Fu) {
-                n64++;
-                return ss;
-            }
+            if (u < 0) return (unsigned)(ss + 1) | 4u;
             scale_row<double>(Fu, Fd);
             double v = fma(Fd[0], Cd[0], fma(Fd[1], Cd[1], fma(Fd[2], Cd[2], Fd[3] * Cd[3])));
-            if (fabs(v) > dot_bound<double>(m, Cd)) {
-                n64++;
-                return (v > 0 ? 1 : -1) * ss;
-            }
+            if (fabs(v) > dot_bound<double>(m, Cd)) return (unsigned)((v > 0 ? 1 : -1) * ss + 1) | 4u;
         }
     }
-    nex++;
     I256 C[4];
     exact_cofactors(m, R, fc, C);
     I256 sum = C[0];
     for (int k = 1; k <= m; k++) sum = i256_add(sum, C[k]);
     int ss = i256_sign(sum);
-    if (!Fu || ss == 0) return ss;
+    if (u < 0 || ss == 0) return (unsigned)(ss + 1);
     I256 v = i256_mul_i64(C[0], Fu[fc[0]]);
     for (int k = 1; k <= m; k++) v = i256_add(v, i256_mul_i64(C[k], Fu[fc[k]]));
-    return i256_sign(v) * ss;
+    return (unsigned)(i256_sign(v) * ss + 1);
 }
 
-__device__ __forceinline__ int slow_sign(const Lane& L, const Slow& S, int a, int b, int c, const long long* Fu,
-                                         bool try_fp64, unsigned& n64, unsigned& nex) {
-    Row4 U;
-    if (Fu)
-        for (int k = 0; k < 4; k++) U.v[k] = Fu[k];
-    else
-        for (int k = 0; k < 4; k++) U.v[k] = 0;
-    unsigned cnt[2] = {0, 0};
-    const int r = slow_sign_impl(L, S, a, b, c, U, Fu != nullptr, try_fp64, cnt);
-    n64 += cnt[0];
-    nex += cnt[1];
-    return r;
+__device__ __forceinline__ int slow_sign(const Slow& S, int a, int b, int c, int u, bool try_fp64, unsigned& n64,
+                                         unsigned& nex) {
+    const unsigned r = slow_sign_impl(S, a, b, c, u, try_fp64);
+    if (r & 4u) n64++;
+    else nex++;
+    return (int)(r & 3u) - 1;
 }
 
 // ------------------------------------------------------------ smem access
-// Per warp: [VMAX][VW][32] slot words followed by [VMAX][32] scratch words.
+// Per warp: [VMAX][VW][32] slot words, then per lane in 16-byte words the
+// scaled rows of the planes met so far ([NC] x 4 Reals) and the tet's corners
+// (3 x int4), then [SCR][32] scratch words (the boundary of a removed region: at most one new vertex per face of
+// the piece).  A vertex on two or three radical planes needs the rows of
+// planes clipped earlier; computing them again (five loads and four exact
+// power distances each) cost more than the polytope surgery, and the kernels
+// are bound by issue and latency at 8 to 13 active lanes a warp.
 template <typename Real, int VMAX>
 struct Store {
     uint32_t* base;
     int lane;
     static constexpr int VW = PrecTraits<Real>::VW;
+    static constexpr int NC = (VMAX - 2) / 2;    // candidates of a tet
+    static constexpr int SCR = NC + 3;           // faces of a piece
+    // FP64 rows take 32 bytes: for the bins of many candidates they would cost
+    // a quarter of the resident warps, more than computing a row again does
+    // (the 60k-tet blob in FP64: clip kernels 1.02 ms without any rows kept,
+    // 1.15 ms with all, see launch_clip)
+    static constexpr bool ROWS = sizeof(Real) == 4 || VMAX < 18;
+    static constexpr int RW = ROWS ? 4 * sizeof(Real) / 4 : 0;   // words of a row
+    static constexpr int WORDS = VMAX * VW + NC * RW + 12 + SCR;   // per lane
+    __device__ __forceinline__ void put_row(int s, const Real R[4]) const {
+        if constexpr (sizeof(Real) == 4) {
+            reinterpret_cast<float4*>(base + VMAX * VW * 32)[s * 32 + lane] = make_float4(R[0], R[1], R[2], R[3]);
+        } else {
+            double2* q = reinterpret_cast<double2*>(base + VMAX * VW * 32) + 64 * s + lane;
+            q[0] = make_double2(R[0], R[1]);
+            q[32] = make_double2(R[2], R[3]);
+        }
+    }
+    __device__ __forceinline__ void get_row(int s, Real R[4]) const {
+        if constexpr (sizeof(Real) == 4) {
+            const float4 v = reinterpret_cast<const float4*>(base + VMAX * VW * 32)[s * 32 + lane];
+            R[0] = v.x;
+            R[1] = v.y;
+            R[2] = v.z;
+            R[3] = v.w;
+        } else {
+            const double2* q = reinterpret_cast<const double2*>(base + VMAX * VW * 32) + 64 * s + lane;
+            const double2 u = q[0], v = q[32];
+            R[0] = u.x;
+            R[1] = u.y;
+            R[2] = v.x;
+            R[3] = v.y;
+        }
+    }
+    // coordinate `axis` of the four corners
+    __device__ __forceinline__ int4& corners(int axis) const {
+        return reinterpret_cast<int4*>(base + (VMAX * VW + NC * RW) * 32)[32 * axis + lane];
+    }
     __device__ __forceinline__ uint32_t& w(int v, int k) const { return base[(v * VW + k) * 32 + lane]; }
-    __device__ __forceinline__ uint32_t& scratch(int j) const { return base[(VMAX * VW + j) * 32 + lane]; }
+    __device__ __forceinline__ uint32_t& scratch(int j) const { return base[(VMAX * VW + NC * RW + 12 + j) * 32 + lane]; }
     __device__ __forceinline__ uint32_t trip(int v) const { return w(v, 0); }
     __device__ __forceinline__ void set_trip(int v, uint32_t t) const { w(v, 0) = t; }
     __device__ __forceinline__ uint32_t nb(int v) const { return w(v, 1); }
@@ -331,18 +367,41 @@ __device__ __forceinline__ double tet_volume6(const int3* X) {
 
 // Warp-wide exclusive scan of a per-lane count + one atomic reservation.
 __device__ __forceinline__ long long warp_reserve(unsigned cnt, unsigned long long* counter) {
-    int lane = threadIdx.x & 31;
-    unsigned inc = cnt;
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(0xffffffffu, cnt != 0);   // counts of 0 or 1
+    unsigned long long base = 0;
+    if (lane == 0 && m) base = atomicAdd(counter, (unsigned long long)__popc(m));
+    return (long long)__shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+}
+
+// Exclusive offsets of three per-thread counts (each below 2^11 per thread,
+// 2^18 per block) in three counters: one scan of the packed counts and one
+// atomic per counter and block.  All threads of the block call it.
+__device__ __forceinline__ void block_reserve3(unsigned n0, unsigned n1, unsigned n2, unsigned long long* counters,
+                                               long long* out) {
+    __shared__ unsigned long long wsum[4], base[3];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned long long v = (unsigned long long)n0 | ((unsigned long long)n1 << 21) | ((unsigned long long)n2 << 42);
+    unsigned long long inc = v;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        unsigned o = __shfl_up_sync(0xffffffffu, inc, off);
+        const unsigned long long o = __shfl_up_sync(0xffffffffu, inc, off);
         if (lane >= off) inc += o;
     }
-    unsigned total = __shfl_sync(0xffffffffu, inc, 31);
-    unsigned long long base = 0;
-    if (lane == 31 && total) base = atomicAdd(counter, (unsigned long long)total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    return (long long)base + (inc - cnt);
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    unsigned long long pre = 0, tot = 0;
+    for (int k = 0; k < nw; k++) {
+        if (k < w) pre += wsum[k];
+        tot += wsum[k];
+    }
+    if (threadIdx.x < 3) {
+        const unsigned long long mine = (tot >> (21 * threadIdx.x)) & 0x1fffffull;
+        base[threadIdx.x] = mine ? atomicAdd(&counters[threadIdx.x], mine) : 0;
+    }
+    __syncthreads();
+    pre += inc - v;
+    for (int k = 0; k < 3; k++) out[k] = (long long)(base[k] + ((pre >> (21 * k)) & 0x1fffffull));
 }
 
 __device__ __forceinline__ bool bit(unsigned long long m0, unsigned long long m1, int v) {
@@ -353,8 +412,8 @@ __device__ __forceinline__ bool bit(unsigned long long m0, unsigned long long m1
 // V - E + F - 1 with carrier weights and its links through tet faces, one RPF
 // record per radical face of a sphere j > i (polygon V - E + 1), one RPE
 // record per edge on two radical planes of spheres > i, one RPV record per
-// vertex on three.  All lanes call it (warp-wide reservations); inactive
-// lanes emit nothing.
+// vertex on three.  All threads of the block call it (block-wide reservations);
+// inactive ones emit nothing.
 template <int VMAX, typename S>
 __device__ __forceinline__ void emit_records(const ClipArgs& A, const Lane& L, const S& V, int nslot, long long p,
                                              bool active) {
@@ -377,9 +436,9 @@ __device__ __forceinline__ void emit_records(const ClipArgs& A, const Lane& L, c
         for (int pl = 4; pl < 4 + L.n; pl++)
             if (((fmask >> pl) & 1) && L.cand[pl - 4] > L.i) nF++;
     }
-    const long long fb = warp_reserve(nF, &A.rcount[0]);
-    const long long eb = warp_reserve(nE, &A.rcount[1]);
-    const long long vb = warp_reserve(nV, &A.rcount[2]);
+    long long at[3];
+    block_reserve3(nF, nE, nV, A.rcount, at);
+    const long long fb = at[0], eb = at[1], vb = at[2];
     if (!active) return;
     A.f_off[p] = (int32_t)fb;
     A.f_cnt[p] = (uint8_t)nF;
@@ -492,32 +551,70 @@ __device__ __forceinline__ void emit_records(const ClipArgs& A, const Lane& L, c
     }
 }
 
+// A piece that is the whole tet: V - E + F - 1 from the ownership bits, links
+// on every shared face, volume and moment in closed form.
+__device__ __forceinline__ void whole_one(const ClipArgs& A, long long p) {
+    const long long t = A.pair_tet[p];
+    const uint32_t own = A.own[t];
+    int3 X[4];
+    for (int k = 0; k < 4; k++) X[k] = ld_int3(A.Xi, A.tets[4 * t + k]);
+    const int32_t* adj = A.adj + 4 * t;
+    unsigned lk = 0xf0u;   // the whole tet has a face on each tet face
+    for (int f = 0; f < 4; f++)
+        if (adj[f] >= 0) lk |= 1u << f;
+    A.pflag[p] = 1;
+    A.c_val[p] = __popc(own & 0xfu) - __popc(own & 0x3f0u) + __popc(own & 0x3c00u) - 1;
+    A.c_link[p] = (uint8_t)lk;
+    A.f_off[p] = 0;
+    A.f_cnt[p] = 0;
+    A.e_off[p] = 0;
+    A.e_cnt[p] = 0;
+    const double vt = tet_volume6(X) / 6.0;
+    const double u3 = A.unit * A.unit * A.unit;
+    A.p_vol[p] = vt * u3;
+    A.p_mom[3 * p + 0] = vt * 0.25 * ((double)X[0].x + X[1].x + X[2].x + X[3].x) * u3 * A.unit;
+    A.p_mom[3 * p + 1] = vt * 0.25 * ((double)X[0].y + X[1].y + X[2].y + X[3].y) * u3 * A.unit;
+    A.p_mom[3 * p + 2] = vt * 0.25 * ((double)X[0].z + X[1].z + X[2].z + X[3].z) * u3 * A.unit;
+}
+
 // ----------------------------------------------------------- clip kernel
-template <typename Real, int VMAX>
-__device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __restrict__ pairs, long long q, bool active,
-                                         const Store<Real, VMAX>& V) {
-    Lane L;
-    long long p = 0;
+// One pair per lane.  With SLOW every predicate that the first stage does not
+// certify goes on to the slower stages; without it such a pair is given up
+// and the lane returns true: the call to the slow stages in the middle of the
+// loop cost the common path a fifth of its resident warps in registers.
+template <typename Real, int VMAX, bool SLOW>
+__device__ __forceinline__ bool clip_one(const ClipArgs& A, const int32_t* __restrict__ pairs, long long q, bool active,
+                                         const Store<Real, VMAX>& V, unsigned* counts) {
+    int p = 0, si = 0, nc = 0;
     int nslot = 0, nlive = 0;
-    bool alive = active, whole = true, degenerate = false;
+    bool alive = active, whole = true, degenerate = false, retry = false;
     unsigned nfast = 0, n64 = 0, nex = 0;
     unsigned nvp = 0;   // constructed vertices with m = 1, 2, 3 radical planes, 10 bits each
-    const Slow S{A.Ci, A.W, A.st};
+    Slow S{A.Xi, nullptr, A.Ci, nullptr, A.W, 0};
+    // the row of sphere s at corner X: pd(X, i) - pd(X, s) = 2 (c_s - c_i).X + K_i - K_s
+    // with K = |c|^2 - w, all exact in 64 bits
+    int3 ci = make_int3(0, 0, 0);
+    long long Ki = 0;
+    auto power0 = [](int3 c, long long w) {
+        return (long long)c.x * c.x + (long long)c.y * c.y + (long long)c.z * c.z - w;
+    };
+    const uint8_t* ord = nullptr;
     if (active) {
         p = pairs[q];
-        L.t = A.pair_tet[p];
-        L.si = (int)(p - A.pair_off[L.t]);
-        L.n = A.cand_cnt[L.t];
-        L.cand = A.cand + L.t * RPD_MAXC;
-        L.i = L.cand[L.si];
-        L.own = A.own[L.t];
-        const int3 ci = ld_int3(A.Ci, L.i);
-        const long long wi = A.W[L.i];
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            L.X[k] = ld_int3(A.Xi, A.tets[4 * L.t + k]);
-            L.di[k] = pd_exact(L.X[k], ci, wi);
-        }
+        const int t = A.pair_tet[p];
+        si = (int)(p - A.pair_off[t]);
+        nc = A.cand_cnt[t];
+        S.tet = A.tets + 4ll * t;
+        S.cand = A.cand + (long long)t * RPD_MAXC;
+        S.i = S.cand[si];
+        ord = A.cand_ord + (long long)t * RPD_MAXC;
+        ci = ld_int3(A.Ci, S.i);
+        Ki = power0(ci, A.W[S.i]);
+        const int4 v = *reinterpret_cast<const int4*>(S.tet);
+        const int3 x0 = ld_int3(A.Xi, v.x), x1 = ld_int3(A.Xi, v.y), x2 = ld_int3(A.Xi, v.z), x3 = ld_int3(A.Xi, v.w);
+        V.corners(0) = make_int4(x0.x, x1.x, x2.x, x3.x);
+        V.corners(1) = make_int4(x0.y, x1.y, x2.y, x3.y);
+        V.corners(2) = make_int4(x0.z, x1.z, x2.z, x3.z);
         // the tet: corner a lies on the three faces != a; neighbours across
         // the dual edges trip[0]->trip[1], trip[1]->trip[2], trip[2]->trip[0]
         V.set_trip(0, pack3(1, 2, 3));
@@ -531,12 +628,35 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
         nslot = nlive = 4;
     }
     // ---------------------------------------------------------- clipping
-    const uint8_t* ord = active ? A.cand_ord + L.t * RPD_MAXC : nullptr;
-    for (int k = 0; alive && k < L.n; k++) {
-        const int s = ord[k];
-        if (s == L.si) continue;
+    // the next plane's sphere is loaded while the current one is clipped
+    int s_next = 0;
+    int3 c_next = make_int3(0, 0, 0);
+    long long w_next = 0;
+    auto fetch = [&](int k) {
+        s_next = ord[k];
+        const int j = S.cand[s_next];
+        c_next = ld_int3(A.Ci, j);
+        w_next = A.W[j];
+    };
+    auto exact_row = [&](int3 c, long long w, long long F[4]) {
+        const int gx = 2 * (c.x - ci.x), gy = 2 * (c.y - ci.y), gz = 2 * (c.z - ci.z);
+        const long long K = Ki - power0(c, w);
+        const int4 X = V.corners(0), Y = V.corners(1), Z = V.corners(2);
+        F[0] = K + (long long)gx * X.x + (long long)gy * Y.x + (long long)gz * Z.x;
+        F[1] = K + (long long)gx * X.y + (long long)gy * Y.y + (long long)gz * Z.y;
+        F[2] = K + (long long)gx * X.z + (long long)gy * Y.z + (long long)gz * Z.z;
+        F[3] = K + (long long)gx * X.w + (long long)gy * Y.w + (long long)gz * Z.w;
+    };
+    if (alive) fetch(0);
+#pragma unroll 1
+    for (int k = 0; alive && k < nc; k++) {
+        const int s = s_next;
+        const int3 cs = c_next;
+        const long long ws = w_next;
+        if (k + 1 < nc) fetch(k + 1);
+        if (s == si) continue;
         long long F[4];
-        row_i64(L, A.Ci, A.W, s, F);
+        exact_row(cs, ws, F);
         if (F[0] < 0 && F[1] < 0 && F[2] < 0 && F[3] < 0) continue;   // plane misses the tet
         if (F[0] > 0 && F[1] > 0 && F[2] > 0 && F[3] > 0) {            // tet inside cell s
             alive = false;
@@ -544,17 +664,22 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
         }
         Real Fr[4];
         scale_row<Real>(F, Fr);
+        if constexpr (V.ROWS) V.put_row(s, Fr);
         const int l = 4 + s;
+        // signs of the plane at the tet's corners, exact (sign + 1, two bits each)
+        unsigned corner_sign = 0;
+#pragma unroll
+        for (int z = 0; z < 4; z++) corner_sign |= (F[z] > 0 ? 2u : (F[z] < 0 ? 0u : 1u)) << (2 * z);
         unsigned long long out0 = 0, out1 = 0;
         int nout = 0;
+#pragma unroll 1
         for (int v = 0; v < nslot; v++) {
             const uint32_t tw = V.trip(v);
             if (is_dead(tw)) continue;
             const int a = tb(tw, 0), b = tb(tw, 1), c = tb(tw, 2);
             int sg;
             if (a < 4 && b < 4 && c < 4) {
-                const long long fv = get4(F, 6 - a - b - c);
-                sg = (fv > 0) - (fv < 0);
+                sg = (int)((corner_sign >> (2 * (6 - a - b - c))) & 3u) - 1;
             } else {
                 Real C0, C1, C2, C3, B;
                 V.get_real(v, 0, C0);
@@ -563,11 +688,14 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
                 V.get_real(v, 3, C3);
                 V.get_real(v, 4, B);
                 const Real val = fma(Fr[0], C0, fma(Fr[1], C1, fma(Fr[2], C2, Fr[3] * C3)));
-                if (fabs(val) > B && !A.force_slow) {
+                if (fabs(val) > B && !(SLOW && A.force_slow)) {
                     sg = val > 0 ? 1 : -1;
                     nfast++;
+                } else if constexpr (!SLOW) {
+                    retry = true;
+                    break;
                 } else {
-                    sg = slow_sign(L, S, a, b, c, F, sizeof(Real) == 4 && A.force_slow < 2, n64, nex);
+                    sg = slow_sign(S, a, b, c, s, sizeof(Real) == 4 && A.force_slow < 2, n64, nex);
                 }
             }
             if (sg == 0) {
@@ -580,7 +708,7 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
                 nout++;
             }
         }
-        if (degenerate) {
+        if (degenerate || retry) {
             alive = false;
             break;
         }
@@ -593,6 +721,7 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
         // boundary of the removed region: dual edges x->y of removed vertices
         // whose neighbour w is kept; one new vertex (x, y, l) each
         int nbd = 0;
+#pragma unroll 1
         for (int r = 0; r < nslot; r++) {
             if (!bit(out0, out1, r)) continue;
             const uint32_t tw = V.trip(r), nw = V.nb(r);
@@ -600,21 +729,22 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
             for (int e = 0; e < 3; e++) {
                 const int w = tb(nw, e);
                 if (bit(out0, out1, w)) continue;
-                if (nbd == VMAX) {
-                    nbd = VMAX + 1;
+                if (nbd == V.SCR) {
+                    nbd = V.SCR + 1;
                     break;
                 }
                 V.scratch(nbd++) = (uint32_t)tb(tw, e) | ((uint32_t)tb(tw, (e + 1) % 3) << 8) | ((uint32_t)w << 16);
             }
             V.set_trip(r, DEAD);
         }
-        if (nbd > VMAX) {
+        if (nbd > V.SCR) {
             dev_fail(A.st, RPD_E_OVERFLOW, CNT_CAPACITY);
             alive = false;
             break;
         }
         // slots: free slots first, then append
         int cur = 0;
+#pragma unroll 1
         for (int j = 0; j < nbd; j++) {
             while (cur < nslot && !is_dead(V.trip(cur))) cur++;
             int h;
@@ -633,10 +763,12 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
             V.set_trip(h, DEAD | 0x00ffffffu);   // reserved (still free for the scan below)
         }
         if (!alive) break;
+#pragma unroll 1
         for (int j = 0; j < nbd; j++) {
             const uint32_t e = V.scratch(j);
             const int x = e & 0xff, y = (e >> 8) & 0xff, w = (e >> 16) & 0xff, h = e >> 24;
             int n1 = -1, n2 = -1;
+#pragma unroll 1
             for (int j2 = 0; j2 < nbd; j2++) {
                 const uint32_t e2 = V.scratch(j2);
                 if ((int)(e2 & 0xff) == y) n1 = e2 >> 24;          // next: starts at y
@@ -665,12 +797,15 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
 #pragma unroll
             for (int z = 0; z < 3; z++) {
                 if (z >= m) break;
-                if (bis[z] == l) {
+                if constexpr (V.ROWS) {
+                    V.get_row(bis[z] - 4, R[z]);
+                } else if (bis[z] == l) {
 #pragma unroll
                     for (int c = 0; c < 4; c++) R[z][c] = Fr[c];
                 } else {
+                    const int j2 = S.cand[bis[z] - 4];
                     long long Fk[4];
-                    row_i64(L, A.Ci, A.W, bis[z] - 4, Fk);
+                    exact_row(ld_int3(A.Ci, j2), A.W[j2], Fk);
                     scale_row<Real>(Fk, R[z]);
                 }
             }
@@ -681,11 +816,15 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
             const Real sa = fabs(C[0]) + fabs(C[1]) + fabs(C[2]) + fabs(C[3]);
             const Real bs = ((Real)(m + 1) * cof_err<Real>(m) + 4 * u * sa) * (1 + 8 * u);
             int ss;
-            if (fabs(sum) > bs && !A.force_slow) {
+            if (fabs(sum) > bs && !(SLOW && A.force_slow)) {
                 ss = sum > 0 ? 1 : -1;
                 nfast++;
+            } else if constexpr (!SLOW) {
+                retry = true;
+                alive = false;
+                break;
             } else {
-                ss = slow_sign(L, S, x, y, l, nullptr, sizeof(Real) == 4 && A.force_slow < 2, n64, nex);
+                ss = slow_sign(S, x, y, l, -1, sizeof(Real) == 4 && A.force_slow < 2, n64, nex);
             }
             if (ss == 0) {
                 degenerate = true;
@@ -703,14 +842,15 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
         if (!alive) break;
         nlive += nbd - nout;
     }
-    if (degenerate) dev_fail(A.st, RPD_E_DEGENERATE, CNT_DEGENERATE);
+    if (degenerate && !retry) dev_fail(A.st, RPD_E_DEGENERATE, CNT_DEGENERATE);
     if (active && nlive < 4) alive = false;
-    dev_count(A.st, CNT_PRED_FAST, nfast);
-    dev_count(A.st, CNT_PRED_FP64, n64);
-    dev_count(A.st, CNT_PRED_EXACT, nex);
-    dev_count(A.st, CNT_NEWVERT1, nvp & 1023u);
-    dev_count(A.st, CNT_NEWVERT2, (nvp >> 10) & 1023u);
-    dev_count(A.st, CNT_NEWVERT3, nvp >> 20);
+    if (retry) nfast = nvp = 0;   // the second pass counts this pair
+    const unsigned tally[6] = {nfast, n64, nex, nvp & 1023u, (nvp >> 10) & 1023u, nvp >> 20};
+#pragma unroll
+    for (int z = 0; z < 6; z++) {
+        const unsigned tot = __reduce_add_sync(0xffffffffu, tally[z]);
+        if ((threadIdx.x & 31) == 0 && tot) atomicAdd(&counts[z], tot);
+    }
 
     // ------------------------- whole pieces here; cut pieces to the queue
     // (their fractional Euler records are emitted by k_records, their volume
@@ -725,7 +865,7 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
             A.qtrip[(2LL * v + 1) * A.qcap + qb] = V.nb(v);
         }
     }
-    if (!active) return;
+    if (!active || retry) return retry;
     A.pflag[p] = alive ? 1 : 0;
     if (!alive) {
         A.c_val[p] = 0;
@@ -733,45 +873,50 @@ __device__ __forceinline__ void clip_one(const ClipArgs& A, const int32_t* __res
         A.f_off[p] = A.e_off[p] = 0;
         A.f_cnt[p] = A.e_cnt[p] = 0;
         A.p_vol[p] = 0.0;
-        A.p_mom[3 * p] = A.p_mom[3 * p + 1] = A.p_mom[3 * p + 2] = 0.0;
-        return;
+        A.p_mom[3ll * p] = A.p_mom[3ll * p + 1] = A.p_mom[3ll * p + 2] = 0.0;
+        return false;
     }
-    if (!whole) return;
-    {   // the whole tet: V - E + F - 1 from the ownership bits, links on every shared face
-        const int32_t* adj = A.adj + 4 * L.t;
-        unsigned lk = 0xf0u;   // the whole tet has a face on each tet face
-        for (int f = 0; f < 4; f++)
-            if (adj[f] >= 0) lk |= 1u << f;
-        A.c_val[p] = __popc(L.own & 0xfu) - __popc(L.own & 0x3f0u) + __popc(L.own & 0x3c00u) - 1;
-        A.c_link[p] = (uint8_t)lk;
-        A.f_off[p] = A.e_off[p] = 0;
-        A.f_cnt[p] = A.e_cnt[p] = 0;
-    }
-    // whole tets: volume and moment in closed form; cut pieces were queued
-    if (whole) {
-        const double vt = tet_volume6(L.X) / 6.0;
-        const double u3 = A.unit * A.unit * A.unit;
-        A.p_vol[p] = vt * u3;
-        A.p_mom[3 * p + 0] = vt * 0.25 * ((double)L.X[0].x + L.X[1].x + L.X[2].x + L.X[3].x) * u3 * A.unit;
-        A.p_mom[3 * p + 1] = vt * 0.25 * ((double)L.X[0].y + L.X[1].y + L.X[2].y + L.X[3].y) * u3 * A.unit;
-        A.p_mom[3 * p + 2] = vt * 0.25 * ((double)L.X[0].z + L.X[1].z + L.X[2].z + L.X[3].z) * u3 * A.unit;
-    }
+    if (!whole) return false;
+    whole_one(A, p);
+    return false;
 }
 
+// The pairs a warp gave up, through the slow stages (all lanes call it).
 template <typename Real, int VMAX>
-__global__ void __launch_bounds__(128) k_clip(ClipArgs A, const int32_t* __restrict__ pairs,
-                                              const int32_t* __restrict__ d_n) {
-    extern __shared__ uint32_t smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Store<Real, VMAX> V{smem + (size_t)warp * VMAX * (PrecTraits<Real>::VW + 1) * 32, lane};
+__device__ __noinline__ void clip_again(const ClipArgs& A, const int32_t* __restrict__ pairs, long long q, bool active,
+                                        uint32_t* base, unsigned* counts) {
+    const Store<Real, VMAX> V{base, (int)(threadIdx.x & 31)};
+    clip_one<Real, VMAX, true>(A, pairs, q, active, V, counts);
+}
+
+// `per` pairs per warp (32, or fewer where the bin has too few to fill the
+// SMs, see pairs_per_warp).  The block's counters go to the device status
+// with one atomic each: one per warp and counter, all on one cache line, kept
+// that line busy for a good part of the kernel.
+template <typename Real, int VMAX>
+__global__ void __launch_bounds__(sizeof(Real) == 4 ? 128 : 32, sizeof(Real) == 4 ? 4 : 1) k_clip(ClipArgs A, const int32_t* __restrict__ pairs,
+                                              const int32_t* __restrict__ d_n, int per) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ unsigned counts[6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const Store<Real, VMAX> V{smem + (size_t)warp * Store<Real, VMAX>::WORDS * 32, lane};
+    if (threadIdx.x < 6) counts[threadIdx.x] = 0;
+    __syncthreads();
     const long long n = *d_n;
     // grid-stride over pairs; q0 is warp-uniform so warp collectives stay converged
-    for (long long q0 = (long long)blockIdx.x * blockDim.x + warp * 32; q0 < n;
-         q0 += (long long)gridDim.x * blockDim.x) {
+    for (long long q0 = ((long long)blockIdx.x * nwarps + warp) * per; q0 < n;
+         q0 += (long long)gridDim.x * nwarps * per) {
         const long long q = q0 + lane;
-        clip_one<Real, VMAX>(A, pairs, q, q < n, V);
+        bool again = lane < per && q < n;
+        if (!A.force_slow) again = clip_one<Real, VMAX, false>(A, pairs, q, again, V, counts);
+        __syncwarp();
+        if (__any_sync(0xffffffffu, again)) clip_again<Real, VMAX>(A, pairs, q, again, V.base, counts);
         __syncwarp();
     }
+    __syncthreads();
+    constexpr int to[6] = {CNT_PRED_FAST, CNT_PRED_FP64, CNT_PRED_EXACT, CNT_NEWVERT1, CNT_NEWVERT2, CNT_NEWVERT3};
+    if (threadIdx.x < 6 && counts[threadIdx.x])
+        atomicAdd(&A.st->cnt[to[threadIdx.x]], (unsigned long long)counts[threadIdx.x]);
 }
 
 // ------------------------------------------------------ fractional Euler records
@@ -792,9 +937,8 @@ __global__ void __launch_bounds__(128) k_records(ClipArgs A) {
     const QStore V{smem + (size_t)warp * VMAX * 2 * 32, lane};
     const long long qn = (long long)*A.qcount;
     const long long n = qn < A.qcap ? qn : A.qcap;
-    const long long q0 = (long long)blockIdx.x * blockDim.x + warp * 32;
-    if (q0 >= n) return;   // warp-uniform
-    const long long q = q0 + lane;
+    if ((long long)blockIdx.x * blockDim.x >= n) return;   // uniform over the block
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = q < n;
     Lane L{};
     long long p = 0;
@@ -1336,31 +1480,6 @@ __global__ void __launch_bounds__(128) k_volume(ClipArgs A, int vmax, int rmax) 
     }
 }
 
-// Whole-tet pieces: a tet with a single candidate lies inside one cell.
-__device__ __forceinline__ void whole_one(const ClipArgs& A, long long p) {
-    const long long t = A.pair_tet[p];
-    const uint32_t own = A.own[t];
-    int3 X[4];
-    for (int k = 0; k < 4; k++) X[k] = ld_int3(A.Xi, A.tets[4 * t + k]);
-    const int32_t* adj = A.adj + 4 * t;
-    unsigned lk = 0xf0u;   // the whole tet has a face on each tet face
-    for (int f = 0; f < 4; f++)
-        if (adj[f] >= 0) lk |= 1u << f;
-    A.pflag[p] = 1;
-    A.c_val[p] = __popc(own & 0xfu) - __popc(own & 0x3f0u) + __popc(own & 0x3c00u) - 1;
-    A.c_link[p] = (uint8_t)lk;
-    A.f_off[p] = 0;
-    A.f_cnt[p] = 0;
-    A.e_off[p] = 0;
-    A.e_cnt[p] = 0;
-    const double vt = tet_volume6(X) / 6.0;
-    const double u3 = A.unit * A.unit * A.unit;
-    A.p_vol[p] = vt * u3;
-    A.p_mom[3 * p + 0] = vt * 0.25 * ((double)X[0].x + X[1].x + X[2].x + X[3].x) * u3 * A.unit;
-    A.p_mom[3 * p + 1] = vt * 0.25 * ((double)X[0].y + X[1].y + X[2].y + X[3].y) * u3 * A.unit;
-    A.p_mom[3 * p + 2] = vt * 0.25 * ((double)X[0].z + X[1].z + X[2].z + X[3].z) * u3 * A.unit;
-}
-
 __global__ void k_whole(ClipArgs A, const int32_t* __restrict__ pairs, const int32_t* __restrict__ d_n) {
     const long long n = *d_n;
     unsigned cnt = 0;
@@ -1369,6 +1488,158 @@ __global__ void k_whole(ClipArgs A, const int32_t* __restrict__ pairs, const int
         cnt++;
     }
     dev_count(A.st, CNT_WHOLE, cnt);
+}
+
+// ---------------------------------------------------------- two candidates
+// A tet with two candidates: one radical plane, so its two pieces, their
+// records, volumes and moments follow from the plane's exact signs at the four
+// corners, in closed form, one thread per tet.  With K the corners on a
+// piece's side, an element of the piece on a tet edge that the plane cuts comes
+// twice (the cut point and the rest of the edge, the same carrier weight with
+// opposite signs), and so does one on a face that it crosses (the segment and
+// the rest of the face); what is left of V - E + F - C is
+//     w(corners in K) - w(edges within K) + w(faces within K)
+// and the radical face's polygon has a vertex per cut edge and an edge per
+// crossed face.  (The general clip, its record and its volume kernel took 312,
+// 93 and some 150 us for the 970 k such pairs of the 2 M-tet organic blob.)
+// Slots of the pairs list come in twos, both pairs of a tet.
+template <typename Real>
+__global__ void __launch_bounds__(128) k_clip2(ClipArgs A, const int32_t* __restrict__ pairs,
+                                               const int32_t* __restrict__ d_n) {
+    typedef typename std::conditional<sizeof(Real) == 4, df, double>::type T;
+    __shared__ unsigned long long base_s;
+    __shared__ unsigned wcount[4], verts;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (threadIdx.x == 0) verts = 0;
+    const bool active = 2 * q + 1 < (long long)*d_n;
+    long long p = 0, t = 0;
+    int i0 = 0, i1 = 0;
+    int3 X[4];
+    long long F[4] = {-1, -1, -1, -1};
+    unsigned K = 15;
+    if (active) {
+        p = pairs[2 * q];
+        t = A.pair_tet[p];
+        i0 = A.cand[t * RPD_MAXC];
+        i1 = A.cand[t * RPD_MAXC + 1];
+        const int4 v = *reinterpret_cast<const int4*>(A.tets + 4 * t);
+        X[0] = ld_int3(A.Xi, v.x);
+        X[1] = ld_int3(A.Xi, v.y);
+        X[2] = ld_int3(A.Xi, v.z);
+        X[3] = ld_int3(A.Xi, v.w);
+        const int3 c0 = ld_int3(A.Ci, i0), c1 = ld_int3(A.Ci, i1);
+        const long long w0 = A.W[i0], w1 = A.W[i1];
+        K = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            F[k] = pd_exact(X[k], c0, w0) - pd_exact(X[k], c1, w1);
+            K |= (F[k] < 0 ? 1u : 0u) << k;
+        }
+    }
+    const bool zero = active && (F[0] == 0 || F[1] == 0 || F[2] == 0 || F[3] == 0);
+    const bool cut = active && !zero && K != 0 && K != 15;
+    // one face record per cut tet: the block reserves its records together
+    const unsigned m = __ballot_sync(0xffffffffu, cut);
+    if (lane == 0) wcount[warp] = (unsigned)__popc(m);
+    __syncthreads();
+    unsigned before = 0, total = 0;
+    for (int w = 0; w < 4; w++) {
+        if (w < warp) before += wcount[w];
+        total += wcount[w];
+    }
+    if (threadIdx.x == 0 && total) {
+        base_s = atomicAdd(&A.rcount[0], (unsigned long long)total);
+        atomicAdd(A.qcount, 2ull * total);   // cut pieces of the bin (a statistic; nothing is queued)
+    }
+    __syncthreads();
+    const uint32_t own = active ? A.own[t] : 0;
+    unsigned ncut = 0;
+    if (cut) {
+        const int4 ad = *reinterpret_cast<const int4*>(A.adj + 4 * t);
+        const unsigned inner = (ad.x >= 0 ? 1u : 0u) | (ad.y >= 0 ? 2u : 0u) | (ad.z >= 0 ? 4u : 0u) | (ad.w >= 0 ? 8u : 0u);
+        // tet edges (bit = tet_edge_index) and faces (bit = opposite corner) by their corners
+        unsigned e_in[2] = {0, 0}, e_cut = 0, f_in[2] = {0, 0}, f_has[2] = {0, 0};
+        constexpr unsigned em[6] = {3, 5, 9, 6, 10, 12};
+#pragma unroll
+        for (int e = 0; e < 6; e++) {
+            const unsigned c = K & em[e];
+            if (c == em[e]) e_in[0] |= 1u << e;
+            else if (c == 0) e_in[1] |= 1u << e;
+            else e_cut |= 1u << e;
+        }
+#pragma unroll
+        for (int f = 0; f < 4; f++) {
+            const unsigned fm = 15u ^ (1u << f), c = K & fm;
+            if (c == fm) f_in[0] |= 1u << f;
+            else if (c == 0) f_in[1] |= 1u << f;
+            if (c) f_has[0] |= 1u << f;
+            if (c != fm) f_has[1] |= 1u << f;
+        }
+        const unsigned crossed = f_has[0] & f_has[1];
+        const unsigned we = (own >> 4) & 63u, wf = (own >> 10) & 15u;
+        ncut = __popc(e_cut);
+        const long long r = (long long)base_s + before + __popc(m & ((1u << lane) - 1u));
+        if (r < A.rcap[0]) {
+            A.rkey[0][r] = ((unsigned long long)i0 << A.key_bits) | (unsigned long long)i1;
+            A.rtet[0][r] = (int32_t)t;
+            A.rval[0][r] = (int16_t)(__popc(we & e_cut) - __popc(wf & crossed) + 1);
+            A.rlink[0][r] = (uint8_t)((crossed & inner) | (crossed << 4));
+        }
+#pragma unroll
+        for (int z = 0; z < 2; z++) {
+            const unsigned Kz = z == 0 ? K : 15u ^ K;
+            A.pflag[p + z] = 1;
+            A.c_val[p + z] = __popc(own & Kz) - __popc(we & e_in[z]) + __popc(wf & f_in[z]);
+            A.c_link[p + z] = (uint8_t)((f_has[z] & inner) | (f_has[z] << 4));
+            A.f_off[p + z] = z == 0 ? (int32_t)r : 0;
+            A.f_cnt[p + z] = z == 0 ? 1 : 0;
+            A.e_off[p + z] = 0;
+            A.e_cnt[p + z] = 0;
+        }
+        const double u3 = A.unit * A.unit * A.unit;
+        const int x0[3] = {X[0].x, X[0].y, X[0].z};
+        for (int z = 0; z < 2; z++) {
+            T fr, mom[3];
+            one_plane_piece<T>(F, X, fr, mom);
+            if constexpr (sizeof(Real) == 4) {   // double-float to the end, one conversion per output
+                const df vt6 = df_from_i128(tet_det6(X));
+                A.p_vol[p + z] = df_to_double(df_mul(vt6, fr)) * (u3 / 6.0);
+                for (int k = 0; k < 3; k++)
+                    A.p_mom[3 * (p + z) + k] =
+                        df_to_double(df_mul(vt6, df_add(df_mul(fr, df_from_i64(x0[k])), mom[k]))) * (u3 * A.unit / 6.0);
+            } else {
+                const double vt = tet_volume6(X) / 6.0;
+                A.p_vol[p + z] = vt * fr * u3;
+                for (int k = 0; k < 3; k++) A.p_mom[3 * (p + z) + k] = vt * (fr * (double)x0[k] + mom[k]) * u3 * A.unit;
+            }
+            for (int k = 0; k < 4; k++) F[k] = -F[k];   // the other piece
+        }
+    } else if (active) {
+        if (zero) dev_fail(A.st, RPD_E_DEGENERATE, CNT_DEGENERATE);
+        for (int z = 0; z < 2; z++) {
+            const bool whole = !zero && K == (z == 0 ? 15u : 0u);   // the plane misses the tet
+            if (whole) {
+                whole_one(A, p + z);
+                continue;
+            }
+            A.pflag[p + z] = 0;
+            A.c_val[p + z] = 0;
+            A.c_link[p + z] = 0;
+            A.f_off[p + z] = A.e_off[p + z] = 0;
+            A.f_cnt[p + z] = A.e_cnt[p + z] = 0;
+            A.p_vol[p + z] = 0.0;
+            for (int k = 0; k < 3; k++) A.p_mom[3 * (p + z) + k] = 0.0;
+        }
+    }
+    // statistics: a vertex per cut edge and piece, each with its orientation known from the signs
+    const unsigned tot = __reduce_add_sync(0xffffffffu, 2 * ncut);
+    if (lane == 0 && tot) atomicAdd(&verts, tot);
+    __syncthreads();
+    if (threadIdx.x == 0 && verts) {
+        atomicAdd(&A.st->cnt[CNT_NEWVERT1], (unsigned long long)verts);
+        atomicAdd(&A.st->cnt[CNT_PRED_FAST], (unsigned long long)verts);
+    }
 }
 
 // Bins by candidate count n: 0: n = 1 (whole tet), 1..3: n = 2..4,
@@ -1461,13 +1732,26 @@ inline void raise_smem_limit(const void* fn, size_t bytes, SmemLimit& L) {
     }
 }
 
+// Pairs per warp of a bin of n: a warp runs as long as its lanes' control
+// flow together, so where a bin has less than a warp of 32 for every SM its
+// warps take fewer pairs.  (205k-tet slab, FP32: splitting below 6 warps per SM
+// 1.65 ms a build, below one 1.54, never 1.55; with FP64 the warps fill the
+// FP64 pipe whatever their active lanes: 60k-tet blob 2.23, 2.30, never 2.18.)
+template <typename Real>
+inline int pairs_per_warp(long long n) {
+    int per = 32;
+    while (sizeof(Real) == 4 && per > 4 && n < 152ll * per) per /= 2;
+    return per;
+}
+
 template <typename Real, int VMAX, int WARPS>
 void launch_clip_t(const ClipArgs& a, const int32_t* pairs, const int32_t* d_n, long long n, cudaStream_t s) {
     if (n <= 0) return;
-    const size_t smem = (size_t)WARPS * VMAX * (PrecTraits<Real>::VW + 1) * 32 * sizeof(uint32_t);
+    const size_t smem = (size_t)WARPS * Store<Real, VMAX>::WORDS * 32 * sizeof(uint32_t);
     static SmemLimit lim;
     raise_smem_limit((const void*)k_clip<Real, VMAX>, smem, lim);
-    k_clip<Real, VMAX><<<grid_for(n, 32 * WARPS), 32 * WARPS, smem, s>>>(a, pairs, d_n);
+    const int per = pairs_per_warp<Real>(n);
+    k_clip<Real, VMAX><<<grid_for(n, per * WARPS), 32 * WARPS, smem, s>>>(a, pairs, d_n, per);
     note_launch();
 }
 
@@ -1514,8 +1798,19 @@ void launch_whole_tets(const ClipArgs& a, const int32_t* pairs, const int32_t* d
     note_launch();
 }
 
+// Two candidates take the closed form, unless a debug switch sends the
+// predicates through the clip's slow stages.
+bool clip_closed_form(const ClipArgs& a, int bin) { return bin == 1 && !a.force_slow; }
+
 void launch_clip(const ClipArgs& a, int bin, int precision, const int32_t* pairs, const int32_t* d_n, long long n,
                  cudaStream_t s) {
+    if (clip_closed_form(a, bin)) {
+        if (n <= 0) return;
+        if (precision == RPD_FP32_FILTERED) k_clip2<float><<<nblk(n / 2, 128), 128, 0, s>>>(a, pairs, d_n);
+        else k_clip2<double><<<nblk(n / 2, 128), 128, 0, s>>>(a, pairs, d_n);
+        note_launch();
+        return;
+    }
     if (precision == RPD_FP32_FILTERED) {
         switch (bin) {
             case 1: launch_clip_t<float, 6, 4>(a, pairs, d_n, n, s); break;
@@ -1528,11 +1823,11 @@ void launch_clip(const ClipArgs& a, int bin, int precision, const int32_t* pairs
         }
     } else {
         switch (bin) {
-            case 1: launch_clip_t<double, 6, 4>(a, pairs, d_n, n, s); break;
-            case 2: launch_clip_t<double, 8, 4>(a, pairs, d_n, n, s); break;
-            case 3: launch_clip_t<double, 10, 4>(a, pairs, d_n, n, s); break;
-            case 4: launch_clip_t<double, 14, 2>(a, pairs, d_n, n, s); break;
-            case 5: launch_clip_t<double, 18, 2>(a, pairs, d_n, n, s); break;
+            case 1: launch_clip_t<double, 6, 1>(a, pairs, d_n, n, s); break;
+            case 2: launch_clip_t<double, 8, 1>(a, pairs, d_n, n, s); break;
+            case 3: launch_clip_t<double, 10, 1>(a, pairs, d_n, n, s); break;
+            case 4: launch_clip_t<double, 14, 1>(a, pairs, d_n, n, s); break;
+            case 5: launch_clip_t<double, 18, 1>(a, pairs, d_n, n, s); break;
             case 6: launch_clip_t<double, 34, 1>(a, pairs, d_n, n, s); break;
             case 7: launch_clip_t<double, 66, 1>(a, pairs, d_n, n, s); break;
         }
@@ -1548,6 +1843,7 @@ void launch_records_t(const ClipArgs& a, long long nmax, cudaStream_t s) {
 }
 
 void launch_records(const ClipArgs& a, int bin, long long n, cudaStream_t s) {
+    if (clip_closed_form(a, bin)) return;   // emitted by the clip
     switch (bin) {
         case 1: launch_records_t<6, 4>(a, n, s); break;
         case 2: launch_records_t<8, 4>(a, n, s); break;
@@ -1561,7 +1857,7 @@ void launch_records(const ClipArgs& a, int bin, long long n, cudaStream_t s) {
 }
 
 void launch_volume(const ClipArgs& a, int bin, int precision, long long n, cudaStream_t s) {
-    if (bin < 1) return;
+    if (bin < 1 || clip_closed_form(a, bin)) return;
     static const int rmax[RPD_NBINS] = {1, 2, 3, 4, 6, 8, 16, 32};   // most candidates of a bin's tets
     const int vw = bin <= 5 ? 4 : (bin == 6 ? 2 : 1);
     if (precision == RPD_FP32_FILTERED) launch_volume_t<float>(a, clip_vmax(bin), rmax[bin], vw, n, s);
