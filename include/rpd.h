@@ -63,18 +63,19 @@ typedef enum { RPD_FP64 = 0, RPD_FP32_FILTERED = 1 } rpd_precision;
 
 typedef struct {
     int32_t precision;    /* rpd_precision                                        */
-    int32_t k;            /* power neighbours kept per mesh vertex, 1..32          */
+    int32_t k;            /* power neighbours per tet corner, 1..32: a tet with more
+                             than min(4 k, 32) spheres near it takes the slower
+                             grid search (the diagram does not depend on k)       */
     int32_t grid_bits;    /* coordinates and radii are rounded to multiples of
                              2^-grid_bits; |x|*2^grid_bits must stay < 2^21       */
     int32_t debug_checks; /* test switches (0 in production): value 1 sends every
                              non-corner clip predicate past the first-stage
                              filter to the FP64 stage, value 2 straight to the
-                             exact 256-bit stage; bit 4 makes the neighbour
-                             search keep distance and id apart (the form used
-                             above 2^17 spheres); bit 8 keeps the heaviest
-                             spheres out of the neighbour grid and scans them
-                             first (a tuning choice, off by default: slower on
-                             the organic blob).  Results must not change.       */
+                             exact 256-bit stage; bit 4 takes the candidates
+                             from neighbour lists of k spheres per mesh vertex
+                             (the form of rpd_euler_static, in the variant used
+                             above 2^17 spheres); bit 8 is accepted and has no
+                             effect.  Results must not change.                  */
     int32_t edge_lengths; /* 1: the volume pass also measures every restricted
                              power edge segment (rpd_edge_lengths and rpd_medial
                              need it, and partial updates keep it); 0: skipped  */

@@ -114,8 +114,6 @@ struct rpd_ctx {
     int64_t* cell_start = nullptr;
     int32_t* cell_ids = nullptr;
     long long* cell_wmax = nullptr;
-    int32_t* knn = nullptr;
-    long long* dplus = nullptr;
     int32_t *cand_cnt = nullptr, *cand = nullptr, *fb_list = nullptr, *fb_count = nullptr;
     uint8_t* cand_ord = nullptr;
     int64_t* pair_off = nullptr;
@@ -157,6 +155,7 @@ struct rpd_ctx {
     long long *d_voff = nullptr, *d_toff = nullptr, *d_soff = nullptr;
     std::vector<long long> h_voff, h_toff, h_soff;
     long long max_shape_ncap = 0;
+    CandPlan plan;   // the candidate stage's blocks and cells
     // mesh bounding box (world units), computed on first use
     bool have_bbox = false;
     double bb_lo[3] = {0, 0, 0}, bb_hi[3] = {0, 0, 0};
@@ -406,6 +405,10 @@ float elapsed(rpd_ctx* c, int a, int b) {
 
 rpd_status build_rest(rpd_ctx* c, rpd_ctx* old);
 
+// The candidates come from per-vertex neighbour lists (knn.cu) instead of
+// packets (cand.cu): only when a debug bit asks for that form.
+bool per_vertex_lists(const rpd_ctx* c) { return (c->opt.debug_checks & 4) != 0; }
+
 // Device, timing events and side streams of a context; the chunk for every
 // buffer sized before the pair count is known.
 rpd_status begin(rpd_ctx* c) {
@@ -419,11 +422,17 @@ rpd_status begin(rpd_ctx* c) {
     if (!bin_streams()) return fail(c, RPD_E_CUDA, "stream creation failed");
     record(c, 0);
     const long long ncap = 2 * ns + 64, pcap = 4 * nt + 1024;
-    const size_t est = sizeof(DevState) + 4 * 3 * (nv + ns) + 8 * ns + 4 * 4 * nt + 4 * nt + 4 * 4 * nt +
-                       prep_tmp_bytes(nt, nv) + sizeof(GridParams) + 8 * (ncap + 1) + 4 * ns + 8 * 2 * ncap +
-                       grid_tmp_bytes(ns, ncap) + 4 * nv * c->K + 8 * nv + 16 * ns + 8 * ns + knn_tmp_bytes(nv) +
-                       4 * nt + (4 + 1) * nt * RPD_MAXC + 4 * nt + 4 + 8 * (nt + 1) + scan_tmp_bytes(nt + 1) +
-                       8 * RPD_NBINS + 8 * pcap + 8 * (3 + RPD_NBINS) + nt + 8 + 42 * 256;
+    size_t est = sizeof(DevState) + 4 * 3 * (nv + ns) + 8 * ns + 4 * 4 * nt + 4 * nt + 4 * 4 * nt +
+                 prep_tmp_bytes(nt, nv) + sizeof(GridParams) + 8 * (ncap + 1) + 4 * ns + 8 * 2 * ncap +
+                 grid_tmp_bytes(ns, ncap) + 16 * ns + 8 * ns + 4 * nt + (4 + 1) * nt * RPD_MAXC + 4 * nt + 4 +
+                 8 * (nt + 1) + scan_tmp_bytes(nt + 1) + 8 * RPD_NBINS + 8 * pcap + 8 * (3 + RPD_NBINS) + nt + 8 +
+                 42 * 256;
+    if (per_vertex_lists(c)) {
+        est += 4 * nv * c->K + 8 * nv + knn_tmp_bytes(nv);
+    } else {
+        cand_plan(c->h_voff.data(), c->h_toff.data(), c->h_soff.data(), c->nshapes, nv, nt, ns, c->plan);
+        est += cand_tmp_bytes(c->plan, nt, nv, ns);
+    }
     NEED(c->reserve(est));
     return RPD_OK;
 }
@@ -515,43 +524,36 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     // cells and an end offset each, laid end to end)
     const bool batch = c->nshapes > 1;
     long long ncap = batch ? 2 * ns + 65ll * c->nshapes : 2 * ns + 64;
-    c->gp = c->alloc<GridParams>(c->nshapes);
-    c->cell_start = c->alloc<int64_t>(ncap + 1);
-    c->cell_ids = c->alloc<int32_t>(ns);
-    c->cell_wmax = c->alloc<long long>(2 * ncap);
-    void* gtmp = c->alloc<char>(grid_tmp_bytes(ns, ncap));
-    c->knn = c->alloc<int32_t>(nv * c->K);
-    c->dplus = c->alloc<long long>(nv);
-    NEED(c->gp && c->cell_start && c->cell_ids && c->cell_wmax && gtmp && c->knn && c->dplus);
-    int4* cell_sph = c->alloc<int4>(ns);
-    long long* cell_w = c->alloc<long long>(ns);
-    void* ktmp = c->alloc<char>(knn_tmp_bytes(nv));
-    NEED(cell_sph && cell_w && ktmp);
-    // with debug bit 8 the heaviest spheres stay out of the grid and every
-    // vertex scans them first (warp-form neighbour search of one shape only)
-    const bool two_word = (c->opt.debug_checks & 4) != 0;
-    const bool heavy = !batch && !two_word && ns <= (1 << 17) && (c->opt.debug_checks & 8) && heavy_count(ns) > 0;
-    long long* wcut = nullptr;
-    int4* hsph = nullptr;
-    long long* hw = nullptr;
-    int* nheavy = nullptr;
-    if (heavy) {
-        wcut = c->alloc<long long>(1);
-        hsph = c->alloc<int4>(heavy_count(ns));
-        hw = c->alloc<long long>(heavy_count(ns));
-        nheavy = c->alloc<int>(1);
-        NEED(wcut && hsph && hw && nheavy);
-        launch_heavy_select(c->Ci, c->W, ns, wcut, hsph, hw, nheavy, s);
+    const bool lists = per_vertex_lists(c);
+    int4* cell_sph = nullptr;
+    long long* cell_w = nullptr;
+    if (lists) {
+        c->gp = c->alloc<GridParams>(c->nshapes);
+        c->cell_start = c->alloc<int64_t>(ncap + 1);
+        c->cell_ids = c->alloc<int32_t>(ns);
+        c->cell_wmax = c->alloc<long long>(2 * ncap);
+        void* gtmp = c->alloc<char>(grid_tmp_bytes(ns, ncap));
+        cell_sph = c->alloc<int4>(ns);
+        cell_w = c->alloc<long long>(ns);
+        NEED(c->gp && c->cell_start && c->cell_ids && c->cell_wmax && gtmp && cell_sph && cell_w);
+        if (batch)
+            launch_sphere_grid_batch(c->Ci, c->W, c->d_soff, c->nshapes, ncap, c->gp, c->cell_start, c->cell_ids,
+                                     cell_sph, cell_w, c->cell_wmax, c->max_shape_ncap, s);
+        else
+            launch_sphere_grid(c->Ci, c->W, ns, ncap, c->gp, c->cell_start, c->cell_ids, cell_sph, cell_w,
+                               c->cell_wmax, gtmp, s);
     }
-    if (batch)
-        launch_sphere_grid_batch(c->Ci, c->W, c->d_soff, c->nshapes, ncap, c->gp, c->cell_start, c->cell_ids, cell_sph,
-                                 cell_w, c->cell_wmax, c->max_shape_ncap, s);
-    else
-        launch_sphere_grid(c->Ci, c->W, ns, ncap, c->gp, c->cell_start, c->cell_ids, cell_sph, cell_w, c->cell_wmax,
-                           gtmp, s, wcut);
-    launch_knn(c->Xi, nv, ns, c->gp, c->cell_start, cell_sph, cell_w, c->cell_wmax, ncap, c->K, c->knn, c->dplus, ktmp,
-               &c->st->err, two_word, s, c->d_voff, c->nshapes, hsph, hw, nheavy);
-    TRY(cuda_check(c, "knn launch"));
+    int32_t* knn = nullptr;
+    long long* dplus = nullptr;
+    if (lists) {
+        knn = c->alloc<int32_t>(nv * c->K);
+        dplus = c->alloc<long long>(nv);
+        void* ktmp = c->alloc<char>(knn_tmp_bytes(nv));
+        NEED(knn && dplus && ktmp);
+        launch_knn(c->Xi, nv, ns, c->gp, c->cell_start, cell_sph, cell_w, c->cell_wmax, ncap, c->K, knn, dplus, ktmp,
+                   &c->st->err, true, s, c->d_voff, c->nshapes);
+    }
+    TRY(cuda_check(c, "neighbour launch"));
     record(c, 3);
     // ---- A2
     c->cand_cnt = c->alloc<int32_t>(nt);
@@ -565,9 +567,30 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     c->bin_fill = c->alloc<int32_t>(RPD_NBINS);
     NEED(c->cand_cnt && c->cand && c->cand_ord && c->fb_list && c->fb_count && c->pair_off && stmp && c->bin_count &&
          c->bin_fill);
-    launch_candidates(c->tets, nt, nv, c->Xi, c->Ci, c->W, c->knn, c->dplus, c->K, c->gp, c->cell_start,
-                      c->cell_ids, c->cell_wmax, c->cand_cnt, c->cand, c->cand_ord, c->fb_list, c->fb_count, c->st, s,
-                      c->d_voff, c->nshapes, hsph, hw, nheavy);
+    if (lists) {
+        launch_candidates(c->tets, nt, nv, c->Xi, c->Ci, c->W, knn, dplus, c->K, c->gp, c->cell_start, c->cell_ids,
+                          c->cell_wmax, c->cand_cnt, c->cand, c->cand_ord, c->fb_list, c->fb_count, c->st, s,
+                          c->d_voff, c->nshapes);
+    } else {
+        void* ctmp = c->alloc<char>(cand_tmp_bytes(c->plan, nt, nv, ns));
+        NEED(ctmp);
+        CandArgs a{};
+        a.T = c->tets;
+        a.nt = nt;
+        a.nv = nv;
+        a.ns = ns;
+        a.Xi = c->Xi;
+        a.Ci = c->Ci;
+        a.W = c->W;
+        a.gather = std::min(4 * c->K, RPD_MAXC);   // four corners' worth of k neighbours
+        a.cand_cnt = c->cand_cnt;
+        a.cand = c->cand;
+        a.cand_ord = c->cand_ord;
+        a.fb_list = c->fb_list;
+        a.fb_count = c->fb_count;
+        a.st = c->st;
+        launch_candidates_packet(a, c->plan, c->d_voff, c->d_soff, ctmp, s);
+    }
     scan_excl(c->cand_cnt, c->pair_off, nt, stmp, s);
     if (old) {   // partial update: clip only the tets whose candidates changed
         c->changed = c->alloc<uint8_t>(nt);

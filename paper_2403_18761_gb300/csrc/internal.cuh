@@ -37,14 +37,7 @@ size_t grid_tmp_bytes(long long ns, long long ncap);
 // of each row of cells along x (index z * dim.y + y).
 void launch_sphere_grid(const int32_t* Ci, const long long* W, long long ns, long long ncap, GridParams* gp,
                         int64_t* cell_start, int32_t* cell_ids, int4* cell_sph, long long* cell_w,
-                        long long* cell_wmax, void* tmp, cudaStream_t s, const long long* wcut = nullptr);
-// Heavy spheres (the up to min(128, ns / 128) largest weights): *wcut = the
-// largest weight left in the grid (spheres above it are heavy), hsph/hw
-// their (centre, id) and weights in id order, *nheavy their count.  Pass
-// wcut to launch_sphere_grid and the rest to launch_knn / launch_candidates.
-int heavy_count(long long ns);
-void launch_heavy_select(const int32_t* Ci, const long long* W, long long ns, long long* wcut, int4* hsph,
-                         long long* hw, int* nheavy, cudaStream_t s);
+                        long long* cell_wmax, void* tmp, cudaStream_t s);
 // k nearest spheres in power distance of every mesh vertex, with D+ = a lower
 // bound of the power distance of every sphere left out of the list.
 // tmp must hold knn_tmp_bytes(nv); ncap bounds the number of grid cells.
@@ -52,8 +45,7 @@ size_t knn_tmp_bytes(long long nv);
 void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams* gp, const int64_t* cell_start,
                 const int4* cell_sph, const long long* cell_w, const long long* cell_wmax, long long ncap, int K,
                 int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s,
-                const long long* voff = nullptr, int nshapes = 1, const int4* hsph = nullptr,
-                const long long* hw = nullptr, const int* nheavy = nullptr);
+                const long long* voff = nullptr, int nshapes = 1);
 // Batches: one grid per shape, all built by one launch (a block per shape).
 // Shape s owns spheres [soff[s], soff[s + 1]) (device array) and cells
 // [2 soff[s] + 65 s, 2 soff[s + 1] + 65 (s + 1)) of cell_start (its
@@ -72,8 +64,63 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                        const GridParams* gp, const int64_t* cell_start, const int32_t* cell_ids,
                        const long long* cell_wmax, int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord,
                        int32_t* fb_list, int32_t* fb_count, DevState* st, cudaStream_t s,
-                       const long long* voff = nullptr, int nshapes = 1, const int4* hsph = nullptr,
-                       const long long* hw = nullptr, const int* nheavy = nullptr);
+                       const long long* voff = nullptr, int nshapes = 1);
+
+// The grid-search fallback of the tets in fb_list.  knn == NULL: cand[32 t]
+// holds the sphere that gives tet t's thresholds; gp == NULL: no sphere grid, every sphere of the shape is tested (soff: shape s owns spheres
+// [soff[s], soff[s + 1]); without a batch all ns).
+void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
+                                const long long* W, long long ns, const int32_t* knn, int K, const GridParams* gp,
+                                const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
+                                const int32_t* fb_list, const int32_t* fb_count, int32_t* cand_cnt, int32_t* cand,
+                                uint8_t* cand_ord, DevState* st, const long long* voff, const long long* soff,
+                                int nshapes, cudaStream_t s);
+
+// ---------------------------------------------------------------- cand.cu
+// A shape's ranges of vertices, tets and spheres, its first vertex and tet
+// packet, leaf, node and order cells, and the halvings of its orders.
+struct CandShape {
+    long long v0, v1, t0, t1, s0, s1;
+    long long pv, pt, l0, n0, cv, ct, cs;
+    int bv, bt, bs;
+};
+// Box of the centres of a leaf's spheres, or of a node's (w: not used).
+struct Leaf {
+    int4 lo, hi;
+};
+struct CandArgs {
+    const int32_t* T;
+    long long nt, nv, ns;
+    const int32_t *Xi, *Ci;
+    const long long* W;
+    int gather;   // spheres a tet may gather before it goes to the fallback (<= RPD_MAXC)
+    int32_t *cand_cnt, *cand;
+    uint8_t* cand_ord;
+    int32_t *fb_list, *fb_count;
+    DevState* st;
+    // set by the launch
+    int nshapes;
+    const CandShape* shapes;   // NULL: one shape, `one`
+    CandShape one;
+    const int32_t *order_t, *order_v, *order_s;   // NULL: as given
+    long long npv, npt, nleaf, nnode;
+    const int4* sph;        // spheres in order: centre, id
+    const long long* sw;    // weights
+    const Leaf *leaf, *node;
+    const long long *lwmax, *nwmax;
+};
+struct CandPlan {
+    bool ordered = false;
+    long long npv = 0, npt = 0, nleaf = 0, nnode = 0, ncell = 0;
+    std::vector<CandShape> shapes;
+};
+// Candidates of every tet by packets: plan on the host (offsets as for
+// batches, not read with one shape), scratch, launches.
+void cand_plan(const long long* voff, const long long* toff, const long long* soff, int nshapes, long long nv,
+               long long nt, long long ns, CandPlan& P);
+size_t cand_tmp_bytes(const CandPlan& P, long long nt, long long nv, long long ns);
+void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* voff, const long long* soff, void* tmp,
+                              cudaStream_t s);
 
 // ---------------------------------------------------------------- clip.cu
 struct ClipArgs {

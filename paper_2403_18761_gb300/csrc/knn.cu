@@ -108,13 +108,12 @@ __device__ __forceinline__ int shape_of(const long long* __restrict__ voff, int 
 // Bounding box of the sphere centres and the largest weight, reduced over
 // the block; thread 0 returns the grid parameters in *out (shared memory).
 __device__ void block_grid_params(const int32_t* __restrict__ Ci, const long long* __restrict__ W, long long ns,
-                                  long long ncap, GridParams* out, long long cut = LLONG_MAX) {
+                                  long long ncap, GridParams* out) {
     __shared__ int smin[3][32], smax[3][32];
     __shared__ long long swm[32];
     int mn[3] = {INT_MAX, INT_MAX, INT_MAX}, mx[3] = {INT_MIN, INT_MIN, INT_MIN};
     long long wm = 0;
     for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-        if (W[i] > cut) continue;   // a heavy sphere: kept out of the grid
         for (int a = 0; a < 3; a++) {
             int v = Ci[3 * i + a];
             mn[a] = min(mn[a], v);
@@ -144,9 +143,9 @@ __device__ void block_grid_params(const int32_t* __restrict__ Ci, const long lon
 }
 
 __global__ void k_bbox(const int32_t* __restrict__ Ci, const long long* __restrict__ W, long long ns, long long ncap,
-                       GridParams* gp, const long long* __restrict__ wcut) {
+                       GridParams* gp) {
     __shared__ GridParams sg;
-    block_grid_params(Ci, W, ns, ncap, &sg, wcut ? *wcut : LLONG_MAX);
+    block_grid_params(Ci, W, ns, ncap, &sg);
     if (threadIdx.x == 0) *gp = sg;
 }
 
@@ -154,7 +153,6 @@ __global__ void k_bbox(const int32_t* __restrict__ Ci, const long long* __restri
 // grid parameters, per-cell counts in shared memory, their exclusive scan
 // (cell_start) and the fill, with no launches in between.
 constexpr int GRID_SMALL_CAP = 11264;   // counts within 44 KB of shared memory
-constexpr int HEAVY_MAX = 128;          // heavy spheres kept out of the grid at most
 
 __device__ __forceinline__ int block_excl_scan(int v, int* total) {
     __shared__ int wsum[32];
@@ -185,12 +183,10 @@ __global__ void __launch_bounds__(1024) k_grid_small(const int32_t* __restrict__
                                                      long long ns, long long ncap, GridParams* gp,
                                                      int64_t* __restrict__ start, int32_t* __restrict__ ids,
                                                      int4* __restrict__ sph, long long* __restrict__ sw,
-                                                     long long* __restrict__ cwmax, long long* __restrict__ rwmax,
-                                                     const long long* __restrict__ wcut) {
+                                                     long long* __restrict__ cwmax, long long* __restrict__ rwmax) {
     extern __shared__ int scount[];
     __shared__ GridParams sg;
-    const long long cut = wcut ? *wcut : LLONG_MAX;
-    block_grid_params(Ci, W, ns, ncap, &sg, cut);
+    block_grid_params(Ci, W, ns, ncap, &sg);
     for (long long q = threadIdx.x; q < ncap; q += blockDim.x) {
         scount[q] = 0;
         cwmax[q] = 0;
@@ -200,7 +196,6 @@ __global__ void __launch_bounds__(1024) k_grid_small(const int32_t* __restrict__
     const GridParams g = sg;
     if (threadIdx.x == 0) *gp = g;
     for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-        if (W[i] > cut) continue;
         const int3 c = cell_of(ld_int3(Ci, i), g);
         const int q = (c.z * g.dim.y + c.y) * g.dim.x + c.x;
         atomicAdd(&scount[q], 1);
@@ -223,7 +218,6 @@ __global__ void __launch_bounds__(1024) k_grid_small(const int32_t* __restrict__
     if (threadIdx.x == 0) start[ncap] = total;
     __syncthreads();
     for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-        if (W[i] > cut) continue;
         const int3 ci = ld_int3(Ci, i);
         const int3 c = cell_of(ci, g);
         const int q = (c.z * g.dim.y + c.y) * g.dim.x + c.x;
@@ -231,66 +225,6 @@ __global__ void __launch_bounds__(1024) k_grid_small(const int32_t* __restrict__
         ids[pos] = (int32_t)i;
         sph[pos] = make_int4(ci.x, ci.y, ci.z, (int)i);
         sw[pos] = W[i];
-    }
-}
-
-// Heavy spheres: the up to H largest power weights.  The neighbour walk stops
-// once the next shell's distance minus the largest weight of the grid exceeds
-// the K-th distance, so a few heavy spheres would keep every vertex walking;
-// they are kept out of the grid and every vertex evaluates them first.  One
-// block: the (H + 1)-th largest weight t by an 8-bit radix select from the
-// top byte down (weights are >= 0), then the spheres with W > t (at most H)
-// in id order by a chunked block scan.
-__global__ void __launch_bounds__(1024) k_heavy_select(const int32_t* __restrict__ Ci,
-                                                       const long long* __restrict__ W, long long ns, int H,
-                                                       long long* __restrict__ wcut, int4* __restrict__ hsph,
-                                                       long long* __restrict__ hw, int* __restrict__ nheavy) {
-    __shared__ int hist[256];
-    __shared__ unsigned long long sprefix;
-    __shared__ long long sneed;
-    if (threadIdx.x == 0) {
-        sprefix = 0;
-        sneed = H + 1;
-    }
-    for (int pos = 7; pos >= 0; pos--) {
-        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
-        __syncthreads();
-        const unsigned long long prefix = sprefix;
-        const unsigned long long hmask = pos == 7 ? 0ull : (~0ull << (8 * (pos + 1)));
-        for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-            const unsigned long long v = (unsigned long long)W[i];
-            if ((v & hmask) == prefix) atomicAdd(&hist[(v >> (8 * pos)) & 0xff], 1);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long need = sneed, cum = 0;
-            int b = 255;
-            for (; b > 0; b--) {
-                if (cum + hist[b] >= need) break;
-                cum += hist[b];
-            }
-            sneed = need - cum;
-            sprefix = prefix | ((unsigned long long)b << (8 * pos));
-        }
-        __syncthreads();
-    }
-    const long long t = (long long)sprefix;
-    int base = 0;
-    for (long long c0 = 0; c0 < ns; c0 += blockDim.x) {
-        const long long i = c0 + threadIdx.x;
-        const int f = i < ns && W[i] > t;
-        int total;
-        const int at = base + block_excl_scan(f, &total);
-        if (f && at < H) {
-            hsph[at] = make_int4(Ci[3 * i], Ci[3 * i + 1], Ci[3 * i + 2], (int)i);
-            hw[at] = W[i];
-        }
-        base += total;
-        __syncthreads();   // block_excl_scan's shared words are reused
-    }
-    if (threadIdx.x == 0) {
-        *wcut = t;
-        *nheavy = min(base, H);
     }
 }
 
@@ -357,10 +291,9 @@ __global__ void __launch_bounds__(1024) k_grid_batch(const int32_t* __restrict__
 
 __global__ void k_cell_count(const int32_t* __restrict__ Ci, const long long* __restrict__ W, long long ns,
                              const GridParams* __restrict__ gp, int32_t* __restrict__ count,
-                             long long* __restrict__ cwmax, long long* __restrict__ rwmax,
-                             const long long* __restrict__ wcut) {
+                             long long* __restrict__ cwmax, long long* __restrict__ rwmax) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ns || (wcut && W[i] > *wcut)) return;
+    if (i >= ns) return;
     GridParams g = *gp;
     int3 c = cell_of(ld_int3(Ci, i), g);
     int q = (c.z * g.dim.y + c.y) * g.dim.x + c.x;
@@ -373,9 +306,9 @@ __global__ void k_cell_count(const int32_t* __restrict__ Ci, const long long* __
 __global__ void k_cell_fill(const int32_t* __restrict__ Ci, const long long* __restrict__ W, long long ns,
                             const GridParams* __restrict__ gp, const int64_t* __restrict__ start,
                             int32_t* __restrict__ fill, int32_t* __restrict__ ids, int4* __restrict__ sph,
-                            long long* __restrict__ sw, const long long* __restrict__ wcut) {
+                            long long* __restrict__ sw) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ns || (wcut && W[i] > *wcut)) return;
+    if (i >= ns) return;
     GridParams g = *gp;
     int3 c = ld_int3(Ci, i);
     int3 cc = cell_of(c, g);
@@ -757,16 +690,13 @@ __device__ __forceinline__ void knn_insert(unsigned long long key, unsigned long
     }
 }
 
-template <bool HEAVY>
 __global__ void __launch_bounds__(256, 4) k_knn_warp(const int32_t* __restrict__ Xi, const uint32_t* __restrict__ vorder,
                                                   long long nv, const GridParams* __restrict__ gp,
                                                   const int64_t* __restrict__ start_all, const int4* __restrict__ sph,
                                                   const long long* __restrict__ sw,
                                                   const long long* __restrict__ rwmax_all, int K,
                                                   int32_t* __restrict__ knn, long long* __restrict__ dplus,
-                                                  const long long* __restrict__ voff, int nshapes,
-                                                  const int4* __restrict__ hsph, const long long* __restrict__ hw,
-                                                  const int* __restrict__ nheavy) {
+                                                  const long long* __restrict__ voff, int nshapes) {
     typedef unsigned long long U;
     const unsigned FULL = 0xffffffffu;
     const U EMPTY = ~0ull;
@@ -783,16 +713,6 @@ __global__ void __launch_bounds__(256, 4) k_knn_warp(const int32_t* __restrict__
     long long dp = LLONG_MAX;  // smallest distance known to be outside the list
     int3 plo = make_int3(1, 1, 1), phi = make_int3(0, 0, 0);   // processed box (empty)
     long long lb2 = LLONG_MAX;
-    // the heavy spheres, kept out of the grid, first
-    const int nh = HEAVY ? *nheavy : 0;
-    for (int hb = 0; hb < nh; hb += 32) {
-        U key = EMPTY;
-        if (hb + lane < nh) {
-            const int4 cs = hsph[hb + lane];
-            key = knn_key(pd_exact(x, make_int3(cs.x, cs.y, cs.z), hw[hb + lane]), cs.w);
-        }
-        knn_insert(key, L, dp, K, lane);
-    }
     for (int r = 0; r < (1 << 22); r++) {
         const int3 blo = make_int3(max(c.x - r, 0), max(c.y - r, 0), max(c.z - r, 0));
         const int3 bhi = make_int3(min(c.x + r, g.dim.x - 1), min(c.y + r, g.dim.y - 1), min(c.z + r, g.dim.z - 1));
@@ -1096,11 +1016,12 @@ constexpr int FB_THREADS = 256;
 
 __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
     const int32_t* __restrict__ T, long long nv, const int32_t* __restrict__ Xi, const int32_t* __restrict__ Ci,
-    const long long* __restrict__ W, const int32_t* __restrict__ knn, int K, const GridParams* __restrict__ gp,
-    const int64_t* __restrict__ start_all, const int32_t* __restrict__ ids, const long long* __restrict__ cwmax_all,
+    const long long* __restrict__ W, long long ns, const int32_t* __restrict__ knn, int K,
+    const GridParams* __restrict__ gp, const int64_t* __restrict__ start_all, const int32_t* __restrict__ ids,
+    const long long* __restrict__ cwmax_all,
     const int32_t* __restrict__ fb_list, const int32_t* __restrict__ fb_count, int32_t* __restrict__ cand_cnt,
     int32_t* __restrict__ cand, uint8_t* __restrict__ cand_ord, DevState* st, const long long* __restrict__ voff,
-    int nshapes, const int4* __restrict__ hsph, const long long* __restrict__ hw, const int* __restrict__ nheavy) {
+    const long long* __restrict__ soff, int nshapes) {
     const unsigned FULL = 0xffffffffu;
     __shared__ int sid[FB_GATHER];
     __shared__ long long sD[FB_GATHER][4];
@@ -1108,7 +1029,6 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
     __shared__ int sn;
     const int tid = threadIdx.x, lane = tid & 31;
     const long long nfb = *fb_count;
-    const int nh = nheavy ? *nheavy : 0;
     for (long long q = blockIdx.x; q < nfb; q += gridDim.x) {
         const long long t = fb_list[q];   // uniform over the block
         int v[4];
@@ -1117,13 +1037,23 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             if (tid == 0) cand_cnt[t] = 0;
             continue;
         }
-        // the grid of the tet's shape (its first corner's)
-        const GridParams g = gp[shape_of(voff, nshapes, v[0])];
+        // the grid and the spheres of the tet's shape (its first corner's)
+        const int shp = shape_of(voff, nshapes, v[0]);
+        const long long s0 = nshapes > 1 && soff ? soff[shp] : 0, s1 = nshapes > 1 && soff ? soff[shp + 1] : ns;
+        GridParams g{};
+        if (gp) g = gp[shp];
         const int64_t* __restrict__ start = start_all + g.cbase;
         const long long* __restrict__ cwmax = cwmax_all + g.cbase;
 
+        // spheres whose corner distances are the thresholds to choose from:
+        // the corners' owners, or the one sphere the packet search left
         int o[4];
-        for (int a = 0; a < 4; a++) o[a] = knn[(long long)v[a] * K];
+        const int ref = knn ? -1 : cand[t * RPD_MAXC];
+        if (knn) {
+            for (int a = 0; a < 4; a++) o[a] = knn[(long long)v[a] * K];
+        } else {
+            for (int a = 0; a < 4; a++) o[a] = ref;
+        }
         long long M[4][4];
         for (int b = 0; b < 4; b++)
             for (int a = 0; a < 4; a++) M[a][b] = pd_exact(X[a], ld_int3(Ci, o[b]), W[o[b]]);
@@ -1141,13 +1071,24 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
         for (int a = 0; a < 4; a++) thr[a] = M[a][bstar];
         if (tid == 0) sn = 0;
         __syncthreads();
+        auto test = [&](int sph) {
+            const int3 cs = ld_int3(Ci, sph);
+            const long long ws = W[sph];
+            bool in = false;
+            for (int a = 0; a < 4; a++) in |= pd_exact(X[a], cs, ws) <= thr[a];
+            if (!in) return;
+            const int pos = atomicAdd(&sn, 1);
+            if (pos < FB_GATHER) sid[pos] = sph;
+        };
+        if (!gp)
+            for (long long i = s0 + tid; i < s1; i += FB_THREADS) test((int)i);
         // A sphere with pd(X_a) <= thr_a has its centre within
         // sqrt(thr_a + wmax) of X_a, so only the cells of the box around the
         // four corners' balls can hold one; each of those cells is opened
         // when some corner a may have a sphere of it within thr_a
         // (|X_a - cell|^2 - max r^2 of the cell <= thr_a).
         int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-        for (int a = 0; a < 4; a++) {
+        for (int a = 0; a < 4 && gp; a++) {
             const long long r2 = thr[a] + g.wmax;
             const long long rad = r2 > 0 ? (long long)sqrt((double)r2) + 2 : 1;
             const long long xa[3] = {X[a].x, X[a].y, X[a].z};
@@ -1158,8 +1099,8 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
                 hi[k] = max(hi[k], (int)max(0LL, min(c1, (long long)dim[k] - 1)));
             }
         }
-        const int bx = hi[0] - lo[0] + 1, by = hi[1] - lo[1] + 1, bxy = bx * by;
-        const int nbox = bxy * (hi[2] - lo[2] + 1);
+        const int bx = gp ? hi[0] - lo[0] + 1 : 0, by = gp ? hi[1] - lo[1] + 1 : 0, bxy = bx * by;
+        const int nbox = gp ? bxy * (hi[2] - lo[2] + 1) : 0;
         for (int bi = tid; bi < nbox; bi += FB_THREADS) {
             const int bz = bi / bxy, rxy = bi - bz * bxy, byy = rxy / bx, bxx = rxy - byy * bx;
             const int qx = lo[0] + bxx, qy = lo[1] + byy, qz = lo[2] + bz;
@@ -1168,25 +1109,7 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             bool open = false;
             for (int a = 0; a < 4; a++) open |= box_dist2(X[a], g, qx, qy, qz) - cw <= thr[a];
             if (!open) continue;
-            for (long long e = start[ci]; e < start[ci + 1]; e++) {
-                const int sph = ids[e];
-                const int3 cs = ld_int3(Ci, sph);
-                const long long ws = W[sph];
-                bool in = false;
-                for (int a = 0; a < 4; a++) in |= pd_exact(X[a], cs, ws) <= thr[a];
-                if (!in) continue;
-                const int pos = atomicAdd(&sn, 1);
-                if (pos < FB_GATHER) sid[pos] = sph;
-            }
-        }
-        // and the heavy spheres, which the grid leaves out
-        for (int h = tid; h < nh; h += FB_THREADS) {
-            const int4 cs = hsph[h];
-            bool in = false;
-            for (int a = 0; a < 4; a++) in |= pd_exact(X[a], make_int3(cs.x, cs.y, cs.z), hw[h]) <= thr[a];
-            if (!in) continue;
-            const int pos = atomicAdd(&sn, 1);
-            if (pos < FB_GATHER) sid[pos] = cs.w;
+            for (long long e = start[ci]; e < start[ci + 1]; e++) test(ids[e]);
         }
         __syncthreads();
         const int n = sn;
@@ -1269,28 +1192,12 @@ size_t grid_tmp_bytes(long long ns, long long ncap) {
     return al(sizeof(int32_t) * (ncap + 1)) * 2 + al(scan_tmp_bytes(ncap));
 }
 
-int heavy_count(long long ns) { return (int)std::min<long long>(HEAVY_MAX, ns / 128); }
-
-void launch_heavy_select(const int32_t* Ci, const long long* W, long long ns, long long* wcut, int4* hsph,
-                         long long* hw, int* nheavy, cudaStream_t s) {
-    const int H = heavy_count(ns);
-    if (H < 1) {
-        const long long big = LLONG_MAX;
-        const int zero = 0;
-        cudaMemcpyAsync(wcut, &big, sizeof(big), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(nheavy, &zero, sizeof(zero), cudaMemcpyHostToDevice, s);
-        return;
-    }
-    k_heavy_select<<<1, 1024, 0, s>>>(Ci, W, ns, H, wcut, hsph, hw, nheavy);
-    note_launch();
-}
-
 void launch_sphere_grid(const int32_t* Ci, const long long* W, long long ns, long long ncap, GridParams* gp,
                         int64_t* cell_start, int32_t* cell_ids, int4* cell_sph, long long* cell_w,
-                        long long* cell_wmax, void* tmp, cudaStream_t s, const long long* wcut) {
+                        long long* cell_wmax, void* tmp, cudaStream_t s) {
     if (ncap <= GRID_SMALL_CAP) {
         k_grid_small<<<1, 1024, sizeof(int) * ncap, s>>>(Ci, W, ns, ncap, gp, cell_start, cell_ids, cell_sph, cell_w,
-                                                         cell_wmax, cell_wmax + ncap, wcut);
+                                                         cell_wmax, cell_wmax + ncap);
         note_launch();
         return;
     }
@@ -1298,15 +1205,15 @@ void launch_sphere_grid(const int32_t* Ci, const long long* W, long long ns, lon
     int32_t* count = (int32_t*)p; p += al(sizeof(int32_t) * (ncap + 1));
     int32_t* fill = (int32_t*)p; p += al(sizeof(int32_t) * (ncap + 1));
     void* stmp = p;
-    k_bbox<<<1, 1024, 0, s>>>(Ci, W, ns, ncap, gp, wcut);
+    k_bbox<<<1, 1024, 0, s>>>(Ci, W, ns, ncap, gp);
     note_launch();
     cudaMemsetAsync(count, 0, sizeof(int32_t) * ncap, s);
     cudaMemsetAsync(fill, 0, sizeof(int32_t) * ncap, s);
     cudaMemsetAsync(cell_wmax, 0, sizeof(long long) * 2 * ncap, s);
-    k_cell_count<<<nblk(ns, 256), 256, 0, s>>>(Ci, W, ns, gp, count, cell_wmax, cell_wmax + ncap, wcut);
+    k_cell_count<<<nblk(ns, 256), 256, 0, s>>>(Ci, W, ns, gp, count, cell_wmax, cell_wmax + ncap);
     note_launch();
     scan_excl(count, cell_start, ncap, stmp, s);
-    k_cell_fill<<<nblk(ns, 256), 256, 0, s>>>(Ci, W, ns, gp, cell_start, fill, cell_ids, cell_sph, cell_w, wcut);
+    k_cell_fill<<<nblk(ns, 256), 256, 0, s>>>(Ci, W, ns, gp, cell_start, fill, cell_ids, cell_sph, cell_w);
     note_launch();
 }
 
@@ -1329,7 +1236,7 @@ void launch_sphere_grid_batch(const int32_t* Ci, const long long* W, const long 
 void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams* gp, const int64_t* cell_start,
                 const int4* cell_sph, const long long* cell_w, const long long* cell_wmax, long long ncap, int K,
                 int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s,
-                const long long* voff, int nshapes, const int4* hsph, const long long* hw, const int* nheavy) {
+                const long long* voff, int nshapes) {
     if (nv == 0) return;
     char* p = (char*)tmp;
     uint64_t* k0 = (uint64_t*)p; p += al(sizeof(uint64_t) * nv);
@@ -1340,14 +1247,8 @@ void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams*
     while ((1ll << bits) < ncap) bits++;
     if ((ns <= (1 << 17) || nshapes > 1) && !two_word) {   // batches: shape-local ids in the key
         // one vertex per warp in input order: the sphere grid stays in cache
-        if (nheavy)
-            k_knn_warp<true><<<nblk(32 * nv, 256), 256, 0, s>>>(Xi, nullptr, nv, gp, cell_start, cell_sph, cell_w,
-                                                                 cell_wmax + ncap, K, knn, dplus, voff, nshapes, hsph,
-                                                                 hw, nheavy);
-        else
-            k_knn_warp<false><<<nblk(32 * nv, 256), 256, 0, s>>>(Xi, nullptr, nv, gp, cell_start, cell_sph, cell_w,
-                                                                  cell_wmax + ncap, K, knn, dplus, voff, nshapes,
-                                                                  nullptr, nullptr, nullptr);
+        k_knn_warp<<<nblk(32 * nv, 256), 256, 0, s>>>(Xi, nullptr, nv, gp, cell_start, cell_sph, cell_w,
+                                                       cell_wmax + ncap, K, knn, dplus, voff, nshapes);
     } else {
         k_vertex_cells<<<nblk(nv, 256), 256, 0, s>>>(Xi, nv, gp, k0, v0);
         note_launch();
@@ -1362,16 +1263,25 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                        const long long* W, const int32_t* knn, const long long* dplus, int K, const GridParams* gp,
                        const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
                        int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord, int32_t* fb_list, int32_t* fb_count,
-                       DevState* st, cudaStream_t s, const long long* voff, int nshapes, const int4* hsph,
-                       const long long* hw, const int* nheavy) {
+                       DevState* st, cudaStream_t s, const long long* voff, int nshapes) {
     if (nt == 0) return;
     cudaMemsetAsync(fb_count, 0, sizeof(int32_t), s);
     k_candidates_warp<<<nblk(32 * nt, 256), 256, 0, s>>>(d_tets, nt, nv, Xi, Ci, W, knn, dplus, K, cand_cnt, cand,
                                                           cand_ord,
                                                fb_list, fb_count, st);
     note_launch();
-    k_candidates_fallback<<<152 * 4, FB_THREADS, 0, s>>>(d_tets, nv, Xi, Ci, W, knn, K, gp, cell_start, cell_ids,
+    launch_candidates_fallback(d_tets, nv, Xi, Ci, W, 0, knn, K, gp, cell_start, cell_ids, cell_wmax, fb_list,
+                               fb_count, cand_cnt, cand, cand_ord, st, voff, nullptr, nshapes, s);
+}
+
+void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
+                                const long long* W, long long ns, const int32_t* knn, int K, const GridParams* gp,
+                                const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
+                                const int32_t* fb_list, const int32_t* fb_count, int32_t* cand_cnt, int32_t* cand,
+                                uint8_t* cand_ord, DevState* st, const long long* voff, const long long* soff,
+                                int nshapes, cudaStream_t s) {
+    k_candidates_fallback<<<152 * 4, FB_THREADS, 0, s>>>(T, nv, Xi, Ci, W, ns, knn, K, gp, cell_start, cell_ids,
                                                          cell_wmax, fb_list, fb_count, cand_cnt, cand, cand_ord, st,
-                                                         voff, nshapes, hsph, hw, nheavy);
+                                                         voff, soff, nshapes);
     note_launch();
 }
