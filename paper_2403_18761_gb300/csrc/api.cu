@@ -64,6 +64,75 @@ void release_events(int dev, cudaEvent_t* ev, int n) {
         if (ev[k]) P.free_ev[dev].push_back(ev[k]);
 }
 
+// What the host reads at a build's two synchronisations, written by one kernel
+// straight into pinned host memory (a copy from each of the arrays that hold
+// these cost some 8 us apiece, eight of them per build).
+struct HostReport {
+    DevState st;
+    long long npairs, npieces, nseg[4];
+    unsigned long long nchanged, rcount[3], qcount[RPD_NBINS];
+    int32_t bins[RPD_NBINS];
+};
+// Recycled blocks: a context holds one while it builds, so there are as many
+// as builds were ever under way at once.  Portable: usable on every device.
+struct ReportPool {
+    std::mutex mu;
+    std::vector<HostReport*> free_blocks;
+};
+ReportPool& report_pool() {
+    static ReportPool p;
+    return p;
+}
+struct ReportBlock {
+    HostReport* h = nullptr;
+    ReportBlock() {
+        ReportPool& P = report_pool();
+        {
+            std::lock_guard<std::mutex> lock(P.mu);
+            if (!P.free_blocks.empty()) {
+                h = P.free_blocks.back();
+                P.free_blocks.pop_back();
+            }
+        }
+        if (!h && cudaHostAlloc((void**)&h, sizeof(HostReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            h = nullptr;
+        }
+    }
+    ~ReportBlock() {
+        if (!h) return;
+        ReportPool& P = report_pool();
+        std::lock_guard<std::mutex> lock(P.mu);
+        P.free_blocks.push_back(h);
+    }
+    ReportBlock(const ReportBlock&) = delete;
+    ReportBlock& operator=(const ReportBlock&) = delete;
+};
+
+// Null sources are skipped.
+struct ReportArgs {
+    const DevState* st;
+    const int64_t *npairs, *npieces;
+    const long long* nseg;
+    const unsigned long long *nchanged, *rcount, *qcount;
+    const int32_t* bins;
+    HostReport* out;
+};
+__global__ void k_report(ReportArgs a) {
+    const int t = threadIdx.x;
+    if (t == 0) {
+        a.out->st.err = a.st->err;
+        if (a.npairs) a.out->npairs = *a.npairs;
+        if (a.npieces) a.out->npieces = *a.npieces;
+        if (a.nchanged) a.out->nchanged = *a.nchanged;
+    }
+    if (t < CNT_NUM) a.out->st.cnt[t] = a.st->cnt[t];
+    if (t < 4 && a.nseg) a.out->nseg[t] = a.nseg[t];
+    if (t < 3 && a.rcount) a.out->rcount[t] = a.rcount[t];
+    if (t < RPD_NBINS && a.qcount) a.out->qcount[t] = a.qcount[t];
+    if (t < RPD_NBINS && a.bins) a.out->bins[t] = a.bins[t];
+}
+
 }  // namespace
 
 // One stream-ordered memory pool per device, owned by the library, that keeps
@@ -244,13 +313,7 @@ const char* dev_reason(int code, const unsigned long long* cnt) {
 // Synchronise the stream and read the device status: counters into the
 // stats, and an error raised on the device as the return value (with
 // raise == false the error code is only left in *code).
-rpd_status check_device(rpd_ctx* c, bool raise = true, int* code = nullptr) {
-    DevState h;
-    if (cudaMemcpyAsync(&h, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
-        cudaStreamSynchronize(c->stream) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(c, RPD_E_CUDA, "CUDA error while reading the device status");
-    }
+rpd_status take_status(rpd_ctx* c, const DevState& h, bool raise, int* code) {
     c->stats.pred_fast = (int64_t)h.cnt[CNT_PRED_FAST];
     c->stats.pred_fp64 = (int64_t)h.cnt[CNT_PRED_FP64];
     c->stats.pred_exact = (int64_t)h.cnt[CNT_PRED_EXACT];
@@ -260,6 +323,29 @@ rpd_status check_device(rpd_ctx* c, bool raise = true, int* code = nullptr) {
     if (code) *code = h.err;
     if (raise && h.err != 0) return fail(c, (rpd_status)h.err, dev_reason(h.err, h.cnt));
     return RPD_OK;
+}
+
+rpd_status check_device(rpd_ctx* c) {
+    DevState h;
+    if (cudaMemcpyAsync(&h, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+        cudaStreamSynchronize(c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, RPD_E_CUDA, "CUDA error while reading the device status");
+    }
+    return take_status(c, h, true, nullptr);
+}
+
+// The same through a report block, which also gets the other values of `a`.
+rpd_status report_device(rpd_ctx* c, ReportArgs a, HostReport* h, bool raise = true, int* code = nullptr) {
+    a.st = c->st;
+    a.out = h;
+    k_report<<<1, 64, 0, c->stream>>>(a);
+    note_launch();
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, RPD_E_CUDA, "CUDA error while reading the device status");
+    }
+    return take_status(c, h->st, raise, code);
 }
 
 rpd_status cuda_check(rpd_ctx* c, const char* where) {
@@ -294,7 +380,7 @@ struct BinStreams {
     bool ready = false;
     cudaStream_t s[RPD_NBINS];
     cudaStream_t util;     // high priority: clearing scratch next to the clip
-    cudaStream_t fin[4];   // high priority: the element kinds, ahead of the volume pass
+    cudaStream_t fin;      // high priority: the element kinds, ahead of the volume pass
 };
 
 BinStreams* bin_streams() {
@@ -310,8 +396,7 @@ BinStreams* bin_streams() {
         int lo = 0, hi = 0;
         cudaDeviceGetStreamPriorityRange(&lo, &hi);
         if (cudaStreamCreateWithPriority(&b.util, cudaStreamNonBlocking, hi) != cudaSuccess) return nullptr;
-        for (int k = 0; k < 4; k++)
-            if (cudaStreamCreateWithPriority(&b.fin[k], cudaStreamNonBlocking, hi) != cudaSuccess) return nullptr;
+        if (cudaStreamCreateWithPriority(&b.fin, cudaStreamNonBlocking, hi) != cudaSuccess) return nullptr;
         b.ready = true;
     }
     return &b;
@@ -617,17 +702,22 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     launch_bin_pairs(c->cand_cnt, c->pair_off, nt, c->pair_tet, c->bins, c->bin_count, c->bin_fill, pcap, c->rcount,
                      c->qcount, s, c->changed);
     cudaStreamWaitEvent(s, c->ev[2], 0);   // mesh combinatorics done
-    long long npairs = 0;
-    int32_t hb[RPD_NBINS];
-    unsigned long long nchanged = (unsigned long long)nt;
-    cudaMemcpyAsync(&npairs, c->pair_off + nt, sizeof(long long), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(hb, c->bin_count, sizeof(hb), cudaMemcpyDeviceToHost, s);
-    if (old) cudaMemcpyAsync(&nchanged, c->d_nchanged, sizeof(nchanged), cudaMemcpyDeviceToHost, s);
-    TRY(check_device(c));   // synchronises: validation errors stop the build here
+    ReportBlock report;
+    NEED(report.h);
+    HostReport* const hr = report.h;
+    hr->nchanged = (unsigned long long)nt;
+    {
+        ReportArgs r{};
+        r.npairs = c->pair_off + nt;
+        r.bins = c->bin_count;
+        r.nchanged = old ? c->d_nchanged : nullptr;
+        TRY(report_device(c, r, hr));   // synchronises: validation errors stop the build here
+    }
+    const long long npairs = hr->npairs;
     c->npairs = npairs;
     c->stats.n_pairs = npairs;
-    c->stats.update_tets = (int64_t)nchanged;
-    for (int b = 0; b < RPD_NBINS; b++) c->stats.bin_pairs[b] = c->hbin[b] = hb[b];
+    c->stats.update_tets = (int64_t)hr->nchanged;
+    for (int b = 0; b < RPD_NBINS; b++) c->stats.bin_pairs[b] = c->hbin[b] = hr->bins[b];
     // ---- A3-A4
     {   // one chunk for the pair, queue, record and finalisation buffers
         size_t est = (size_t)npairs * 760 + ((size_t)ns * 64 + (4 << 20));
@@ -716,7 +806,6 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
         ktmp2 = c->alloc<char>(keep_tmp_bytes(npairs, old->nrec[2]));
         NEED(ktmp2);
     }
-    long long h[5];
     for (int attempt = 0; attempt < 2; attempt++) {
         for (int k = 0; k < 3; k++) {
             a.rcap[k] = cap[k];
@@ -750,30 +839,31 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
         record(c, 5);   // clip and record kernels done, scratch clear: the four kinds fork here
         // ---- A5-A7, the four kinds side by side on high-priority streams; the
         // record counts stay on the device (grids sized by the capacities)
-        for (int kind = 1; kind <= 4; kind++) {
-            cudaStream_t sk = bs->fin[kind - 1];
-            cudaStreamWaitEvent(sk, c->ev[5], 0);
-            if (c->kind_ok[kind - 1]) {
-                launch_finalize(c->clip, kind, fcap[kind - 1], fcap[kind - 1], c->ns, c->key_bits,
-                                c->fout[kind - 1], ftmp[kind - 1], sk);
-            } else {
-                cudaMemsetAsync(d_nseg + kind - 1, 0, sizeof(long long), sk);
+        cudaStreamWaitEvent(bs->fin, c->ev[5], 0);
+        {
+            FinalJob jobs[4];
+            int nj = 0;
+            for (int kind = 1; kind <= 4; kind++) {
+                if (c->kind_ok[kind - 1]) jobs[nj++] = {kind, fcap[kind - 1], c->fout[kind - 1], ftmp[kind - 1]};
+                else cudaMemsetAsync(d_nseg + kind - 1, 0, sizeof(long long), bs->fin);
             }
-            cudaEventRecord(c->ev[6 + kind - 1], sk);
+            launch_finalize(c->clip, jobs, nj, c->ns, c->key_bits, bs->fin);
         }
+        cudaEventRecord(c->ev[6], bs->fin);
         scan_excl(a.pflag, c->piece_off, npairs, ptmp, s);
         TRY(cuda_check(c, "finalize launch"));
-        for (int kind = 1; kind <= 4; kind++) cudaStreamWaitEvent(s, c->ev[6 + kind - 1], 0);
+        cudaStreamWaitEvent(s, c->ev[6], 0);
         for (int b = 0; b < RPD_NBINS; b++)   // volume passes
             if (c->hbin[b]) cudaStreamWaitEvent(s, c->evc[1 + RPD_NBINS + b], 0);
-        unsigned long long cnt[3], qc[RPD_NBINS];
-        cudaMemcpyAsync(cnt, c->rcount, sizeof(cnt), cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(qc, c->qcount, sizeof(qc), cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(h, d_nseg, sizeof(long long) * 4, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(h + 4, c->piece_off + npairs, sizeof(long long), cudaMemcpyDeviceToHost, s);
         int dev_err = 0;
-        TRY(check_device(c, false, &dev_err));
-        for (int b = 0; b < RPD_NBINS; b++) c->stats.bin_cut[b] = (int64_t)qc[b];
+        ReportArgs r{};
+        r.rcount = c->rcount;
+        r.qcount = c->qcount;
+        r.nseg = d_nseg;
+        r.npieces = c->piece_off + npairs;
+        TRY(report_device(c, r, hr, false, &dev_err));
+        const unsigned long long* cnt = hr->rcount;
+        for (int b = 0; b < RPD_NBINS; b++) c->stats.bin_cut[b] = (int64_t)hr->qcount[b];
         bool fits = true;
         for (int k = 0; k < 3; k++) {
             c->nrec[k] = (long long)cnt[k];
@@ -796,12 +886,12 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     }
     for (int k = 0; k < 3; k++) c->stats.n_records[k + 1] = c->nrec[k];
     for (int k = 0; k < 4; k++) {
-        c->nkeys[k] = h[k];
-        c->stats.n_keys[k] = h[k];
+        c->nkeys[k] = hr->nseg[k];
+        c->stats.n_keys[k] = hr->nseg[k];
     }
-    c->npieces = h[4];
-    c->stats.n_pieces = h[4];
-    c->stats.n_records[0] = h[4];
+    c->npieces = hr->npieces;
+    c->stats.n_pieces = hr->npieces;
+    c->stats.n_records[0] = hr->npieces;
     for (int k = 0; k < 4; k++) {
         c->ftmp[k] = ftmp[k];
         c->fcap[k] = fcap[k];
@@ -828,7 +918,7 @@ void stage_times(rpd_ctx* c) {
         c->stats.ms_clip_kernels = std::max(c->stats.ms_clip_kernels, k);
         c->stats.ms_clip_span = std::max(c->stats.ms_clip_span, w);
     }
-    for (int k = 0; k < 4; k++) c->stats.ms_finalize[k] = elapsed(c, 5, 6 + k);   // the kinds run side by side
+    for (int k = 0; k < 4; k++) c->stats.ms_finalize[k] = elapsed(c, 5, 6);   // the kinds share their launches
     c->timed = true;
 }
 

@@ -320,8 +320,15 @@ struct ClearList {
 };
 void finalize_clear_list(int kind, long long ncap, long long ns, void* tmp, ClearList& L);
 void launch_clear(const ClearList& L, cudaStream_t s);
-void launch_finalize(const ClipArgs& a, int kind, long long n, long long ncap, long long ns, int key_bits,
-                     const FinalOut& out, void* tmp, cudaStream_t s);
+// One kind's finalisation: kind 1: n = the number of pairs; kinds 2..4: n =
+// the record capacity (the record count is read on the device, a.rcount).
+struct FinalJob {
+    int kind;
+    long long n;
+    FinalOut out;
+    void* tmp;
+};
+void launch_finalize(const ClipArgs& a, const FinalJob* jobs, int njob, long long ns, int key_bits, cudaStream_t s);
 // One launch copying n_keys int32 key entries and n values of elem (1 or 4)
 // bytes; a NULL source skips that part.
 void launch_copy_rows(const int32_t* keys, int32_t* d_keys, long long n_keys, const void* vals, void* d_vals,

@@ -249,7 +249,8 @@ extern "C" rpd_status rpd_euler_static(const double* d_verts, int64_t nv, const 
     void* ftmp = ar.take<char>(finalize_tmp_bytes(kind, n, ns));
     NEED_S(!ar.full);
     launch_finalize_clear(kind, n, ns, ftmp, s);
-    launch_finalize(a, kind, n, n, ns, b, fo, ftmp, s);
+    const FinalJob job{kind, n, fo, ftmp};
+    launch_finalize(a, &job, 1, ns, b, s);
     long long m = 0;
     cudaMemcpyAsync(&m, fo.count, sizeof(long long), cudaMemcpyDeviceToHost, s);
     TRY_S(read_status(st, s));

@@ -78,7 +78,7 @@ __device__ __forceinline__ int find_slot(const ClipArgs& A, long long t, int sph
     return found;
 }
 
-__global__ void k_link_cells(ClipArgs A, long long npairs, int32_t* __restrict__ parent) {
+__device__ __forceinline__ void link_cells(const ClipArgs& A, long long npairs, int32_t* __restrict__ parent) {
     long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= npairs || A.pflag[p] != 1) return;
     unsigned lk = A.c_link[p];
@@ -105,7 +105,7 @@ __device__ __forceinline__ long long rec_count(const ClipArgs& A, int which, lon
     return n < nmax ? n : nmax;
 }
 
-__global__ void k_link_records(ClipArgs A, int which, long long nmax, int32_t* __restrict__ parent) {
+__device__ __forceinline__ void link_records(const ClipArgs& A, int which, long long nmax, int32_t* __restrict__ parent) {
     long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nrec = rec_count(A, which, nmax);   // records past it were never written
     if (r >= nrec) return;
@@ -144,8 +144,9 @@ __global__ void k_link_records(ClipArgs A, int which, long long nmax, int32_t* _
 
 // ------------------------------------------------------ aggregation (A5-A7)
 // Cells: chi and root counts summed straight into per-sphere slots.
-__global__ void k_cell_agg(ClipArgs A, long long npairs, int32_t* __restrict__ parent, int32_t* __restrict__ cchi,
-                           int32_t* __restrict__ cbeta, uint8_t* __restrict__ cpres) {
+__device__ __forceinline__ void cell_agg(const ClipArgs& A, long long npairs, int32_t* __restrict__ parent,
+                                         int32_t* __restrict__ cchi, int32_t* __restrict__ cbeta,
+                                         uint8_t* __restrict__ cpres) {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = p < npairs && A.pflag[p] == 1;
     int i = -1, c = 0, r = 0;
@@ -172,7 +173,7 @@ __global__ void k_cell_agg(ClipArgs A, long long npairs, int32_t* __restrict__ p
     cpres[i] = 1;
 }
 
-__global__ void k_cell_emit(long long ns, const uint8_t* __restrict__ cpres, const int64_t* __restrict__ pos,
+__device__ __forceinline__ void cell_emit(long long ns, const uint8_t* __restrict__ cpres, const int64_t* __restrict__ pos,
                             const int32_t* __restrict__ cchi, const int32_t* __restrict__ cbeta,
                             int32_t* __restrict__ keys, int32_t* __restrict__ chi, int32_t* __restrict__ beta,
                             uint8_t* __restrict__ flag, long long* __restrict__ count) {
@@ -189,7 +190,7 @@ __global__ void k_cell_emit(long long ns, const uint8_t* __restrict__ cpres, con
 
 // Faces, edges, vertices: records hashed by key; chi and root counts summed
 // into the key's slot.
-__global__ void k_rec_agg(ClipArgs A, int which, long long nmax, int32_t* __restrict__ parent, uint64_t* __restrict__ tk,
+__device__ __forceinline__ void rec_agg(const ClipArgs& A, int which, long long nmax, int32_t* __restrict__ parent, uint64_t* __restrict__ tk,
                           int32_t* __restrict__ tchi, int32_t* __restrict__ tbeta, unsigned long long mask,
                           int shift) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -207,7 +208,7 @@ __global__ void k_rec_agg(ClipArgs A, int which, long long nmax, int32_t* __rest
 
 // Occupied slots appended (warp-aggregated) to (key, slot) lists; each key
 // counted in the bucket of its first sphere.
-__global__ void k_table_compact(const uint64_t* __restrict__ tk, long long cap, int shift, uint64_t* __restrict__ ck,
+__device__ __forceinline__ void table_compact(const uint64_t* __restrict__ tk, long long cap, int shift, uint64_t* __restrict__ ck,
                                 uint32_t* __restrict__ cs, unsigned long long* __restrict__ count,
                                 int32_t* __restrict__ bcount) {
     const long long h = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -228,7 +229,7 @@ __global__ void k_table_compact(const uint64_t* __restrict__ tk, long long cap, 
 }
 
 // (key, slot) into the bucket of the key's first sphere (any order inside).
-__global__ void k_bucket_fill(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cs,
+__device__ __forceinline__ void bucket_fill(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ cs,
                               const unsigned long long* __restrict__ count, long long nmax, int shift,
                               const int64_t* __restrict__ bstart, int32_t* __restrict__ bfill,
                               uint64_t* __restrict__ bk, uint32_t* __restrict__ bs) {
@@ -242,7 +243,7 @@ __global__ void k_bucket_fill(const uint64_t* __restrict__ ck, const uint32_t* _
 }
 
 // Rank inside the bucket, then the output row: sorted key, chi, beta0, flag.
-__global__ void k_bucket_emit(const uint64_t* __restrict__ bk, const uint32_t* __restrict__ bs,
+__device__ __forceinline__ void bucket_emit(const uint64_t* __restrict__ bk, const uint32_t* __restrict__ bs,
                               const unsigned long long* __restrict__ count, long long nmax, int kind, int b,
                               const int64_t* __restrict__ bstart, const int32_t* __restrict__ tchi,
                               const int32_t* __restrict__ tbeta, int32_t* __restrict__ keys,
@@ -261,6 +262,102 @@ __global__ void k_bucket_emit(const uint64_t* __restrict__ bk, const uint32_t* _
     chi[q] = c;
     beta[q] = bb;
     flag[q] = (bb == 1 && c == 1) ? 1 : 0;
+}
+
+// ------------------------------------------------- the kinds side by side
+// One launch per step for all the kinds asked for, blockIdx.y the kind's job:
+// a step is short (3 to 100 us), so a launch per step and kind on a stream of
+// its own cost a small build more on the host than the kernels took.
+struct FinKind {
+    int kind;
+    long long n;                 // pieces (kind 1) or record capacity
+    int32_t* parent;
+    uint64_t* tk;                // hash table of 2^(64 - tshift) slots
+    int32_t *tchi, *tbeta;
+    int tshift, shift;           // hash shift; shift of a key's first sphere
+    long long cap;
+    unsigned long long* cnt;
+    int32_t *bcount, *bfill;
+    int64_t* bstart;
+    int32_t *cchi, *cbeta;
+    uint8_t* cpres;
+    uint64_t *ck, *bk;
+    uint32_t *cs, *bs;
+    FinalOut out;
+};
+struct FinArgs {
+    ClipArgs a;
+    int key_bits, njob;
+    long long ns;
+    FinKind k[4];
+};
+
+__global__ void k_fin_link(FinArgs F) {
+    const FinKind& k = F.k[blockIdx.y];
+    if (k.kind == 1) link_cells(F.a, k.n, k.parent);
+    else if (k.kind < 4) link_records(F.a, k.kind - 2, k.n, k.parent);   // vertices are points
+}
+__global__ void k_fin_agg(FinArgs F) {
+    const FinKind& k = F.k[blockIdx.y];
+    if ((long long)blockIdx.x * blockDim.x >= k.n) return;   // uniform over the block
+    if (k.kind == 1) cell_agg(F.a, k.n, k.parent, k.cchi, k.cbeta, k.cpres);
+    else rec_agg(F.a, k.kind - 2, k.n, k.kind < 4 ? k.parent : nullptr, k.tk, k.tchi, k.tbeta,
+                 (unsigned long long)(k.cap - 1), k.tshift);
+}
+__global__ void k_fin_compact(FinArgs F) {
+    const FinKind& k = F.k[blockIdx.y];
+    if (k.kind == 1 || (long long)blockIdx.x * blockDim.x >= k.cap) return;   // uniform over the block
+    table_compact(k.tk, k.cap, k.shift, k.ck, k.cs, k.cnt, k.bcount);
+}
+// First row of every sphere's keys: an exclusive scan of the counts, one block
+// per kind (up to SCAN_ONE spheres; above that the library's scan).
+constexpr long long SCAN_ONE = 32768;
+__global__ void __launch_bounds__(1024) k_fin_scan(FinArgs F) {
+    __shared__ int wsum[32];
+    const FinKind& k = F.k[blockIdx.y];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int per = (int)((F.ns + 1023) / 1024);
+    const long long lo = min((long long)threadIdx.x * per, F.ns), hi = min(lo + per, F.ns);
+    int sum = 0;
+    for (long long i = lo; i < hi; i++) sum += k.kind == 1 ? (int)k.cpres[i] : k.bcount[i];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        int t = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        wsum[lane] = t;
+    }
+    __syncthreads();
+    long long run = incl - sum + (w > 0 ? wsum[w - 1] : 0);
+    for (long long i = lo; i < hi; i++) {
+        k.bstart[i] = run;
+        run += k.kind == 1 ? (int)k.cpres[i] : k.bcount[i];
+    }
+    if (threadIdx.x == 0) k.bstart[F.ns] = wsum[31];
+}
+__global__ void k_fin_fill(FinArgs F) {
+    const FinKind& k = F.k[blockIdx.y];
+    if (k.kind == 1)
+        cell_emit(F.ns, k.cpres, k.bstart, k.cchi, k.cbeta, k.out.keys, k.out.chi, k.out.beta, k.out.flag, k.out.count);
+    else
+        bucket_fill(k.ck, k.cs, k.cnt, k.n, k.shift, k.bstart, k.bfill, k.bk, k.bs);
+}
+__global__ void k_fin_emit(FinArgs F) {
+    const FinKind& k = F.k[blockIdx.y];
+    if (k.kind == 1) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *k.out.count = (long long)*k.cnt;
+    bucket_emit(k.bk, k.bs, k.cnt, k.n, k.kind, F.key_bits, k.bstart, k.tchi, k.tbeta, k.out.keys, k.out.chi,
+                k.out.beta, k.out.flag);
 }
 
 __global__ void k_copy_rows(const int32_t* __restrict__ keys, int32_t* __restrict__ d_keys, long long nk,
@@ -410,65 +507,81 @@ void launch_finalize_clear(int kind, long long ncap, long long ns, void* tmp, cu
     launch_clear(C, s);
 }
 
-void launch_finalize(const ClipArgs& a, int kind, long long n, long long ncap, long long ns, int key_bits,
-                     const FinalOut& out, void* tmp, cudaStream_t s) {
-    // kind 1: n = the number of pairs; kinds 2..4: n = the record capacity,
-    // the record count itself is read on the device (a.rcount)
-    const Layout L = layout(kind, ncap, ns);
-    char* base = (char*)tmp;
-    int32_t* parent = (int32_t*)base;
-    int32_t* bcount = (int32_t*)(base + L.o_bcount);
-    int32_t* bfill = (int32_t*)(base + L.o_bfill);
-    int64_t* bstart = (int64_t*)(base + L.o_bstart);
-    void* stmp = base + L.o_scan;
-    if (kind == 1) {
-        int32_t* cchi = (int32_t*)(base + L.o_cchi);
-        int32_t* cbeta = cchi + ns;
-        uint8_t* cpres = (uint8_t*)(base + L.o_cpres);
-        if (n > 0) {
-            k_link_cells<<<nblk(n, 256), 256, 0, s>>>(a, n, parent);
-            note_launch();
-            k_cell_agg<<<nblk(n, 256), 256, 0, s>>>(a, n, parent, cchi, cbeta, cpres);
-            note_launch();
+void launch_finalize(const ClipArgs& a, const FinalJob* jobs, int njob, long long ns, int key_bits, cudaStream_t s) {
+    if (njob <= 0) return;
+    FinArgs F;
+    F.a = a;
+    F.key_bits = key_bits;
+    F.njob = njob;
+    F.ns = ns;
+    void* scan_tmp[4];
+    // grid sizes: pieces or records that are linked, all that are aggregated,
+    // table slots, and keys or spheres (at most records, spheres)
+    long long n_link = 0, n_agg = 0, n_cap = 0, n_key = 0, n_fill = 0;
+    for (int j = 0; j < njob; j++) {
+        const FinalJob& q = jobs[j];
+        const Layout L = layout(q.kind, q.n, ns);
+        char* base = (char*)q.tmp;
+        FinKind& k = F.k[j];
+        k.kind = q.kind;
+        k.n = q.n;
+        k.parent = (int32_t*)base;
+        const int tb = q.kind == 1 ? 0 : table_bits(q.n);
+        k.cap = 1ll << tb;
+        k.tshift = 64 - tb;
+        k.shift = (q.kind - 1) * key_bits;   // first sphere of a key
+        k.tk = (uint64_t*)(base + L.o_tk);
+        k.tchi = (int32_t*)(base + L.o_tchi);
+        k.tbeta = k.tchi + k.cap;
+        k.cnt = (unsigned long long*)(base + L.o_cnt);
+        k.bcount = (int32_t*)(base + L.o_bcount);
+        k.bfill = (int32_t*)(base + L.o_bfill);
+        k.bstart = (int64_t*)(base + L.o_bstart);
+        k.cchi = (int32_t*)(base + L.o_cchi);
+        k.cbeta = k.cchi + ns;
+        k.cpres = (uint8_t*)(base + L.o_cpres);
+        k.ck = (uint64_t*)(base + L.o_ck);
+        k.cs = (uint32_t*)(base + L.o_cs);
+        k.bk = (uint64_t*)(base + L.o_bk);
+        k.bs = (uint32_t*)(base + L.o_bs);
+        k.out = q.out;
+        scan_tmp[j] = base + L.o_scan;
+        if (q.kind < 4) n_link = std::max(n_link, q.n);
+        n_agg = std::max(n_agg, q.n);
+        if (q.kind > 1) {
+            n_cap = std::max(n_cap, k.cap);
+            n_key = std::max(n_key, q.n);
         }
-        scan_excl(cpres, bstart, ns, stmp, s);
-        k_cell_emit<<<nblk(ns, 256), 256, 0, s>>>(ns, cpres, bstart, cchi, cbeta, out.keys, out.chi, out.beta,
-                                                  out.flag, out.count);
-        note_launch();
-        return;
+        n_fill = std::max(n_fill, q.kind == 1 ? ns : q.n);
     }
-    const int which = kind - 2;
-    const int tb = table_bits(ncap);
-    const long long cap = 1ll << tb;
-    uint64_t* tk = (uint64_t*)(base + L.o_tk);
-    int32_t* tchi = (int32_t*)(base + L.o_tchi);
-    int32_t* tbeta = tchi + cap;
-    unsigned long long* cnt = (unsigned long long*)(base + L.o_cnt);
-    uint64_t* ck = (uint64_t*)(base + L.o_ck);
-    uint32_t* cs = (uint32_t*)(base + L.o_cs);
-    uint64_t* bk = (uint64_t*)(base + L.o_bk);
-    uint32_t* bs = (uint32_t*)(base + L.o_bs);
-    const int shift = (kind - 1) * key_bits;   // first sphere of a key
-    if (n > 0) {
-        if (which < 2) {   // faces and edges have components across tets; vertices are points
-            k_link_records<<<nblk(n, 256), 256, 0, s>>>(a, which, n, parent);
-            note_launch();
+    auto grid = [&](long long n) { return dim3(std::max(nblk(n, 256), 1u), (unsigned)njob); };
+    if (n_link > 0) {
+        k_fin_link<<<grid(n_link), 256, 0, s>>>(F);
+        note_launch();
+    }
+    if (n_agg > 0) {
+        k_fin_agg<<<grid(n_agg), 256, 0, s>>>(F);
+        note_launch();
+    }
+    if (n_cap > 0) {
+        k_fin_compact<<<grid(n_cap), 256, 0, s>>>(F);
+        note_launch();
+    }
+    if (ns <= SCAN_ONE) {
+        k_fin_scan<<<dim3(1, (unsigned)njob), 1024, 0, s>>>(F);
+        note_launch();
+    } else {
+        for (int j = 0; j < njob; j++) {
+            if (F.k[j].kind == 1) scan_excl(F.k[j].cpres, F.k[j].bstart, ns, scan_tmp[j], s);
+            else scan_excl(F.k[j].bcount, F.k[j].bstart, ns, scan_tmp[j], s);
         }
-        k_rec_agg<<<nblk(n, 256), 256, 0, s>>>(a, which, n, which < 2 ? parent : nullptr, tk, tchi, tbeta,
-                                               (unsigned long long)(cap - 1), 64 - tb);
-        note_launch();
     }
-    k_table_compact<<<nblk(cap, 256), 256, 0, s>>>(tk, cap, shift, ck, cs, cnt, bcount);
+    k_fin_fill<<<grid(n_fill), 256, 0, s>>>(F);
     note_launch();
-    scan_excl(bcount, bstart, ns, stmp, s);
-    if (n > 0) {
-        k_bucket_fill<<<nblk(n, 256), 256, 0, s>>>(ck, cs, cnt, n, shift, bstart, bfill, bk, bs);
-        note_launch();
-        k_bucket_emit<<<nblk(n, 256), 256, 0, s>>>(bk, bs, cnt, n, kind, key_bits, bstart, tchi, tbeta, out.keys,
-                                                   out.chi, out.beta, out.flag);
+    if (n_cap > 0) {
+        k_fin_emit<<<grid(n_key), 256, 0, s>>>(F);
         note_launch();
     }
-    cudaMemcpyAsync(out.count, cnt, sizeof(long long), cudaMemcpyDeviceToDevice, s);
 }
 
 void launch_copy_rows(const int32_t* keys, int32_t* d_keys, long long n_keys, const void* vals, void* d_vals,
