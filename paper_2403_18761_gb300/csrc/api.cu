@@ -186,7 +186,7 @@ struct rpd_ctx {
     int32_t *cand_cnt = nullptr, *cand = nullptr, *fb_list = nullptr, *fb_count = nullptr;
     uint8_t* cand_ord = nullptr;
     int64_t* pair_off = nullptr;
-    int32_t *pair_tet = nullptr, *bins = nullptr, *bin_count = nullptr, *bin_fill = nullptr;
+    int32_t *pair_tet = nullptr, *bins = nullptr, *bin_count = nullptr;
     long long hbin[RPD_NBINS] = {};
     int32_t* qpair[RPD_NBINS] = {};
     uint8_t* qnv[RPD_NBINS] = {};
@@ -648,10 +648,12 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     c->fb_count = c->alloc<int32_t>(1);
     c->pair_off = c->alloc<int64_t>(nt + 1);
     void* stmp = c->alloc<char>(scan_tmp_bytes(nt + 1));
-    c->bin_count = c->alloc<int32_t>(RPD_NBINS);
-    c->bin_fill = c->alloc<int32_t>(RPD_NBINS);
-    NEED(c->cand_cnt && c->cand && c->cand_ord && c->fb_list && c->fb_count && c->pair_off && stmp && c->bin_count &&
-         c->bin_fill);
+    BinCounters bc;
+    bc.set(c->alloc<char>(BinCounters::BYTES));
+    NEED(c->cand_cnt && c->cand && c->cand_ord && c->fb_list && c->fb_count && c->pair_off && stmp && bc.mem);
+    c->bin_count = bc.count;
+    c->rcount = bc.rcount;
+    c->qcount = bc.qcount;
     if (lists) {
         launch_candidates(c->tets, nt, nv, c->Xi, c->Ci, c->W, knn, dplus, c->K, c->gp, c->cell_start, c->cell_ids,
                           c->cell_wmax, c->cand_cnt, c->cand, c->cand_ord, c->fb_list, c->fb_count, c->st, s,
@@ -684,7 +686,7 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
         launch_cand_diff(c->cand_cnt, c->cand, c->cand_ord, old->cand_cnt, old->cand, old->cand_ord, nt, c->changed,
                          c->d_nchanged, s);
     }
-    launch_bin_count(c->cand_cnt, nt, c->bin_count, s, c->changed);
+    launch_bin_count(c->cand_cnt, nt, bc, s, c->changed);
     TRY(cuda_check(c, "candidate launch"));
     record(c, 4);
     // the pairs are put in bin order before the pair count is read, with room
@@ -696,11 +698,8 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     }
     c->pair_tet = c->alloc<int32_t>(pcap);
     c->bins = c->alloc<int32_t>(pcap);
-    c->rcount = c->alloc<unsigned long long>(3);
-    c->qcount = c->alloc<unsigned long long>(RPD_NBINS);
-    NEED(c->pair_tet && c->bins && c->rcount && c->qcount);
-    launch_bin_pairs(c->cand_cnt, c->pair_off, nt, c->pair_tet, c->bins, c->bin_count, c->bin_fill, pcap, c->rcount,
-                     c->qcount, s, c->changed);
+    NEED(c->pair_tet && c->bins);
+    launch_bin_pairs(c->cand_cnt, c->pair_off, nt, c->pair_tet, c->bins, bc, pcap, s, c->changed);
     cudaStreamWaitEvent(s, c->ev[2], 0);   // mesh combinatorics done
     ReportBlock report;
     NEED(report.h);
@@ -731,8 +730,8 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
         c->pair_tet = c->alloc<int32_t>(npairs);
         c->bins = c->alloc<int32_t>(npairs);
         NEED(c->pair_tet && c->bins);
-        launch_bin_pairs(c->cand_cnt, c->pair_off, nt, c->pair_tet, c->bins, c->bin_count, c->bin_fill, npairs,
-                         c->rcount, c->qcount, s, c->changed);
+        cudaMemsetAsync(bc.fill, 0, sizeof(int32_t) * RPD_NBINS, s);
+        launch_bin_pairs(c->cand_cnt, c->pair_off, nt, c->pair_tet, c->bins, bc, npairs, s, c->changed);
     }
     for (int b = 1; b < RPD_NBINS; b++) {
         long long n = c->hbin[b];

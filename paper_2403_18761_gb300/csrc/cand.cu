@@ -315,7 +315,13 @@ __device__ __forceinline__ long long leaf_near(const Box& b, const Leaf& f, long
                     z = max(max(f.lo.z - b.hi[2], b.lo[2] - f.hi.z), 0);
     return x * x + y * y + z * z - wmax;
 }
-// ... at one point.
+// ... and one sphere.
+__device__ __forceinline__ long long box_near(const Box& b, int4 c, long long w) {
+    const long long x = max(max(c.x - b.hi[0], b.lo[0] - c.x), 0), y = max(max(c.y - b.hi[1], b.lo[1] - c.y), 0),
+                    z = max(max(c.z - b.hi[2], b.lo[2] - c.z), 0);
+    return x * x + y * y + z * z - w;
+}
+// ... over the leaf's spheres, at one point.
 __device__ __forceinline__ long long leaf_near(int3 p, const Leaf& f, long long wmax) {
     const long long x = max(max(f.lo.x - p.x, p.x - f.hi.x), 0), y = max(max(f.lo.y - p.y, p.y - f.hi.y), 0),
                     z = max(max(f.lo.z - p.z, p.z - f.hi.z), 0);
@@ -551,10 +557,17 @@ __global__ void __launch_bounds__(32 * WARPS) k_candidates_packet(CandArgs A, co
     int* near_l = near_s[warp];
     int nn = 0;
     walk(A, S, b, cj, vj, R, [&](long long, int e, int n) {
+        int4 s = make_int4(0, 0, 0, 0);
+        long long w = 0;
         bool take = lane < n;
+        if (take) {   // within the thresholds at some point of the box?
+            s = A.sph[e + lane];
+            w = A.sw[e + lane];
+            take = box_near(b, s, w) <= R;
+        }
+        if (!__any_sync(FULL, take)) return;
         if (take) {
-            const int4 s = A.sph[e + lane];
-            const long long vs = pd4(b, s, A.sw[e + lane]);
+            const long long vs = pd4(b, s, w);
             for (int k = 0; k < nd && take; k++) take = reaches(b, s, vs, dom_c[warp][k], dom_v[warp][k]);
         }
         const unsigned m = __ballot_sync(FULL, take);

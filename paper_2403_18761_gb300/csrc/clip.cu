@@ -1677,29 +1677,21 @@ __global__ void k_bin_count(const int32_t* __restrict__ cand_cnt, long long nt, 
     warp_bin_add(n, n > 0 ? bin_of(n) : 0, bin_count);
 }
 
-__global__ void k_bin_prefix(const int32_t* __restrict__ bin_count, int32_t* __restrict__ bin_fill,
-                             unsigned long long* __restrict__ rcount, unsigned long long* __restrict__ qcount) {
-    int run = 0;
-    for (int b = 0; b < RPD_NBINS; b++) {
-        bin_fill[b] = run;
-        run += bin_count[b];
-        if (qcount) qcount[b] = 0;
-    }
-    if (rcount)
-        for (int k = 0; k < 3; k++) rcount[k] = 0;
-}
-
 // Writes past cap are dropped (the caller bins again with room for all pairs).
 // Every pair gets its tet in pair_tet; only the pairs of the tets `only`
 // marks (all when NULL) are put into the bins.
 __global__ void k_bin_pairs(const int32_t* __restrict__ cand_cnt, const int64_t* __restrict__ pair_off, long long nt,
-                            int32_t* __restrict__ pair_tet, int32_t* __restrict__ bins, int32_t* __restrict__ bin_fill,
-                            long long cap, const uint8_t* __restrict__ only) {
+                            int32_t* __restrict__ pair_tet, int32_t* __restrict__ bins,
+                            const int32_t* __restrict__ bin_count, int32_t* __restrict__ bin_fill, long long cap,
+                            const uint8_t* __restrict__ only) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int n = t < nt ? cand_cnt[t] : 0;
     const int nb = (t < nt && (!only || only[t])) ? n : 0;
-    const int base = warp_bin_add(nb, nb > 0 ? bin_of(nb) : 0, bin_fill);
+    const int bin = nb > 0 ? bin_of(nb) : 0;
+    int base = warp_bin_add(nb, bin, bin_fill);
     if (n <= 0) return;
+    for (int b = 0; b < RPD_NBINS - 1; b++)   // the bins before this one
+        if (b < bin) base += bin_count[b];
     const long long off = pair_off[t];
     for (int k = 0; k < n; k++) {
         if (off + k < cap) pair_tet[off + k] = (int32_t)t;
@@ -1775,20 +1767,18 @@ int clip_vmax(int bin) {
     return v[bin];
 }
 
-void launch_bin_count(const int32_t* cand_cnt, long long nt, int32_t* bin_count, cudaStream_t s, const uint8_t* only) {
-    cudaMemsetAsync(bin_count, 0, sizeof(int32_t) * RPD_NBINS, s);
+void launch_bin_count(const int32_t* cand_cnt, long long nt, const BinCounters& c, cudaStream_t s,
+                      const uint8_t* only) {
+    cudaMemsetAsync(c.mem, 0, BinCounters::BYTES, s);
     if (nt == 0) return;
-    k_bin_count<<<nblk(nt, 256), 256, 0, s>>>(cand_cnt, nt, bin_count, only);
+    k_bin_count<<<nblk(nt, 256), 256, 0, s>>>(cand_cnt, nt, c.count, only);
     note_launch();
 }
 
 void launch_bin_pairs(const int32_t* cand_cnt, const int64_t* pair_off, long long nt, int32_t* pair_tet, int32_t* bins,
-                      const int32_t* bin_count, int32_t* bin_fill, long long cap, unsigned long long* rcount,
-                      unsigned long long* qcount, cudaStream_t s, const uint8_t* only) {
-    k_bin_prefix<<<1, 1, 0, s>>>(bin_count, bin_fill, rcount, qcount);
-    note_launch();
+                      const BinCounters& c, long long cap, cudaStream_t s, const uint8_t* only) {
     if (nt == 0) return;
-    k_bin_pairs<<<nblk(nt, 256), 256, 0, s>>>(cand_cnt, pair_off, nt, pair_tet, bins, bin_fill, cap, only);
+    k_bin_pairs<<<nblk(nt, 256), 256, 0, s>>>(cand_cnt, pair_off, nt, pair_tet, bins, c.count, c.fill, cap, only);
     note_launch();
 }
 

@@ -172,18 +172,32 @@ struct ClipArgs {
 // Pairs are grouped into bins by the candidate count n of their tet
 // (0: n = 1, whole tet; 1..3: n = 2..4; 4: 5-6; 5: 7-8; 6: 9-16; 7: 17-32).
 #define RPD_NBINS 8
+// Counters of the binning and the clip in one block, cleared by one memset
+// (launch_bin_count): pairs per bin, the binning's cursors, records per kind,
+// queued pieces per bin.
+struct BinCounters {
+    char* mem = nullptr;
+    int32_t *count = nullptr, *fill = nullptr;
+    unsigned long long *rcount = nullptr, *qcount = nullptr;
+    static constexpr size_t BYTES = 8 * RPD_NBINS + 8 * (3 + RPD_NBINS);
+    void set(void* p) {
+        mem = (char*)p;
+        count = (int32_t*)mem;
+        fill = count + RPD_NBINS;
+        rcount = (unsigned long long*)(fill + RPD_NBINS);
+        qcount = rcount + 3;
+    }
+};
 int clip_vmax(int bin);
 // `only` (NULL = every tet) restricts the binning to the tets it marks.
-void launch_bin_count(const int32_t* cand_cnt, long long nt, int32_t* bin_count, cudaStream_t s,
+void launch_bin_count(const int32_t* cand_cnt, long long nt, const BinCounters& c, cudaStream_t s,
                       const uint8_t* only = nullptr);
 // bins: one array of npairs pair ids, bin b starting at sum of earlier counts.
 // Pairs grouped by bin (pair_tet and bins hold cap entries; writes past cap
-// are dropped); also zeroes the record and queue counters when given.
+// are dropped).  The cursors start at 0.
 // pair_tet is filled for every pair, the bins only for the tets `only` marks.
-void launch_bin_pairs(const int32_t* cand_cnt, const int64_t* pair_off, long long nt, int32_t* pair_tet,
-                      int32_t* bins, const int32_t* bin_count, int32_t* bin_fill, long long cap,
-                      unsigned long long* rcount, unsigned long long* qcount, cudaStream_t s,
-                      const uint8_t* only = nullptr);
+void launch_bin_pairs(const int32_t* cand_cnt, const int64_t* pair_off, long long nt, int32_t* pair_tet, int32_t* bins,
+                      const BinCounters& c, long long cap, cudaStream_t s, const uint8_t* only = nullptr);
 // Pair counts are read on the device (d_n); n/nmax only size the grid.
 void launch_whole_tets(const ClipArgs& a, const int32_t* pairs, const int32_t* d_n, long long nmax, cudaStream_t s);
 void launch_clip(const ClipArgs& a, int bin, int precision, const int32_t* pairs, const int32_t* d_n, long long n,

@@ -14,31 +14,31 @@
 
 namespace {
 
-__global__ void k_snap_points(const double* __restrict__ x, long long n3, double scale, int32_t* __restrict__ out,
-                              DevState* st) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n3) return;
-    double v = x[i] * scale;
-    if (!(fabs(v) <= (double)RPD_COORD_MAX)) {   // also rejects NaN
-        dev_fail(st, RPD_E_INVALID, CNT_INVALID);
-        out[i] = 0;
-        return;
+// Vertex coordinates, sphere centres and radii, one after the other.
+__global__ void k_snap(const double* __restrict__ x, long long nx, const double* __restrict__ c, long long nc,
+                       const double* __restrict__ r, long long nr, double scale, int32_t* __restrict__ Xi,
+                       int32_t* __restrict__ Ci, long long* __restrict__ W, DevState* st) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nx + nc) {
+        const double v = (i < nx ? x[i] : c[i - nx]) * scale;
+        int32_t* out = i < nx ? Xi + i : Ci + (i - nx);
+        if (!(fabs(v) <= (double)RPD_COORD_MAX)) {   // also rejects NaN
+            dev_fail(st, RPD_E_INVALID, CNT_INVALID);
+            *out = 0;
+            return;
+        }
+        *out = (int32_t)rint(v);
+    } else if (i < nx + nc + nr) {
+        const long long k = i - nx - nc;
+        const double v = r[k] * scale;
+        if (!(v >= 0.0 && v <= (double)(1 << 22))) {
+            dev_fail(st, RPD_E_INVALID, CNT_INVALID);
+            W[k] = 0;
+            return;
+        }
+        const long long q = (long long)rint(v);
+        W[k] = q * q;
     }
-    out[i] = (int32_t)rint(v);
-}
-
-__global__ void k_snap_radii(const double* __restrict__ r, long long n, double scale, long long* __restrict__ W,
-                             DevState* st) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double v = r[i] * scale;
-    if (!(v >= 0.0 && v <= (double)(1 << 22))) {
-        dev_fail(st, RPD_E_INVALID, CNT_INVALID);
-        W[i] = 0;
-        return;
-    }
-    long long q = (long long)rint(v);
-    W[i] = q * q;
 }
 
 // Mesh combinatorics by hashing: every tet inserts its 4 faces (sorted vertex
@@ -222,18 +222,11 @@ size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
 void launch_snap(const double* d_verts, long long nv, const double* d_centers, const double* d_radii, long long ns,
                  int grid_bits, int32_t* Xi, int32_t* Ci, long long* W, DevState* st, cudaStream_t s) {
-    double scale = ldexp(1.0, grid_bits);
-    const int T = 256;
-    if (nv) {
-        k_snap_points<<<nblk(3 * nv, T), T, 0, s>>>(d_verts, 3 * nv, scale, Xi, st);
-        note_launch();
-    }
-    if (ns) {
-        k_snap_points<<<nblk(3 * ns, T), T, 0, s>>>(d_centers, 3 * ns, scale, Ci, st);
-        note_launch();
-        k_snap_radii<<<nblk(ns, T), T, 0, s>>>(d_radii, ns, scale, W, st);
-        note_launch();
-    }
+    const long long n = 3 * nv + 3 * ns + ns;
+    if (n == 0) return;
+    k_snap<<<nblk(n, 256), 256, 0, s>>>(d_verts, 3 * nv, d_centers, 3 * ns, d_radii, ns, ldexp(1.0, grid_bits), Xi, Ci,
+                                        W, st);
+    note_launch();
 }
 
 static int log2_cap(long long n) {

@@ -64,7 +64,28 @@ __global__ void scan_tiles(const T* __restrict__ in, int64_t* __restrict__ out, 
         if (i < n) out[i] = pre;
         pre += v[k];
     }
-    if (threadIdx.x == 0) tile_sum[blockIdx.x] = tot;
+    if (threadIdx.x == 0) {
+        tile_sum[blockIdx.x] = tot;
+        if (gridDim.x == 1) out[n] = tot;
+    }
+}
+
+// Every tile adds the sums of the tiles before it, which it sums itself: up to
+// SCAN_FLAT tiles that is a few reads per thread, and cheaper than the three
+// more launches of a scan of the sums.
+constexpr long long SCAN_FLAT = 4096;
+__global__ void scan_finish(int64_t* __restrict__ out, long long n, const int64_t* __restrict__ tile_sum) {
+    __shared__ long long tot;
+    long long part = 0;
+    for (long long j = threadIdx.x; j < blockIdx.x; j += SCAN_THREADS) part += tile_sum[j];
+    block_excl_scan(part, &tot);
+    const long long add = tot;
+    const long long base = (long long)blockIdx.x * SCAN_TILE;
+    for (int k = threadIdx.x; k < SCAN_TILE; k += SCAN_THREADS) {
+        const long long i = base + k;
+        if (i < n) out[i] += add;
+    }
+    if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) out[n] = add + tile_sum[blockIdx.x];
 }
 
 __global__ void scan_add(int64_t* __restrict__ out, long long n, const int64_t* __restrict__ tile_off) {
@@ -74,10 +95,7 @@ __global__ void scan_add(int64_t* __restrict__ out, long long n, const int64_t* 
         long long i = base + k;
         if (i < n) out[i] += add;
     }
-}
-
-__global__ void scan_total(int64_t* out, long long n, const int64_t* tile_off, long long ntiles) {
-    out[n] = tile_off[ntiles];
+    if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) out[n] = tile_off[gridDim.x];
 }
 
 long long n_tiles(long long n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
@@ -102,15 +120,13 @@ void scan_impl(const T* in, int64_t* out, long long n, void* tmp, cudaStream_t s
     void* rest = toff + t + 1;
     scan_tiles<T><<<(unsigned)t, SCAN_THREADS, 0, s>>>(in, out, n, tsum);
     note_launch();
-    if (t == 1) {
-        cudaMemsetAsync(toff, 0, sizeof(int64_t), s);
-        cudaMemcpyAsync(toff + 1, tsum, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
+    if (t == 1) return;
+    if (t <= SCAN_FLAT) {
+        scan_finish<<<(unsigned)t, SCAN_THREADS, 0, s>>>(out, n, tsum);
     } else {
         scan_impl<int64_t>(tsum, toff, t, rest, s);
         scan_add<<<(unsigned)t, SCAN_THREADS, 0, s>>>(out, n, toff);
-        note_launch();
     }
-    scan_total<<<1, 1, 0, s>>>(out, n, toff, t);
     note_launch();
 }
 

@@ -145,8 +145,8 @@ extern "C" rpd_status rpd_euler_static(const double* d_verts, int64_t nv, const 
     int32_t* fb_count = ar.take<int32_t>(1);
     int64_t* pair_off = ar.take<int64_t>(nt + 1);
     void* stmp = ar.take<char>(scan_tmp_bytes(nt + 1));
-    int32_t* bin_count = ar.take<int32_t>(RPD_NBINS);
-    int32_t* bin_fill = ar.take<int32_t>(RPD_NBINS);
+    BinCounters bc;
+    bc.set(ar.take<char>(BinCounters::BYTES));
     NEED_S(!ar.full);
     cudaMemsetAsync(st, 0, sizeof(DevState), s);
     cudaMemcpyAsync(tets, d_tets, sizeof(int32_t) * 4 * nt, cudaMemcpyDeviceToDevice, s);
@@ -158,18 +158,16 @@ extern "C" rpd_status rpd_euler_static(const double* d_verts, int64_t nv, const 
     launch_candidates(tets, nt, nv, Xi, Ci, W, knn, dplus, K, gp, cell_start, cell_ids, cell_wmax, cand_cnt, cand,
                       cand_ord, fb_list, fb_count, st, s);
     scan_excl(cand_cnt, pair_off, nt, stmp, s);
-    launch_bin_count(cand_cnt, nt, bin_count, s);
+    launch_bin_count(cand_cnt, nt, bc, s);
     long long npairs = 0;
     int32_t hb[RPD_NBINS];
     cudaMemcpyAsync(&npairs, pair_off + nt, sizeof(long long), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(hb, bin_count, sizeof(hb), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(hb, bc.count, sizeof(hb), cudaMemcpyDeviceToHost, s);
     TRY_S(read_status(st, s));
     // ---- A3-A4
     ClipArgs a{};
     int32_t* pair_tet = ar.take<int32_t>(npairs);
     int32_t* bins = ar.take<int32_t>(npairs);
-    unsigned long long* rcount = ar.take<unsigned long long>(3);
-    unsigned long long* qcount = ar.take<unsigned long long>(RPD_NBINS);
     a.tets = tets;
     a.Xi = Xi;
     a.Ci = Ci;
@@ -191,7 +189,7 @@ extern "C" rpd_status rpd_euler_static(const double* d_verts, int64_t nv, const 
     a.f_cnt = ar.take<uint8_t>(npairs);
     a.e_off = ar.take<int32_t>(npairs);
     a.e_cnt = ar.take<uint8_t>(npairs);
-    a.rcount = rcount;
+    a.rcount = bc.rcount;
     a.key_bits = b;
     a.force_slow = o.debug_checks & 3;
     a.uf_limit = uf_iteration_limit();
@@ -214,26 +212,26 @@ extern "C" rpd_status rpd_euler_static(const double* d_verts, int64_t nv, const 
         qtrip[bb] = ar.take<uint32_t>(2LL * hb[bb] * clip_vmax(bb));
     }
     NEED_S(!ar.full);
-    launch_bin_pairs(cand_cnt, pair_off, nt, pair_tet, bins, bin_count, bin_fill, npairs, rcount, qcount, s);
+    launch_bin_pairs(cand_cnt, pair_off, nt, pair_tet, bins, bc, npairs, s);
     long long off = 0;
     for (int bb = 0; bb < RPD_NBINS; bb++) {
         const long long nb = hb[bb];
         if (bb == 0) {
-            launch_whole_tets(a, bins, bin_count, nb, s);
+            launch_whole_tets(a, bins, bc.count, nb, s);
         } else if (nb > 0) {
             ClipArgs ab = a;
             ab.qpair = qpair[bb];
             ab.qnv = qnv[bb];
             ab.qtrip = qtrip[bb];
             ab.qcap = nb;
-            ab.qcount = qcount + bb;
-            launch_clip(ab, bb, o.precision, bins + off, bin_count + bb, nb, s);
+            ab.qcount = bc.qcount + bb;
+            launch_clip(ab, bb, o.precision, bins + off, bc.count + bb, nb, s);
             launch_records(ab, bb, nb, s);
         }
         off += nb;
     }
     unsigned long long cnt[3];
-    cudaMemcpyAsync(cnt, rcount, sizeof(cnt), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(cnt, bc.rcount, sizeof(cnt), cudaMemcpyDeviceToHost, s);
     TRY_S(read_status(st, s));
     for (int k = 0; k < 3; k++)
         if ((long long)cnt[k] > rc[k]) return fail_static(RPD_E_OVERFLOW, "element records exceed their capacity");
