@@ -411,7 +411,8 @@ __device__ __forceinline__ void nearest_on_triangle(const double* T, const doubl
 constexpr int SHRINK_ITERS = 100;
 
 // Sphere shrinking against all boundary triangles except the pin's own, one
-// warp (and block) per pin.
+// block per pin: one warp where there are pins enough to fill the SMs, else
+// NW warps that share out the groups and meet once per iteration.
 //
 // FP64 runs at 1/64 of the FP32 rate here, so a warp-wide FP64 point-triangle
 // test (a few hundred FP64 instructions) costs about two microseconds of an
@@ -436,22 +437,30 @@ constexpr int SHRINK_ITERS = 100;
 // (distance, lowest index) minimum is that of testing them all.
 //
 // On a 125k-tet slab (28k boundary triangles, a pin on each) a scan of all
-// bounding balls by an 8-CTA cluster per pin took 152.8 ms, 24 pins 0.66 ms.
+// bounding balls by an 8-CTA cluster per pin took 152.8 ms, 24 pins 0.60 ms;
+// this search 1.55 ms, and 24 pins 0.25 ms with one warp each, 0.21 with four
+// (eight: 0.23).
 // Output centre and radius (NaN for a pin row without a face).
-__global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, ShrinkIndex S, long long ntri,
+template <int NW>
+__global__ void __launch_bounds__(32 * NW) k_shrink(const double* __restrict__ tri, ShrinkIndex S, long long ntri,
                                                const double* __restrict__ pins, const double* __restrict__ normals,
                                                const int32_t* __restrict__ faces, double r0,
                                                const double* __restrict__ r_start, double* __restrict__ centres,
                                                double* __restrict__ radii, int32_t* __restrict__ iters,
                                                int32_t* __restrict__ restarted) {
     const unsigned FULL = 0xffffffffu;
-    __shared__ int list[64];      // collected triangles (sorted positions)
-    __shared__ float list_lb[64];
+    __shared__ int list_s[NW][64];      // collected triangles (sorted positions) of each warp
+    __shared__ float list_lb_s[NW][64];
+    __shared__ unsigned ub_s;           // the warps' bound (bits of a float >= 0)
+    __shared__ double near_d[NW], near_q[NW][3];   // the warps' nearest triangles
+    __shared__ int near_k[NW];
     const long long j = blockIdx.x;
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int* list = list_s[warp];
+    float* list_lb = list_lb_s[warp];
     const int own = faces[j];
     if (own < 0) {
-        if (lane == 0) {
+        if (threadIdx.x == 0) {
             for (int k = 0; k < 3; k++) centres[3 * j + k] = nan("");
             radii[j] = nan("");
             iters[j] = 0;
@@ -470,21 +479,39 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
     int rs_flag = 0;
     double r = warm ? rs : r0;
     int it = 0;
-    for (; it < SHRINK_ITERS; it++) {   // everything that steers the loop is uniform over the warp
+    for (; it < SHRINK_ITERS; it++) {   // everything that steers the loop is uniform over the block
         const double c[3] = {p[0] + r * n[0], p[1] + r * n[1], p[2] + r * n[2]};
         const float cx = (float)c[0], cy = (float)c[1], cz = (float)c[2];
         const float cslack = 3.0f * 0x1p-18f * fmaxf(fabsf(cx), fmaxf(fabsf(cy), fabsf(cz)));
         float ub = __double2float_ru(r * (1.0 + 0x1p-20));
+        if (NW > 1) {
+            if (threadIdx.x == 0) ub_s = __float_as_uint(ub);
+            __syncthreads();
+        }
+        // lower the bound to v (all lanes call it), and take the other warps' in
+        auto tighten = [&](float v) {
+            unsigned u = __reduce_min_sync(FULL, __float_as_uint(v));
+            if (NW > 1) {
+                if (lane == 0) {
+                    const unsigned o = *(volatile unsigned*)&ub_s;
+                    if (u < o) atomicMin(&ub_s, u);
+                    else u = o;
+                }
+                u = __shfl_sync(FULL, u, 0);
+            }
+            ub = fminf(ub, __uint_as_float(u));
+        };
         if (fresh) {   // far from the fixed point: a first bound from the groups of two or more triangles
             float far = INFINITY;
-            for (long long g = lane; g < ngroup; g += 32) {
+            for (long long g = threadIdx.x; g < ngroup; g += 32 * NW) {
                 if (32 * g + 1 >= ntri) continue;   // a lone triangle may be the pin's own
                 const float4 lo = S.glo[g], hi = S.ghi[g];
                 const float fx = fmaxf(fabsf(cx - lo.x), fabsf(cx - hi.x)), fy = fmaxf(fabsf(cy - lo.y), fabsf(cy - hi.y)),
                             fz = fmaxf(fabsf(cz - lo.z), fabsf(cz - hi.z));
                 far = fminf(far, sqrtf(fx * fx + fy * fy + fz * fz) * (1.0f + 0x1p-18f) + cslack);
             }
-            ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(far))));
+            tighten(far);
+            if (NW > 1) __syncthreads();   // every warp starts from the best
         }
         double bd = INFINITY, bq[3] = {0, 0, 0};
         int bi = -1, cnt = 0;
@@ -508,12 +535,12 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
                         for (int z = 0; z < 3; z++) bq[z] = q[z];
                     }
                 }
-                ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(d32))));
+                tighten(d32);
             }
             cnt -= m;
             __syncwarp();
         };
-        for (long long g0 = 0; g0 < ngroup; g0 += 32) {
+        for (long long g0 = 32 * warp; g0 < ngroup; g0 += 32 * NW) {
             float lbg = INFINITY;
             if (g0 + lane < ngroup) {
                 const float4 lo = S.glo[g0 + lane], hi = S.ghi[g0 + lane];
@@ -540,7 +567,7 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
                         far = v + m;
                     }
                 }
-                ub = fminf(ub, __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(far))));
+                tighten(far);
                 const unsigned in = __ballot_sync(FULL, lb <= ub);
                 if (lb <= ub) {
                     const int at = cnt + __popc(in & ((1u << lane) - 1u));
@@ -584,6 +611,26 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
             }
         }
         src = __shfl_sync(FULL, src, 0);
+        double q[3] = {__shfl_sync(FULL, bq[0], src), __shfl_sync(FULL, bq[1], src), __shfl_sync(FULL, bq[2], src)};
+        if (NW > 1) {   // over the warps
+            if (lane == 0) {
+                near_d[warp] = d;
+                near_k[warp] = k;
+                for (int z = 0; z < 3; z++) near_q[warp][z] = q[z];
+            }
+            __syncthreads();
+            d = near_d[0];
+            k = near_k[0];
+            int w = 0;
+            for (int z = 1; z < NW; z++)
+                if (near_d[z] < d || (near_d[z] == d && near_k[z] >= 0 && (k < 0 || near_k[z] < k))) {
+                    d = near_d[z];
+                    k = near_k[z];
+                    w = z;
+                }
+            for (int z = 0; z < 3; z++) q[z] = near_q[w][z];
+            __syncthreads();   // read before the next iteration writes them
+        }
         fresh = false;
         // empty ball (within rounding): done, unless it is a proposed one
         bool stop = false;
@@ -596,8 +643,6 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
                 stop = true;
             }
         } else {
-            const double q[3] = {__shfl_sync(FULL, bq[0], src), __shfl_sync(FULL, bq[1], src),
-                                 __shfl_sync(FULL, bq[2], src)};
             const double pq[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
             const double dn = pq[0] * n[0] + pq[1] * n[1] + pq[2] * n[2];
             const double rn = (pq[0] * pq[0] + pq[1] * pq[1] + pq[2] * pq[2]) / (2.0 * dn);
@@ -607,7 +652,7 @@ __global__ void __launch_bounds__(32) k_shrink(const double* __restrict__ tri, S
         warm = false;
         if (stop) break;
     }
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
         for (int k = 0; k < 3; k++) centres[3 * j + k] = p[k] + r * n[k];
         radii[j] = r;
         iters[j] = it + 1;
@@ -815,8 +860,14 @@ void launch_shrink(const double* tri, const ShrinkIndex& S, long long ntri, cons
                    const int32_t* faces, long long n, double r0, const double* r_start, double* centres, double* radii,
                    int32_t* iters, int32_t* restarted, cudaStream_t s) {
     if (n <= 0) return;
-    k_shrink<<<(unsigned)n, 32, 0, s>>>(tri, S, ntri, pins, normals, faces, r0, r_start, centres, radii, iters,
-                                        restarted);
+    // four warps per pin while that leaves SMs with a few warps at most (a pin's
+    // iterations are a serial chain), one above
+    if (n <= 152 * 2)
+        k_shrink<4><<<(unsigned)n, 128, 0, s>>>(tri, S, ntri, pins, normals, faces, r0, r_start, centres, radii, iters,
+                                                restarted);
+    else
+        k_shrink<1><<<(unsigned)n, 32, 0, s>>>(tri, S, ntri, pins, normals, faces, r0, r_start, centres, radii, iters,
+                                               restarted);
     note_launch();
 }
 
