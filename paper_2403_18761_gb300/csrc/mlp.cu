@@ -153,7 +153,7 @@ constexpr int PSTRIDE = 37440;   // floats of one CTA's partial gradient: NPARAM
 constexpr int IW0 = 0, IW1 = IW0 + HID * NIN, IW2 = IW1 + HID * HID, IW1T = IW2 + HID * HID, IW2T = IW1T + HID * HID,
               NIMG = IW2T + HID * HID;
 
-// Shared memory of one CTA (one per SM): 220 KB.
+// Shared memory of one CTA (one per SM): 226 KB.
 struct StepSmem {
     __nv_bfloat16 x[TM * NIN], xt[NIN * TM];   // the tile's inputs, by row and transposed
     __nv_bfloat16 w0[HID * NIN];
@@ -161,6 +161,7 @@ struct StepSmem {
     __nv_bfloat16 row[TM * HID];                  // the A operand: H0, H1, dZ2, dZ1 by row
     __nv_bfloat16 h0t[HID * TM], h1t[HID * TM];   // transposed activations (weight gradients' B operand)
     __nv_bfloat16 zt[HID * TM];                   // H2, then dZ2, dZ1, dZ0, transposed (their A operand)
+    uint32_t mask[3][2][STEP_THREADS];            // ReLU masks by layer, 32 columns a word
     float bias[3][HID], w3[HID], ypart[2][TM], dy[TM], red[HID], lred[4];
     uint64_t bar;
     uint32_t tmem;
@@ -211,7 +212,7 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 // SM: eight dependent MMA batches of about 0.1 us each and as many epilogues
 // through shared memory.  The form before this one ran a kernel per layer and
 // direction with global round trips in between and one FP32 atomic per weight
-// and tile: 206 us per step of 8192 rows, 17 launches; now 2 launches.
+// and tile: 206 us per step of 8192 rows, 17 launches; now 33 us and 2.
 //
 // Rows past n (the last tile's) have zero activations and dy = 0.
 // x rows: row r of the pass is row (cur[0] + r) mod n_total of the data when
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     k_mlp_step(const float* __restrict__ x, const float* __restrict__ t, long long n, int n_in, long long n_total,
                long long* __restrict__ cur, const float* __restrict__ p, const __nv_bfloat16* __restrict__ img,
                float* __restrict__ y, float* __restrict__ part, int* __restrict__ err) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int quad = warp & 3, half = warp >> 2;   // TMEM lanes 32 quad.., columns 64 half..
@@ -313,11 +314,11 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             mma_commit(&S.bar);
         }
         end_mma();
-        // hidden layers 0 and 1: bias, ReLU, BF16; the ReLU masks stay in registers
-        uint32_t mask[3][2];
-#pragma unroll
+        // hidden layers 0 and 1: bias, ReLU, BF16 (the loops over layers and
+        // column halves stay rolled: 137 registers instead of 255, same time)
+#pragma unroll 1
         for (int layer = 0; layer < 2; layer++) {
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < 2; c++) {
                 const int c0 = 64 * half + 32 * c;
                 float v[32];
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
                     o[k] = __float2bfloat16(live ? fmaxf(v[k] + S.bias[layer][c0 + k], 0.0f) : 0.0f);
                     mk |= (__bfloat162float(o[k]) > 0.0f ? 1u : 0u) << k;
                 }
-                mask[layer][c] = mk;
+                S.mask[layer][c][tid] = mk;
                 if (GRAD) {
                     put_tile(S.row, layer == 0 ? S.h0t : S.h1t, m, c0, o);
                 } else {
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         if (GRAD) load_image(S.wa, img + IW2T, HID * HID);   // W1 has been consumed
         // layer 2 and the head
         float ys = 0.0f;
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < 2; c++) {
             const int c0 = 64 * half + 32 * c;
             float v[32];
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
                 mk |= (h > 0.0f ? 1u : 0u) << k;
                 ys += h * S.w3[c0 + k];
             }
-            mask[2][c] = mk;
+            S.mask[2][c][tid] = mk;
             if (GRAD) put_tile(nullptr, S.zt, m, c0, o);
         }
         S.ypart[half][m] = ys;
@@ -391,16 +392,17 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         gw3 += col_sum(true);
         const float dy = S.dy[m];
         __syncthreads();   // H2 has been read
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < 2; c++) {
             const int c0 = 64 * half + 32 * c;
+            const uint32_t mk = S.mask[2][c][tid];
             __align__(16) __nv_bfloat16 o[32];
 #pragma unroll
-            for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mask[2][c] >> k) & 1u ? dy * S.w3[c0 + k] : 0.0f);
+            for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mk >> k) & 1u ? dy * S.w3[c0 + k] : 0.0f);
             put_tile(S.row, S.zt, m, c0, o);
         }
         // layers 2 and 1: weight gradient and input gradient in one batch
-#pragma unroll
+#pragma unroll 1
         for (int layer = 2; layer >= 1; layer--) {
             if (layer == 2) cp_async_wait<1>();   // W2^T
             else cp_async_wait<0>();              // W1^T
@@ -410,16 +412,19 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
                 issue(layer == 2 ? DW2 : DW1, S.zt, layer == 2 ? S.h1t : S.h0t, TM, HID, !first);
                 mma_commit(&S.bar);
             }
-            gb[layer] += col_sum(false);   // beside the MMAs: both only read zt
+            const float cs = col_sum(false);   // beside the MMAs: both only read zt
+            gb[2] += layer == 2 ? cs : 0.0f;
+            gb[1] += layer == 2 ? 0.0f : cs;
             end_mma();
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < 2; c++) {
                 const int c0 = 64 * half + 32 * c;
+                const uint32_t mk = S.mask[layer - 1][c][tid];
                 float v[32];
                 tmem_ld32(T0 + D + tlane + (uint32_t)c0, v);
                 __align__(16) __nv_bfloat16 o[32];
 #pragma unroll
-                for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mask[layer - 1][c] >> k) & 1u ? v[k] : 0.0f);
+                for (int k = 0; k < 32; k++) o[k] = __float2bfloat16((mk >> k) & 1u ? v[k] : 0.0f);
                 put_tile(layer == 2 ? S.row : nullptr, S.zt, m, c0, o);
             }
         }
@@ -437,10 +442,12 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         // this CTA's partial gradient: the accumulators, then the column sums
         float* g = part + (long long)blockIdx.x * PSTRIDE;
         if (ok) {
+#pragma unroll 1
             for (int layer = 0; layer < 3; layer++) {
                 const int K = layer == 0 ? NIN : HID;
                 const uint32_t d = layer == 0 ? DW0 : (layer == 1 ? DW1 : DW2);
                 float* gw = g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2)) + (long long)m * K;
+#pragma unroll 1
                 for (int c = 0; c < 2; c++) {
                     const int c0 = K == HID ? 64 * half + 32 * c : 0;
                     if (K == NIN && (half || c)) continue;   // warp-uniform
@@ -506,32 +513,51 @@ __global__ void k_cast_weights(const float* __restrict__ p, __nv_bfloat16* __res
     if (i < NPARAM) put_weight(img, i, p[i]);
 }
 
-// Sum of the CTAs' partial gradients, in CTA order, into g; loss at NPARAM.
+// Sum of the CTAs' partial gradients for parameter i, loss at NPARAM: PGROUP
+// threads each sum every PGROUP-th CTA's, then the first adds the groups' sums
+// in order (only its result counts).  One thread summing all 64 waited for
+// memory most of its 9.6 us (6.5 now).
+constexpr int PGROUP = 8, PCOLS = 32;   // a block: 32 parameters x 8 groups
 __device__ __forceinline__ float part_sum(const float* __restrict__ part, int np, long long i) {
+    __shared__ float sums[PGROUP][PCOLS];
+    const int col = threadIdx.x % PCOLS, grp = threadIdx.x / PCOLS;
     float s = 0.0f;
+    if (i <= NPARAM) {
 #pragma unroll 8
-    for (int c = 0; c < np; c++) s += part[(long long)c * PSTRIDE + i];
+        for (int c = grp; c < np; c += PGROUP) s += part[(long long)c * PSTRIDE + i];
+    }
+    sums[grp][col] = s;
+    __syncthreads();
+    if (grp) return 0.0f;
+    for (int g = 1; g < PGROUP; g++) s += sums[g][col];
     return s;
 }
+__device__ __forceinline__ long long part_param() {
+    return (long long)blockIdx.x * PCOLS + threadIdx.x % PCOLS;
+}
 
-__global__ void k_grad_sum(const float* __restrict__ part, int np, float* __restrict__ g, float* __restrict__ loss) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NPARAM) g[i] = part_sum(part, np, i);
-    if (i == NPARAM) *loss = part_sum(part, np, i);
+__global__ void __launch_bounds__(PGROUP* PCOLS) k_grad_sum(const float* __restrict__ part, int np,
+                                                            float* __restrict__ g, float* __restrict__ loss) {
+    const long long i = part_param();
+    const float s = part_sum(part, np, i);
+    if (threadIdx.x >= PCOLS) return;
+    if (i < NPARAM) g[i] = s;
+    if (i == NPARAM) *loss = s;
 }
 
 // Adam step on the FP32 master parameters: the gradient summed from the
 // partials, step number cur[1] (bias corrections 1 - b^step), the BF16 tile
 // images of the new weights, and the next batch's first row.
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ part, int np, float* __restrict__ g,
+__global__ void __launch_bounds__(PGROUP* PCOLS) k_adam(float* __restrict__ p, const float* __restrict__ part, int np, float* __restrict__ g,
                        float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ img,
                        float* __restrict__ loss, float lr, float b1, float b2, float eps, long long* __restrict__ cur,
                        long long b, long long n_total) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) cur[0] = (cur[0] + b) % n_total;   // read by k_mlp_step only
-    if (i == NPARAM) *loss = part_sum(part, np, i);
-    if (i >= NPARAM) return;
+    const long long i = part_param();
     const float gi = part_sum(part, np, i);
+    if (threadIdx.x >= PCOLS) return;
+    if (i == 0) cur[0] = (cur[0] + b) % n_total;   // read by k_mlp_step only
+    if (i == NPARAM) *loss = gi;
+    if (i >= NPARAM) return;
     const float step = (float)cur[1];
     const float c1 = 1.0f - powf(b1, step), c2 = 1.0f - powf(b2, step);
     const float mi = b1 * m[i] + (1.0f - b1) * gi, vi = b2 * v[i] + (1.0f - b2) * gi * gi;
@@ -571,7 +597,8 @@ struct rpd_mlp {
 
 namespace {
 
-size_t step_smem() { return sizeof(StepSmem) + 1024; }
+size_t step_smem() { return sizeof(StepSmem); }
+static_assert(sizeof(StepSmem) <= 227 * 1024, "shared memory of one CTA");
 
 int step_ctas(long long n) { return (int)std::min<long long>((n + TM - 1) / TM, MAX_CTAS); }
 
@@ -713,7 +740,7 @@ rpd_status rpd_mlp_grad(rpd_mlp* q, const float* d_x, const float* d_t, int64_t 
     if (!q || n < 1 || !d_x || !d_t) return RPD_E_INVALID;
     TRY_M(ensure_part(q, n));
     run_step(q, d_x, d_t, n, nullptr);
-    k_grad_sum<<<nblk(NPARAM + 1, 256), 256, 0, q->stream>>>(q->part, step_ctas(n), q->g, q->loss);
+    k_grad_sum<<<nblk(NPARAM + 1, PCOLS), PGROUP * PCOLS, 0, q->stream>>>(q->part, step_ctas(n), q->g, q->loss);
     note_launch();
     if (d_grad) cudaMemcpyAsync(d_grad, q->g, sizeof(float) * NPARAM, cudaMemcpyDeviceToDevice, q->stream);
     if (h_loss) cudaMemcpyAsync(h_loss, q->loss, sizeof(float), cudaMemcpyDeviceToHost, q->stream);
@@ -733,8 +760,9 @@ rpd_status rpd_mlp_train(rpd_mlp* q, const float* d_x, const float* d_t, int64_t
         cudaMemcpyAsync(q->cur, c0, sizeof(c0), cudaMemcpyHostToDevice, q->stream);
         for (int it = 0; it < steps; it++) {
             run_step(q, d_x, d_t, b, nullptr, n);
-            k_adam<<<nblk(NPARAM + 1, 256), 256, 0, q->stream>>>(q->p, q->part, step_ctas(b), q->g, q->m, q->v, q->img,
-                                                                  q->loss, lr, 0.9f, 0.999f, 1e-8f, q->cur, b, n);
+            k_adam<<<nblk(NPARAM + 1, PCOLS), PGROUP * PCOLS, 0, q->stream>>>(q->p, q->part, step_ctas(b), q->g, q->m,
+                                                                              q->v, q->img, q->loss, lr, 0.9f, 0.999f,
+                                                                              1e-8f, q->cur, b, n);
             note_launch();
         }
         q->step += steps;
