@@ -676,7 +676,7 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
         a.fb_list = c->fb_list;
         a.fb_count = c->fb_count;
         a.st = c->st;
-        launch_candidates_packet(a, c->plan, c->d_voff, c->d_soff, ctmp, s);
+        launch_candidates_packet(a, c->plan, c->d_voff, ctmp, s);
     }
     scan_excl(c->cand_cnt, c->pair_off, nt, stmp, s);
     if (old) {   // partial update: clip only the tets whose candidates changed

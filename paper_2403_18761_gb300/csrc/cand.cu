@@ -710,8 +710,7 @@ size_t cand_tmp_bytes(const CandPlan& P, long long nt, long long nv, long long n
            al(sizeof(int64_t) * (P.ncell + 1)) + 3 * al(sizeof(uint32_t) * n) + al(scan_tmp_bytes(P.ncell));
 }
 
-void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* voff, const long long* soff, void* tmp,
-                              cudaStream_t s) {
+void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* voff, void* tmp, cudaStream_t s) {
     if (a.nt == 0) return;
     char* p = (char*)tmp;
     auto take = [&](size_t bytes) {
@@ -779,6 +778,12 @@ void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* vo
     note_launch();
     k_candidates_packet<<<nblk(P.npt, WARPS), 32 * WARPS, 0, s>>>(a, owner);
     note_launch();
-    launch_candidates_fallback(a.T, a.nv, a.Xi, a.Ci, a.W, a.ns, nullptr, 0, nullptr, nullptr, nullptr, nullptr,
-                               a.fb_list, a.fb_count, a.cand_cnt, a.cand, a.cand_ord, a.st, voff, soff, S, s);
+    FallbackTree tree;
+    tree.shapes = a.shapes;
+    tree.one = a.one;
+    tree.leaf = leaf;
+    tree.lwmax = lwmax;
+    tree.sph = sph;
+    launch_candidates_fallback(a.T, a.nv, a.Xi, a.Ci, a.W, tree, nullptr, 0, nullptr, nullptr, nullptr, nullptr,
+                               a.fb_list, a.fb_count, a.cand_cnt, a.cand, a.cand_ord, a.st, voff, S, s);
 }

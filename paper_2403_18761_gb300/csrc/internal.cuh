@@ -66,16 +66,6 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                        int32_t* fb_list, int32_t* fb_count, DevState* st, cudaStream_t s,
                        const long long* voff = nullptr, int nshapes = 1);
 
-// The grid-search fallback of the tets in fb_list.  knn == NULL: cand[32 t]
-// holds the sphere that gives tet t's thresholds; gp == NULL: no sphere grid, every sphere of the shape is tested (soff: shape s owns spheres
-// [soff[s], soff[s + 1]); without a batch all ns).
-void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
-                                const long long* W, long long ns, const int32_t* knn, int K, const GridParams* gp,
-                                const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
-                                const int32_t* fb_list, const int32_t* fb_count, int32_t* cand_cnt, int32_t* cand,
-                                uint8_t* cand_ord, DevState* st, const long long* voff, const long long* soff,
-                                int nshapes, cudaStream_t s);
-
 // ---------------------------------------------------------------- cand.cu
 // A shape's ranges of vertices, tets and spheres, its first vertex and tet
 // packet, leaf, node and order cells, and the halvings of its orders.
@@ -88,6 +78,25 @@ struct CandShape {
 struct Leaf {
     int4 lo, hi;
 };
+// The sphere tree's leaves, for the fallback of the packet search.
+struct FallbackTree {
+    const CandShape* shapes = nullptr;   // NULL: one shape, `one`
+    CandShape one{};
+    const Leaf* leaf = nullptr;
+    const long long* lwmax = nullptr;
+    const int4* sph = nullptr;
+};
+// The fallback (knn.cu) of the tets in fb_list: every sphere within the
+// thresholds that a sphere o gives (pd <= pd(., o) at some corner), then the
+// exact corner test.  With neighbour lists (knn) o is the best of the corners'
+// owners and the spheres come from the grid; without, o = cand[32 t] and they
+// come from the tree's leaves.
+void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
+                                const long long* W, const FallbackTree& tree, const int32_t* knn, int K,
+                                const GridParams* gp, const int64_t* cell_start, const int32_t* cell_ids,
+                                const long long* cell_wmax, const int32_t* fb_list, const int32_t* fb_count,
+                                int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord, DevState* st,
+                                const long long* voff, int nshapes, cudaStream_t s);
 struct CandArgs {
     const int32_t* T;
     long long nt, nv, ns;
@@ -119,8 +128,7 @@ struct CandPlan {
 void cand_plan(const long long* voff, const long long* toff, const long long* soff, int nshapes, long long nv,
                long long nt, long long ns, CandPlan& P);
 size_t cand_tmp_bytes(const CandPlan& P, long long nt, long long nv, long long ns);
-void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* voff, const long long* soff, void* tmp,
-                              cudaStream_t s);
+void launch_candidates_packet(CandArgs a, const CandPlan& P, const long long* voff, void* tmp, cudaStream_t s);
 
 // ---------------------------------------------------------------- clip.cu
 struct ClipArgs {

@@ -1003,12 +1003,14 @@ __global__ void __launch_bounds__(256, 5) k_candidates_warp(
     if (lane == 0) cand_cnt[t] = __popc(kmask);
 }
 
-// Fallback for a tet whose corner lists are not complete enough: one block
+// Fallback for a tet whose corner lists are not complete enough, or which has
+// more spheres near it than the packet search takes: one block
 // per tet collects every sphere m with pd(X_a, m) <= pd(X_a, o_b*) for some
 // corner a (b* as in the warp form), then applies the same exact corner
-// filter and orders.  The threads split all grid cells (each cell and each
-// sphere seen once, so the list needs no duplicate check; cells pruned by
-// their largest weight) and append through a shared counter.  A bounded scan
+// filter and orders.  The threads split all grid cells, or the leaves of the
+// packet search's tree (each sphere seen once, so the list needs no duplicate
+// check; cells and leaves pruned by their largest weight), and append through
+// a shared counter.  A bounded scan
 // replaces a ring search, whose stop test with the largest weight of all
 // spheres can keep it going over most of the grid.
 constexpr int FB_GATHER = 128;   // spheres gathered per tet at most
@@ -1016,12 +1018,12 @@ constexpr int FB_THREADS = 256;
 
 __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
     const int32_t* __restrict__ T, long long nv, const int32_t* __restrict__ Xi, const int32_t* __restrict__ Ci,
-    const long long* __restrict__ W, long long ns, const int32_t* __restrict__ knn, int K,
+    const long long* __restrict__ W, FallbackTree tree, const int32_t* __restrict__ knn, int K,
     const GridParams* __restrict__ gp, const int64_t* __restrict__ start_all, const int32_t* __restrict__ ids,
     const long long* __restrict__ cwmax_all,
     const int32_t* __restrict__ fb_list, const int32_t* __restrict__ fb_count, int32_t* __restrict__ cand_cnt,
     int32_t* __restrict__ cand, uint8_t* __restrict__ cand_ord, DevState* st, const long long* __restrict__ voff,
-    const long long* __restrict__ soff, int nshapes) {
+    int nshapes) {
     const unsigned FULL = 0xffffffffu;
     __shared__ int sid[FB_GATHER];
     __shared__ long long sD[FB_GATHER][4];
@@ -1037,9 +1039,8 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             if (tid == 0) cand_cnt[t] = 0;
             continue;
         }
-        // the grid and the spheres of the tet's shape (its first corner's)
+        // the grid, or the leaves, of the tet's shape (its first corner's)
         const int shp = shape_of(voff, nshapes, v[0]);
-        const long long s0 = nshapes > 1 && soff ? soff[shp] : 0, s1 = nshapes > 1 && soff ? soff[shp + 1] : ns;
         GridParams g{};
         if (gp) g = gp[shp];
         const int64_t* __restrict__ start = start_all + g.cbase;
@@ -1080,8 +1081,27 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             const int pos = atomicAdd(&sn, 1);
             if (pos < FB_GATHER) sid[pos] = sph;
         };
-        if (!gp)
-            for (long long i = s0 + tid; i < s1; i += FB_THREADS) test((int)i);
+        if (!gp) {   // the leaves that may hold a sphere within a threshold, 32 at a time
+            const CandShape& S = tree.shapes ? tree.shapes[shp] : tree.one;
+            const long long nl = (S.s1 - S.s0 + 31) / 32;
+            for (long long l0 = tid & ~31; l0 < nl; l0 += FB_THREADS) {
+                bool open = false;
+                if (l0 + lane < nl) {
+                    const Leaf f = tree.leaf[S.l0 + l0 + lane];
+                    const long long wm = tree.lwmax[S.l0 + l0 + lane];
+                    for (int a = 0; a < 4; a++) {
+                        const long long dx = max(max(f.lo.x - X[a].x, X[a].x - f.hi.x), 0),
+                                        dy = max(max(f.lo.y - X[a].y, X[a].y - f.hi.y), 0),
+                                        dz = max(max(f.lo.z - X[a].z, X[a].z - f.hi.z), 0);
+                        open |= dx * dx + dy * dy + dz * dz - wm <= thr[a];
+                    }
+                }
+                for (unsigned m = __ballot_sync(FULL, open); m; m &= m - 1) {
+                    const long long e = S.s0 + 32 * (l0 + __ffs(m) - 1) + lane;
+                    if (e < S.s1) test(tree.sph[e].w);
+                }
+            }
+        }
         // A sphere with pd(X_a) <= thr_a has its centre within
         // sqrt(thr_a + wmax) of X_a, so only the cells of the box around the
         // four corners' balls can hold one; each of those cells is opened
@@ -1270,18 +1290,18 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                                                           cand_ord,
                                                fb_list, fb_count, st);
     note_launch();
-    launch_candidates_fallback(d_tets, nv, Xi, Ci, W, 0, knn, K, gp, cell_start, cell_ids, cell_wmax, fb_list,
-                               fb_count, cand_cnt, cand, cand_ord, st, voff, nullptr, nshapes, s);
+    launch_candidates_fallback(d_tets, nv, Xi, Ci, W, FallbackTree{}, knn, K, gp, cell_start, cell_ids, cell_wmax, fb_list,
+                               fb_count, cand_cnt, cand, cand_ord, st, voff, nshapes, s);
 }
 
 void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
-                                const long long* W, long long ns, const int32_t* knn, int K, const GridParams* gp,
-                                const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
-                                const int32_t* fb_list, const int32_t* fb_count, int32_t* cand_cnt, int32_t* cand,
-                                uint8_t* cand_ord, DevState* st, const long long* voff, const long long* soff,
-                                int nshapes, cudaStream_t s) {
-    k_candidates_fallback<<<152 * 4, FB_THREADS, 0, s>>>(T, nv, Xi, Ci, W, ns, knn, K, gp, cell_start, cell_ids,
+                                const long long* W, const FallbackTree& tree, const int32_t* knn, int K,
+                                const GridParams* gp, const int64_t* cell_start, const int32_t* cell_ids,
+                                const long long* cell_wmax, const int32_t* fb_list, const int32_t* fb_count,
+                                int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord, DevState* st,
+                                const long long* voff, int nshapes, cudaStream_t s) {
+    k_candidates_fallback<<<152 * 4, FB_THREADS, 0, s>>>(T, nv, Xi, Ci, W, tree, knn, K, gp, cell_start, cell_ids,
                                                          cell_wmax, fb_list, fb_count, cand_cnt, cand, cand_ord, st,
-                                                         voff, soff, nshapes);
+                                                         voff, nshapes);
     note_launch();
 }
