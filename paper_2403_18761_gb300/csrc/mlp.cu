@@ -153,15 +153,25 @@ constexpr int PSTRIDE = 37440;   // floats of one CTA's partial gradient: NPARAM
 constexpr int IW0 = 0, IW1 = IW0 + HID * NIN, IW2 = IW1 + HID * HID, IW1T = IW2 + HID * HID, IW2T = IW1T + HID * HID,
               NIMG = IW2T + HID * HID;
 
-// Shared memory of one CTA (one per SM): 226 KB.
+// Shared memory of one CTA (one per SM): 222 KB.
+// A transposed tile has the core matrices of a column block of eight rows next
+// to each other and the blocks TR_LBO bytes apart: the lanes of a warp hold
+// consecutive columns, and this stride spreads their eight-column blocks over
+// the banks (consecutive core matrices along K put them all on the same eight:
+// four-way conflicts on every transposed store, 11k a CTA; now 330).
+constexpr uint32_t TR_LBO = 16 * 128 + 32;
+constexpr int TR_ELEMS = 16 * (int)TR_LBO / 2;
 struct StepSmem {
-    __nv_bfloat16 x[TM * NIN], xt[NIN * TM];   // the tile's inputs, by row and transposed
+    union {
+        __nv_bfloat16 x[TM * NIN];             // the tile's inputs by row, for the first GEMM only
+        uint32_t mask[3][2][STEP_THREADS];     // then ReLU masks by layer, 32 columns a word
+    };
+    __nv_bfloat16 xt[NIN * TM];                // inputs transposed
     __nv_bfloat16 w0[HID * NIN];
     __nv_bfloat16 wa[HID * HID], wb[HID * HID];   // W1 then W2^T; W2 then W1^T
     __nv_bfloat16 row[TM * HID];                  // the A operand: H0, H1, dZ2, dZ1 by row
-    __nv_bfloat16 h0t[HID * TM], h1t[HID * TM];   // transposed activations (weight gradients' B operand)
-    __nv_bfloat16 zt[HID * TM];                   // H2, then dZ2, dZ1, dZ0, transposed (their A operand)
-    uint32_t mask[3][2][STEP_THREADS];            // ReLU masks by layer, 32 columns a word
+    __nv_bfloat16 h0t[TR_ELEMS], h1t[TR_ELEMS];   // transposed activations (weight gradients' B operand)
+    __nv_bfloat16 zt[TR_ELEMS];                   // H2, then dZ2, dZ1, dZ0, transposed (their A operand)
     float bias[3][HID], w3[HID], ypart[2][TM], dy[TM], red[HID], lred[4];
     uint64_t bar;
     uint32_t tmem;
@@ -175,6 +185,10 @@ __device__ __forceinline__ void load_image(__nv_bfloat16* dst, const __nv_bfloat
 
 __device__ __forceinline__ char* at(__nv_bfloat16* base, int row, int k, int kdim) {
     return reinterpret_cast<char*>(base) + tile_off(row, k, kdim);
+}
+
+__device__ __forceinline__ char* at_tr(__nv_bfloat16* base, int row, int k) {
+    return reinterpret_cast<char*>(base) + (uint32_t)(k >> 3) * TR_LBO + (uint32_t)((row >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2);
 }
 
 // 32 values of one tile row m, columns c0..c0+31, as BF16: by row (when row
@@ -193,7 +207,7 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
     for (int q = 0; q < 16; q++) {   // columns c0 + 2q (even lane's) and c0 + 2q + 1 (odd lane's)
         const uint32_t other = __shfl_xor_sync(0xffffffffu, w[q], 1);
         const uint32_t v = odd ? __byte_perm(w[q], other, 0x3276) : __byte_perm(w[q], other, 0x5410);
-        *reinterpret_cast<uint32_t*>(at(tr, c0 + 2 * q + odd, m & ~1, TM)) = v;
+        *reinterpret_cast<uint32_t*>(at_tr(tr, c0 + 2 * q + odd, m & ~1)) = v;
     }
 }
 
@@ -212,7 +226,10 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 // SM: eight dependent MMA batches of about 0.1 us each and as many epilogues
 // through shared memory.  The form before this one ran a kernel per layer and
 // direction with global round trips in between and one FP32 atomic per weight
-// and tile: 206 us per step of 8192 rows, 17 launches; now 33 us and 2.
+// and tile: 206 us per step of 8192 rows, 17 launches; now 29 us and 2.  Of the
+// shared memory wavefronts of this kernel half were bank conflicts before the
+// transposed tiles were padded (TR_LBO), and the partial gradients went out one
+// line per lane: 25.0 us then, 20.6 us now, 100 steps of 8192 rows 3.29 -> 2.90 ms.
 //
 // Rows past n (the last tile's) have zero activations and dy = 0.
 // x rows: row r of the pass is row (cur[0] + r) mod n_total of the data when
@@ -253,10 +270,13 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         __syncthreads();
         fence_after_sync();
     };
-    auto issue = [&](uint32_t d, __nv_bfloat16* a, __nv_bfloat16* b, int K, int N, bool acc) {
+    // operands by row (consecutive core matrices along K), or transposed (tr)
+    auto issue = [&](uint32_t d, __nv_bfloat16* a, bool a_tr, __nv_bfloat16* b, bool b_tr, int K, int N, bool acc) {
         const uint32_t idesc = instr_desc(TM, N), a0 = smem_u32(a), b0 = smem_u32(b);
+        const uint32_t al = a_tr ? TR_LBO : 128u, as = a_tr ? 128u : 16u * K;
+        const uint32_t bl = b_tr ? TR_LBO : 128u, bs = b_tr ? 128u : 16u * K;
         for (int j = 0; j < K / 16; j++)
-            mma_bf16(T0 + d, smem_desc(a0 + 256u * j, 128u, 16u * K), smem_desc(b0 + 256u * j, 128u, 16u * K), idesc,
+            mma_bf16(T0 + d, smem_desc(a0 + 2u * al * j, al, as), smem_desc(b0 + 2u * bl * j, bl, bs), idesc,
                      acc || j > 0);
     };
     auto end_mma = [&]() {   // every thread waits for the committed MMAs; uniform over the CTA
@@ -272,7 +292,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         float s = 0.0f;
 #pragma unroll
         for (int q = 0; q < 8; q++) {
-            const uint4 v = *reinterpret_cast<const uint4*>(at(S.zt, col, r0 + 8 * q, TM));
+            const uint4 v = *reinterpret_cast<const uint4*>(at_tr(S.zt, col, r0 + 8 * q));
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
             for (int z = 0; z < 4; z++) {
@@ -310,7 +330,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         cp_async_wait<2>();   // W0 (first tile)
         begin_mma();
         if (tid == 0) {
-            issue(D, S.x, S.w0, NIN, HID, false);
+            issue(D, S.x, false, S.w0, false, NIN, HID, false);
             mma_commit(&S.bar);
         }
         end_mma();
@@ -343,7 +363,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             else cp_async_wait<0>();              // W2 (and whatever was loaded behind it)
             begin_mma();
             if (tid == 0) {
-                issue(D, S.row, layer == 0 ? S.wa : S.wb, HID, HID, false);
+                issue(D, S.row, false, layer == 0 ? S.wa : S.wb, false, HID, HID, false);
                 mma_commit(&S.bar);
             }
             end_mma();
@@ -408,8 +428,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             else cp_async_wait<0>();              // W1^T
             begin_mma();
             if (tid == 0) {
-                issue(D, S.row, layer == 2 ? S.wa : S.wb, HID, HID, false);
-                issue(layer == 2 ? DW2 : DW1, S.zt, layer == 2 ? S.h1t : S.h0t, TM, HID, !first);
+                issue(D, S.row, false, layer == 2 ? S.wa : S.wb, false, HID, HID, false);
+                issue(layer == 2 ? DW2 : DW1, S.zt, true, layer == 2 ? S.h1t : S.h0t, true, TM, HID, !first);
                 mma_commit(&S.bar);
             }
             const float cs = col_sum(false);   // beside the MMAs: both only read zt
@@ -430,7 +450,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         }
         begin_mma();
         if (tid == 0) {
-            issue(DW0, S.zt, S.xt, TM, NIN, !first);
+            issue(DW0, S.zt, true, S.xt, false, TM, NIN, !first);
             mma_commit(&S.bar);
         }
         gb[0] += col_sum(false);
@@ -441,12 +461,17 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     if (GRAD) {
         // this CTA's partial gradient: the accumulators, then the column sums
         float* g = part + (long long)blockIdx.x * PSTRIDE;
+        // (through shared memory: a lane holds a row, so stores straight from
+        // the accumulators would touch 32 lines each)
+        constexpr int LD = HID + 4;
+        float* stage = reinterpret_cast<float*>(S.wa);   // wa, wb and row are free now
+        static_assert(TM * LD * sizeof(float) <= 3 * sizeof(S.wa), "stage");
         if (ok) {
 #pragma unroll 1
             for (int layer = 0; layer < 3; layer++) {
                 const int K = layer == 0 ? NIN : HID;
                 const uint32_t d = layer == 0 ? DW0 : (layer == 1 ? DW1 : DW2);
-                float* gw = g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2)) + (long long)m * K;
+                float* gw = g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2));
 #pragma unroll 1
                 for (int c = 0; c < 2; c++) {
                     const int c0 = K == HID ? 64 * half + 32 * c : 0;
@@ -455,9 +480,15 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
                     tmem_ld32(T0 + d + tlane + (uint32_t)c0, v);
 #pragma unroll
                     for (int q = 0; q < 8; q++)
-                        reinterpret_cast<float4*>(gw + c0)[q] =
+                        *reinterpret_cast<float4*>(stage + m * LD + c0 + 4 * q) =
                             make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                 }
+                __syncthreads();
+                const int per = K / 4;   // 16-byte words a row
+                for (int i = tid; i < HID * per; i += STEP_THREADS)
+                    reinterpret_cast<float4*>(gw)[i] =
+                        *reinterpret_cast<const float4*>(stage + (i / per) * LD + 4 * (i % per));
+                __syncthreads();
             }
         }
         const int col = tid & 127;
