@@ -226,10 +226,11 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 // SM: eight dependent MMA batches of about 0.1 us each and as many epilogues
 // through shared memory.  The form before this one ran a kernel per layer and
 // direction with global round trips in between and one FP32 atomic per weight
-// and tile: 206 us per step of 8192 rows, 17 launches; now 29 us and 2.  Of the
+// and tile: 206 us per step of 8192 rows, 17 launches; now 24 us and 2.  Of the
 // shared memory wavefronts of this kernel half were bank conflicts before the
 // transposed tiles were padded (TR_LBO), and the partial gradients went out one
-// line per lane: 25.0 us then, 20.6 us now, 100 steps of 8192 rows 3.29 -> 2.90 ms.
+// line per lane: 25.0 us then, 20.6 us now, 100 steps of 8192 rows 3.29 -> 2.90 ms (2.43 with
+// the launches overlapped, launch_step).
 //
 // Rows past n (the last tile's) have zero activations and dy = 0.
 // x rows: row r of the pass is row (cur[0] + r) mod n_total of the data when
@@ -237,8 +238,8 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 template <bool GRAD>
 __global__ void __launch_bounds__(STEP_THREADS, 1)
     k_mlp_step(const float* __restrict__ x, const float* __restrict__ t, long long n, int n_in, long long n_total,
-               long long* __restrict__ cur, const float* __restrict__ p, const __nv_bfloat16* __restrict__ img,
-               float* __restrict__ y, float* __restrict__ part, int* __restrict__ err) {
+               long long* __restrict__ cur, const float* p, const __nv_bfloat16* img, float* __restrict__ y,
+               float* __restrict__ part, int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -246,9 +247,15 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     const int m = 32 * quad + lane;                // this thread's row of the tile
     const uint32_t D = 0, DW2 = 128, DW1 = 256, DW0 = 384;   // TMEM columns
     const uint32_t tlane = (uint32_t)(32 * quad) << 16;
-    const long long base = cur ? cur[0] : 0;
     if (warp == 0) tmem_alloc(&S.tmem, 512);
     if (tid == 0) mbar_init(&S.bar, 1);
+    // In a training run the launches overlap (launch_step): the next k_adam may
+    // become resident now, and this CTA waits for the last one to end before it
+    // reads anything (p and img carry no __restrict__: their loads must not be
+    // taken for invariant and moved above the wait).
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    const long long base = cur ? cur[0] : 0;
     load_image(S.w0, img + IW0, HID * NIN);
     for (int k = tid; k < HID; k += STEP_THREADS) {
         S.bias[0][k] = p[OB0 + k];
@@ -549,7 +556,7 @@ __global__ void k_cast_weights(const float* __restrict__ p, __nv_bfloat16* __res
 // in order (only its result counts).  One thread summing all 64 waited for
 // memory most of its 9.6 us (6.5 now).
 constexpr int PGROUP = 8, PCOLS = 32;   // a block: 32 parameters x 8 groups
-__device__ __forceinline__ float part_sum(const float* __restrict__ part, int np, long long i) {
+__device__ __forceinline__ float part_sum(const float* part, int np, long long i) {
     __shared__ float sums[PGROUP][PCOLS];
     const int col = threadIdx.x % PCOLS, grp = threadIdx.x / PCOLS;
     float s = 0.0f;
@@ -579,10 +586,12 @@ __global__ void __launch_bounds__(PGROUP* PCOLS) k_grad_sum(const float* __restr
 // Adam step on the FP32 master parameters: the gradient summed from the
 // partials, step number cur[1] (bias corrections 1 - b^step), the BF16 tile
 // images of the new weights, and the next batch's first row.
-__global__ void __launch_bounds__(PGROUP* PCOLS) k_adam(float* __restrict__ p, const float* __restrict__ part, int np, float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ img,
-                       float* __restrict__ loss, float lr, float b1, float b2, float eps, long long* __restrict__ cur,
-                       long long b, long long n_total) {
+__global__ void __launch_bounds__(PGROUP* PCOLS)
+    k_adam(float* p, const float* part, int np, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
+           __nv_bfloat16* img, float* __restrict__ loss, float lr, float b1, float b2, float eps, long long* cur,
+           long long b, long long n_total) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();   // k_mlp_step's partials and cur[1]
     const long long i = part_param();
     const float gi = part_sum(part, np, i);
     if (threadIdx.x >= PCOLS) return;
@@ -663,16 +672,31 @@ rpd_status launch_check(rpd_mlp* q) {
 // Forward, and with t backward into the partial gradients.  With n_total > 0
 // the n rows are the training batch that starts at the device cursor's row of
 // the n_total data rows (x and t are the whole data).
-void run_step(rpd_mlp* q, const float* x, const float* t, long long n, float* y, long long n_total = 0) {
-    const int ctas = step_ctas(n);
-    long long* cur = n_total > 0 ? q->cur : nullptr;
-    if (t)
-        k_mlp_step<true><<<ctas, STEP_THREADS, step_smem(), q->stream>>>(x, t, n, q->n_in, n_total, cur, q->p, q->img,
-                                                                          y, q->part, q->err);
-    else
-        k_mlp_step<false><<<ctas, STEP_THREADS, step_smem(), q->stream>>>(x, t, n, q->n_in, n_total, cur, q->p, q->img,
-                                                                           y, q->part, q->err);
+// One kernel behind the last one of the stream; with overlap its CTAs may
+// become resident before that one has ended (programmatic dependent launch; the
+// kernel itself waits for the end), which takes the launch gap and the prologue
+// out of a run of dependent launches: 29.0 -> 24.3 us per training step.  Only for a kernel whose predecessor in the stream is one
+// of these too.
+template <class... P, class... A>
+void launch_step(rpd_mlp* q, void (*kernel)(P...), int blocks, int threads, size_t smem, bool overlap, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = q->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     note_launch();
+}
+
+void run_step(rpd_mlp* q, const float* x, const float* t, long long n, float* y, long long n_total = 0,
+              bool overlap = false) {
+    launch_step(q, t ? k_mlp_step<true> : k_mlp_step<false>, step_ctas(n), STEP_THREADS, step_smem(), overlap, x, t, n,
+                q->n_in, n_total, n_total > 0 ? q->cur : nullptr, q->p, q->img, y, q->part, q->err);
 }
 
 void cast_weights(rpd_mlp* q) {
@@ -790,11 +814,9 @@ rpd_status rpd_mlp_train(rpd_mlp* q, const float* d_x, const float* d_t, int64_t
         const long long c0[2] = {0, q->step};
         cudaMemcpyAsync(q->cur, c0, sizeof(c0), cudaMemcpyHostToDevice, q->stream);
         for (int it = 0; it < steps; it++) {
-            run_step(q, d_x, d_t, b, nullptr, n);
-            k_adam<<<nblk(NPARAM + 1, PCOLS), PGROUP * PCOLS, 0, q->stream>>>(q->p, q->part, step_ctas(b), q->g, q->m,
-                                                                              q->v, q->img, q->loss, lr, 0.9f, 0.999f,
-                                                                              1e-8f, q->cur, b, n);
-            note_launch();
+            run_step(q, d_x, d_t, b, nullptr, n, it > 0);
+            launch_step(q, k_adam, nblk(NPARAM + 1, PCOLS), PGROUP * PCOLS, 0, true, q->p, q->part, step_ctas(b), q->g,
+                        q->m, q->v, q->img, q->loss, lr, 0.9f, 0.999f, 1e-8f, q->cur, b, n);
         }
         q->step += steps;
     }
