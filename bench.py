@@ -49,10 +49,10 @@ PLANNED_FLOP_PER_PIECE = {16: 2500.0, 32: 4500.0}
 # 3x3 cofactors, 56 flop) plus its orientation test and stored bound (17).
 FLOP_SIGN_TEST = 7
 FLOP_NEW_VERTEX = (17, 26, 73)   # by m = 1, 2, 3
-# DRAM bytes (read + write) per step of the clip kernels (k_clip over all bins
-# + k_whole), from one ncu capture of the current kernels per workload and
+# DRAM bytes (read + write) per step of the clip kernels (k_clip over its bins,
+# k_clip2 and k_whole), from one ncu capture of the current kernels per workload and
 # precision; a workload missing here reports traffic null.
-CLIP_TRAFFIC_BYTES = {("blob_c3", "fp32"): 894.12e6}
+CLIP_TRAFFIC_BYTES = {("blob_c3", "fp32"): 915.0e6}
 # CPU legs per workload, sized for 10-30 s each on the 16 host cores: tets of
 # the brute-force oracle sample, of its 1-thread sample, fraction of tets for
 # the same-algorithm baseline, tets per step of the reference arm.
@@ -130,7 +130,7 @@ def clip_roofline(stage, k, workload, precision, peaks, hbm_gbs, stage64=None):
           (precision + "_executed"): flop_exec / (ms * 1e-3) / 1e12 / peak}
     if traffic is not None and hbm_gbs:
         fr["hbm"] = traffic / (ms * 1e-3) / 1e9 / hbm_gbs
-    out = {"kernel": "k_clip over all candidate-count bins + k_whole (side by side on the bin streams; "
+    out = {"kernel": "k_clip over its candidate-count bins + k_clip2 + k_whole (side by side on the bin streams; "
                      "timed to the end of the record kernels that follow them there)",
            "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
            "traffic": traffic, "flop_per_launch": flop_planned, "flop_per_piece": PLANNED_FLOP_PER_PIECE[kk],
@@ -449,8 +449,8 @@ def repair_leg(nshapes, stream, dev, seed=20240330):
                          "roofline": {"bound": "tensor", "achieved": mlp_tf, "unit": "TFLOP/s",
                                       "peak": bf16_peak, "frac": (mlp_tf / bf16_peak) if bf16_peak else None,
                                       "flop": gemm_flop,
-                                      "note": "tcgen05 BF16 GEMMs of 128-row tiles (one CTA each), 15 kernels "
-                                              "per step replayed from a CUDA graph; latency-bound at this batch"},
+                                      "note": "tcgen05 BF16 GEMMs of 128-row tiles (one CTA each), two kernels "
+                                              "per step, forward and backward fused; latency-bound at this batch"},
                          "setup_s": time.perf_counter() - t0},
             **summary}
 

@@ -138,15 +138,15 @@ rpd_status rpd_build(const double* d_verts, int64_t nv, const int32_t* d_tets, i
  * ...) and spheres [h_sphere_off[s], ...) (HOST i64[nshapes + 1] prefix
  * offsets from 0); tets hold GLOBAL vertex indices, each inside its own shape
  * (RPD_E_INVALID otherwise).  Every stage runs once over the union: the
- * neighbour search walks one sphere grid per shape, so a tet sees only its
+ * candidate search lays out one sphere tree per shape, so a tet sees only its
  * own shape's spheres, and the pairs of all shapes are binned together by
  * candidate count, so shapes of uneven size share the launches.  Results use
  * global tet and sphere ids; shape s's rows of every table are contiguous
  * (rpd_batch_offsets) and equal those of rpd_build on shape s alone with its
  * ids shifted by its offsets.
  * Limits: fewer than 2^21 spheres in all (RPV keys, as for rpd_build, need
- * fewer than 2^16), at most 5600 per shape (one grid of 2 n_s + 64 cells in
- * shared memory), shapes of >= 4 vertices, 1 tet and 1 sphere; no
+ * fewer than 2^16), at most 5600 per shape (the debug neighbour search
+ * keeps one grid of 2 n_s + 64 cells in shared memory), shapes of >= 4 vertices, 1 tet and 1 sphere; no
  * rpd_insert (and so no repair loop) on a batch context.
  * Synchronises like rpd_build.
  */
@@ -424,9 +424,8 @@ rpd_status rpd_mlp_grad(rpd_mlp* mlp, const float* d_x, const float* d_t, int64_
 /* `steps` Adam steps with learning rate lr on consecutive batches of `batch`
  * rows (row r of a batch is row (start + r) mod n, each batch starting where
  * the last ended; shuffle the rows beforehand); *h_loss = the last step's
- * loss.  The batch rows are chosen on the device, so one step's launches are
- * captured once as a CUDA graph on the network's private stream and replayed
- * `steps` times. */
+ * loss.  Two launches a step on the network's stream; the batch rows are
+ * chosen on the device. */
 rpd_status rpd_mlp_train(rpd_mlp* mlp, const float* d_x, const float* d_t, int64_t n, int32_t steps, int32_t batch,
                          float lr, float* h_loss);
 void rpd_mlp_destroy(rpd_mlp* mlp);

@@ -2,8 +2,8 @@
 // a time).  The shapes' vertices, tets and spheres are concatenated; every
 // stage runs once over the union (one launch per stage, the pairs of all
 // shapes binned together by candidate count), and a tet sees only the
-// spheres of its own shape because the neighbour search walks a grid per
-// shape (knn.cu).  These kernels check that no tet reaches into another
+// spheres of its own shape because the candidate search lays out a tree per
+// shape (cand.cu).  These kernels check that no tet reaches into another
 // shape and cut the sorted result tables into per-shape ranges.
 #include <cuda_runtime.h>
 #include <stdint.h>
