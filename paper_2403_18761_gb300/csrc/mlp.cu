@@ -172,7 +172,7 @@ struct StepSmem {
     __nv_bfloat16 row[TM * HID];                  // the A operand: H0, H1, dZ2, dZ1 by row
     __nv_bfloat16 h0t[TR_ELEMS], h1t[TR_ELEMS];   // transposed activations (weight gradients' B operand)
     __nv_bfloat16 zt[TR_ELEMS];                   // H2, then dZ2, dZ1, dZ0, transposed (their A operand)
-    float bias[3][HID], w3[HID], ypart[2][TM], dy[TM], red[HID], lred[4];
+    float bias[3][HID], w3[HID], dy[TM], red[HID], lred[4];
     uint64_t bar;
     uint32_t tmem;
 };
@@ -304,8 +304,12 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
 #pragma unroll
             for (int z = 0; z < 4; z++) {
                 const float2 f = __bfloat1622float2(h[z]);
-                if (weighted) s += f.x * S.dy[r0 + 8 * q + 2 * z] + f.y * S.dy[r0 + 8 * q + 2 * z + 1];
-                else s += f.x + f.y;
+                if (weighted) {
+                    s += __fmul_rn(f.x, S.dy[r0 + 8 * q + 2 * z]);
+                    s += __fmul_rn(f.y, S.dy[r0 + 8 * q + 2 * z + 1]);
+                } else {
+                    s += f.x + f.y;
+                }
             }
         }
         return s;
@@ -376,8 +380,13 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             end_mma();
         }
         if (GRAD) load_image(S.wa, img + IW2T, HID * HID);   // W1 has been consumed
-        // layer 2 and the head
-        float ys = 0.0f;
+        // layer 2 and the head: the products with w3 in groups of four columns,
+        // by row in the place of the consumed A operand, then added across the
+        // groups 16, 8, 4, 2 and 1 apart.  The order is part of the result: dy's
+        // last bit decides how dZ2 rounds to BF16, and another order moved the
+        // gradients by 4e-5 in norm, where their own FP32 sums are good to 2e-7
+        float* heads = reinterpret_cast<float*>(S.row);   // [32 groups][TM]
+        static_assert(32 * TM * sizeof(float) <= sizeof(S.row), "heads");
 #pragma unroll 1
         for (int c = 0; c < 2; c++) {
             const int c0 = 64 * half + 32 * c;
@@ -388,18 +397,30 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
 #pragma unroll
             for (int k = 0; k < 32; k++) {
                 o[k] = __float2bfloat16(live ? fmaxf(v[k] + S.bias[2][c0 + k], 0.0f) : 0.0f);
-                const float h = __bfloat162float(o[k]);
-                mk |= (h > 0.0f ? 1u : 0u) << k;
-                ys += h * S.w3[c0 + k];
+                v[k] = __bfloat162float(o[k]);
+                mk |= (v[k] > 0.0f ? 1u : 0u) << k;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                float s = __fmul_rn(v[4 * q], S.w3[c0 + 4 * q]);
+#pragma unroll
+                for (int z = 1; z < 4; z++) s = __fmaf_rn(v[4 * q + z], S.w3[c0 + 4 * q + z], s);
+                heads[(c0 / 4 + q) * TM + m] = s;
             }
             S.mask[2][c][tid] = mk;
             if (GRAD) put_tile(nullptr, S.zt, m, c0, o);
         }
-        S.ypart[half][m] = ys;
         if (GRAD) load_image(S.wb, img + IW1T, HID * HID);   // W2 has been consumed
         __syncthreads();
         if (half == 0) {
-            const float yr = S.ypart[0][m] + S.ypart[1][m] + b3;
+            float s[16];
+#pragma unroll
+            for (int q = 0; q < 16; q++) s[q] = heads[q * TM + m] + heads[(q + 16) * TM + m];
+#pragma unroll
+            for (int off = 8; off; off >>= 1)
+#pragma unroll
+                for (int q = 0; q < off; q++) s[q] += s[q + off];
+            const float yr = s[0] + b3;
             if (y && live) y[m0 + m] = yr;
             if (GRAD) {
                 long long src = m0 + m;
@@ -412,7 +433,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             }
         }
         if (!GRAD) {
-            __syncthreads();   // ypart and the operands are rewritten by the next tile
+            __syncthreads();   // the operands are rewritten by the next tile
             continue;
         }
         __syncthreads();
