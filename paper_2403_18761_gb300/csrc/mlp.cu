@@ -217,10 +217,10 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 // by row (the next GEMM's A operand) and, with GRAD, transposed (the weight
 // gradient's B operand).  The head (w3, b3) runs on the CUDA cores.  Backward:
 // dZ2 from the head's gradient and the ReLU mask; then per layer one batch of
-// MMAs computes the weight gradient, accumulated in TMEM over all of the CTA's
-// tiles, and the input gradient, whose epilogue masks it into the next dZ.
-// At the end every CTA writes its own partial gradient, which k_adam sums in
-// order: no atomics.
+// MMAs computes the tile's weight gradient, in an accumulator of its own, and the
+// input gradient, whose epilogue masks it into the next dZ.  Every CTA adds
+// its tiles' weight gradients up in its own partial gradient, which k_adam sums
+// in order: no atomics.
 //
 // What bounds it: latency.  A training batch of 8192 rows is 64 tiles, one per
 // SM: eight dependent MMA batches of about 0.1 us each and as many epilogues
@@ -278,13 +278,13 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         fence_after_sync();
     };
     // operands by row (consecutive core matrices along K), or transposed (tr)
-    auto issue = [&](uint32_t d, __nv_bfloat16* a, bool a_tr, __nv_bfloat16* b, bool b_tr, int K, int N, bool acc) {
+    auto issue = [&](uint32_t d, __nv_bfloat16* a, bool a_tr, __nv_bfloat16* b, bool b_tr, int K, int N) {
         const uint32_t idesc = instr_desc(TM, N), a0 = smem_u32(a), b0 = smem_u32(b);
         const uint32_t al = a_tr ? TR_LBO : 128u, as = a_tr ? 128u : 16u * K;
         const uint32_t bl = b_tr ? TR_LBO : 128u, bs = b_tr ? 128u : 16u * K;
         for (int j = 0; j < K / 16; j++)
             mma_bf16(T0 + d, smem_desc(a0 + 2u * al * j, al, as), smem_desc(b0 + 2u * bl * j, bl, bs), idesc,
-                     acc || j > 0);
+                     j > 0);
     };
     auto end_mma = [&]() {   // every thread waits for the committed MMAs; uniform over the CTA
         const bool done = mbar_wait(&S.bar, phase);
@@ -314,8 +314,48 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         }
         return s;
     };
+    // The tile's weight gradients into this CTA's partial gradient, which the
+    // first tile sets.  FP32 additions, not more MMAs into the same accumulators:
+    // those round towards zero, and over the 103 tiles of a CTA at 2 M rows left
+    // W0's gradient 2.2e-5 off in norm (1.8e-6 so, 2.7e-6 with FP32 atomics; 1.33 ->
+    // 2.21 ms a step there, nothing where a CTA has one tile).  Through shared
+    // memory: a lane holds a row, so stores straight from the accumulators would
+    // touch 32 lines each.
+    auto add_weights = [&](bool set) {
+        constexpr int LD = HID + 4;
+        float* stage = reinterpret_cast<float*>(S.wa);   // wa, wb and row are free now
+        static_assert(TM * LD * sizeof(float) <= 3 * sizeof(S.wa), "stage");
+        float* g = part + (long long)blockIdx.x * PSTRIDE;
+#pragma unroll 1
+        for (int layer = 0; layer < 3; layer++) {
+            const int K = layer == 0 ? NIN : HID;
+            const uint32_t d = layer == 0 ? DW0 : (layer == 1 ? DW1 : DW2);
+            float4* gw = reinterpret_cast<float4*>(g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2)));
+#pragma unroll 1
+            for (int c = 0; c < 2; c++) {
+                const int c0 = K == HID ? 64 * half + 32 * c : 0;
+                if (K == NIN && (half || c)) continue;   // warp-uniform
+                float v[32];
+                tmem_ld32(T0 + d + tlane + (uint32_t)c0, v);
+#pragma unroll
+                for (int q = 0; q < 8; q++)
+                    *reinterpret_cast<float4*>(stage + m * LD + c0 + 4 * q) =
+                        make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            }
+            __syncthreads();
+            const int per = K / 4;   // 16-byte words a row
+            for (int i = tid; i < HID * per; i += STEP_THREADS) {
+                float4 w = *reinterpret_cast<const float4*>(stage + (i / per) * LD + 4 * (i % per));
+                if (!set) {   // (the same thread's word of the last tile)
+                    const float4 o = gw[i];
+                    w = make_float4(o.x + w.x, o.y + w.y, o.z + w.z, o.w + w.w);
+                }
+                gw[i] = w;
+            }
+            __syncthreads();
+        }
+    };
     const long long ntile = (n + TM - 1) / TM;
-    bool first = true;
     for (long long tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x) {
         const long long m0 = tile * TM;
         load_image(S.wa, img + IW1, HID * HID);
@@ -341,7 +381,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         cp_async_wait<2>();   // W0 (first tile)
         begin_mma();
         if (tid == 0) {
-            issue(D, S.x, false, S.w0, false, NIN, HID, false);
+            issue(D, S.x, false, S.w0, false, NIN, HID);
             mma_commit(&S.bar);
         }
         end_mma();
@@ -374,7 +414,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             else cp_async_wait<0>();              // W2 (and whatever was loaded behind it)
             begin_mma();
             if (tid == 0) {
-                issue(D, S.row, false, layer == 0 ? S.wa : S.wb, false, HID, HID, false);
+                issue(D, S.row, false, layer == 0 ? S.wa : S.wb, false, HID, HID);
                 mma_commit(&S.bar);
             }
             end_mma();
@@ -456,8 +496,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             else cp_async_wait<0>();              // W1^T
             begin_mma();
             if (tid == 0) {
-                issue(D, S.row, false, layer == 2 ? S.wa : S.wb, false, HID, HID, false);
-                issue(layer == 2 ? DW2 : DW1, S.zt, true, layer == 2 ? S.h1t : S.h0t, true, TM, HID, !first);
+                issue(D, S.row, false, layer == 2 ? S.wa : S.wb, false, HID, HID);
+                issue(layer == 2 ? DW2 : DW1, S.zt, true, layer == 2 ? S.h1t : S.h0t, true, TM, HID);
                 mma_commit(&S.bar);
             }
             const float cs = col_sum(false);   // beside the MMAs: both only read zt
@@ -478,47 +518,17 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         }
         begin_mma();
         if (tid == 0) {
-            issue(DW0, S.zt, true, S.xt, false, TM, NIN, !first);
+            issue(DW0, S.zt, true, S.xt, false, TM, NIN);
             mma_commit(&S.bar);
         }
         gb[0] += col_sum(false);
         end_mma();
-        first = false;
+        if (ok) add_weights(blockIdx.x == tile);
     }
     cp_async_wait<0>();
     if (GRAD) {
-        // this CTA's partial gradient: the accumulators, then the column sums
+        // the column sums of this CTA's partial gradient
         float* g = part + (long long)blockIdx.x * PSTRIDE;
-        // (through shared memory: a lane holds a row, so stores straight from
-        // the accumulators would touch 32 lines each)
-        constexpr int LD = HID + 4;
-        float* stage = reinterpret_cast<float*>(S.wa);   // wa, wb and row are free now
-        static_assert(TM * LD * sizeof(float) <= 3 * sizeof(S.wa), "stage");
-        if (ok) {
-#pragma unroll 1
-            for (int layer = 0; layer < 3; layer++) {
-                const int K = layer == 0 ? NIN : HID;
-                const uint32_t d = layer == 0 ? DW0 : (layer == 1 ? DW1 : DW2);
-                float* gw = g + (layer == 0 ? OW0 : (layer == 1 ? OW1 : OW2));
-#pragma unroll 1
-                for (int c = 0; c < 2; c++) {
-                    const int c0 = K == HID ? 64 * half + 32 * c : 0;
-                    if (K == NIN && (half || c)) continue;   // warp-uniform
-                    float v[32];
-                    tmem_ld32(T0 + d + tlane + (uint32_t)c0, v);
-#pragma unroll
-                    for (int q = 0; q < 8; q++)
-                        *reinterpret_cast<float4*>(stage + m * LD + c0 + 4 * q) =
-                            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                }
-                __syncthreads();
-                const int per = K / 4;   // 16-byte words a row
-                for (int i = tid; i < HID * per; i += STEP_THREADS)
-                    reinterpret_cast<float4*>(gw)[i] =
-                        *reinterpret_cast<const float4*>(stage + (i / per) * LD + 4 * (i % per));
-                __syncthreads();
-            }
-        }
         const int col = tid & 127;
         const float sums[4] = {gb[0], gb[1], gb[2], gw3};
         const long long to[4] = {OB0, OB1, OB2, OW3};
