@@ -238,8 +238,7 @@ __device__ __forceinline__ void put_tile(__nv_bfloat16* row, __nv_bfloat16* tr, 
 template <bool GRAD>
 __global__ void __launch_bounds__(STEP_THREADS, 1)
     k_mlp_step(const float* __restrict__ x, const float* __restrict__ t, long long n, int n_in, long long n_total,
-               long long* __restrict__ cur, const float* p, const __nv_bfloat16* img, float* __restrict__ y,
-               float* __restrict__ part, int* __restrict__ err) {
+               long long* cur, const float* p, const __nv_bfloat16* img, float* __restrict__ y, float* part, int* err) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -251,8 +250,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     if (tid == 0) mbar_init(&S.bar, 1);
     // In a training run the launches overlap (launch_step): the next k_adam may
     // become resident now, and this CTA waits for the last one to end before it
-    // reads anything (p and img carry no __restrict__: their loads must not be
-    // taken for invariant and moved above the wait).
+    // reads or writes anything.  No pointer to what either of the two kernels
+    // writes (cur, p, img, part, err here; in k_adam also g, m, v and loss) may
+    // carry __restrict__: it would allow loads and stores to be moved above the
+    // wait.
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
     const long long base = cur ? cur[0] : 0;
@@ -618,11 +619,12 @@ __global__ void __launch_bounds__(PGROUP* PCOLS) k_grad_sum(const float* __restr
 // partials, step number cur[1] (bias corrections 1 - b^step), the BF16 tile
 // images of the new weights, and the next batch's first row.
 __global__ void __launch_bounds__(PGROUP* PCOLS)
-    k_adam(float* p, const float* part, int np, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-           __nv_bfloat16* img, float* __restrict__ loss, float lr, float b1, float b2, float eps, long long* cur,
-           long long b, long long n_total) {
+    k_adam(float* p, const float* part, int np, float* g, float* m, float* v, __nv_bfloat16* img, float* loss, float lr,
+           float b1, float b2, float eps, long long* cur, long long b, long long n_total) {
     cudaTriggerProgrammaticLaunchCompletion();
-    cudaGridDependencySynchronize();   // k_mlp_step's partials and cur[1]
+    // k_mlp_step's partials and cur[1], and through it the last k_adam's m, v and
+    // cur[0] (no __restrict__ on any of them, see k_mlp_step)
+    cudaGridDependencySynchronize();
     const long long i = part_param();
     const float gi = part_sum(part, np, i);
     if (threadIdx.x >= PCOLS) return;
