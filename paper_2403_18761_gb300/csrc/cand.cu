@@ -445,8 +445,9 @@ __global__ void __launch_bounds__(32 * WARPS) k_vertex_owners(CandArgs A, int32_
         __syncwarp();
         const int nt = __popc(m);
         for (int u = sub; u < nt; u += 4) test(list[u]);
-        dv = nearest();   // (the shuffles also end the reads of the list)
+        dv = nearest();
         R = warp_max(in ? dv : LLONG_MIN);
+        __syncwarp();   // the list has been read before the next leaf's is written (shuffles order no memory)
     });
     // the nearest over the four lanes; two lanes as near: a tie
 #pragma unroll
