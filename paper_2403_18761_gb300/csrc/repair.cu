@@ -511,7 +511,10 @@ __global__ void __launch_bounds__(32 * NW) k_shrink(const double* __restrict__ t
                 far = fminf(far, sqrtf(fx * fx + fy * fy + fz * fz) * (1.0f + 0x1p-18f) + cslack);
             }
             tighten(far);
-            if (NW > 1) __syncthreads();   // every warp starts from the best
+            if (NW > 1) {   // every warp starts from the best
+                __syncthreads();
+                ub = fminf(ub, __uint_as_float(*(volatile unsigned*)&ub_s));
+            }
         }
         double bd = INFINITY, bq[3] = {0, 0, 0};
         int bi = -1, cnt = 0;
