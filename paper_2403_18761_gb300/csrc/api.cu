@@ -1233,6 +1233,7 @@ static rpd_status ensure_boundary(rpd_ctx* c, double** tri, int32_t** face_of) {
         int32_t* f = c->alloc<int32_t>(nb + 1);
         if (!t || !f) return fail(c, RPD_E_OOM, "device allocation failed");
         launch_boundary_fill(c->tets, c->adj, c->Xi, c->nt, pos, ldexp(1.0, -c->opt.grid_bits), t, f, s);
+        record(c, 7);   // for an index that is built beside a capture (ensure_shrink_index)
         TRY(cuda_check(c, "boundary launch"));
         c->btri = t;
         c->btri_face = f;
@@ -1243,13 +1244,40 @@ static rpd_status ensure_boundary(rpd_ctx* c, double** tri, int32_t** face_of) {
     return RPD_OK;
 }
 
+// Calls that a stream capture of any thread would forbid are allowed in this
+// thread for as long as it lives.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The shrinking's search structure over the boundary triangles, built on
-// first use.
+// first use.  When that is a shrinking under capture, the index is built at
+// once on the library's stream: captured, its memory would exist only in the
+// graph's replays, and the context would keep pointers to it.
 static rpd_status ensure_shrink_index(rpd_ctx* c, double** tri) {
     int32_t* face_of = nullptr;
     TRY(ensure_boundary(c, tri, &face_of));
     if (c->shrink_index.order || c->nbtri == 0) return RPD_OK;
     const long long nb = c->nbtri, ng = (nb + 31) / 32;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, RPD_E_CUDA, "CUDA error before the shrink index");
+    }
+    RelaxedCapture relaxed;
+    struct Aside {   // the context's stream while the index is built
+        rpd_ctx* c;
+        cudaStream_t own;
+        ~Aside() { c->stream = own; }
+    } aside{c, c->stream};
+    if (cap != cudaStreamCaptureStatusNone) {
+        BinStreams* bs = bin_streams();
+        if (!bs) return fail(c, RPD_E_CUDA, "stream creation failed");
+        c->stream = bs->util;
+        cudaStreamWaitEvent(c->stream, c->ev[7], 0);   // the boundary triangles
+    }
     ShrinkIndex S;
     S.order = c->alloc<uint32_t>(nb);
     S.ball = c->alloc<float4>(nb);
@@ -1261,6 +1289,10 @@ static rpd_status ensure_shrink_index(rpd_ctx* c, double** tri) {
         return fail(c, RPD_E_OOM, "device allocation failed");
     launch_shrink_index(*tri, face_of, nb, c->Xi, c->nv, ldexp(1.0, -c->opt.grid_bits), S, tmp, c->stream);
     TRY(cuda_check(c, "shrink index launch"));
+    if (cap != cudaStreamCaptureStatusNone && cudaStreamSynchronize(c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, RPD_E_CUDA, "CUDA error in the shrink index");
+    }
     c->shrink_index = S;
     return RPD_OK;
 }
