@@ -145,9 +145,10 @@ rpd_status rpd_build(const double* d_verts, int64_t nv, const int32_t* d_tets, i
  * (rpd_batch_offsets) and equal those of rpd_build on shape s alone with its
  * ids shifted by its offsets.
  * Limits: fewer than 2^21 spheres in all (RPV keys, as for rpd_build, need
- * fewer than 2^16), at most 5600 per shape (the debug neighbour search
- * keeps one grid of 2 n_s + 64 cells in shared memory), shapes of >= 4 vertices, 1 tet and 1 sphere; no
- * rpd_insert (and so no repair loop) on a batch context.
+ * fewer than 2^16), at most 5600 per shape (a limit of this interface, no
+ * longer of the search behind it; larger shapes go through rpd_build), shapes
+ * of >= 4 vertices, 1 tet and 1 sphere; no debug bit 4; no rpd_insert (and so
+ * no repair loop) on a batch context.
  * Synchronises like rpd_build.
  */
 rpd_status rpd_build_batch(const double* d_verts, const int32_t* d_tets, const double* d_centers,

@@ -219,11 +219,10 @@ struct rpd_ctx {
     long long nbtri = -1;
     ShrinkIndex shrink_index;   // their search structure (built with the first shrinking)
     // batches (rpd_build_batch): shape offsets of vertices, tets and spheres
-    // (device copies and the host's), and the largest per-shape grid
+    // (device copies and the host's)
     int nshapes = 1;
     long long *d_voff = nullptr, *d_toff = nullptr, *d_soff = nullptr;
     std::vector<long long> h_voff, h_toff, h_soff;
-    long long max_shape_ncap = 0;
     CandPlan plan;   // the candidate stage's blocks and cells
     // mesh bounding box (world units), computed on first use
     bool have_bbox = false;
@@ -494,6 +493,8 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old);
 // packets (cand.cu): only when a debug bit asks for that form.
 bool per_vertex_lists(const rpd_ctx* c) { return (c->opt.debug_checks & 4) != 0; }
 
+constexpr long long BATCH_SPHERES = 5600;   // spheres of a batch's shape at most (include/rpd.h)
+
 // Device, timing events and side streams of a context; the chunk for every
 // buffer sized before the pair count is known.
 rpd_status begin(rpd_ctx* c) {
@@ -508,12 +509,12 @@ rpd_status begin(rpd_ctx* c) {
     record(c, 0);
     const long long ncap = 2 * ns + 64, pcap = 4 * nt + 1024;
     size_t est = sizeof(DevState) + 4 * 3 * (nv + ns) + 8 * ns + 4 * 4 * nt + 4 * nt + 4 * 4 * nt +
-                 prep_tmp_bytes(nt, nv) + sizeof(GridParams) + 8 * (ncap + 1) + 4 * ns + 8 * 2 * ncap +
-                 grid_tmp_bytes(ns, ncap) + 16 * ns + 8 * ns + 4 * nt + (4 + 1) * nt * RPD_MAXC + 4 * nt + 4 +
+                 prep_tmp_bytes(nt, nv) + 4 * nt + (4 + 1) * nt * RPD_MAXC + 4 * nt + 4 +
                  8 * (nt + 1) + scan_tmp_bytes(nt + 1) + 8 * RPD_NBINS + 8 * pcap + 8 * (3 + RPD_NBINS) + nt + 8 +
                  42 * 256;
     if (per_vertex_lists(c)) {
-        est += 4 * nv * c->K + 8 * nv + knn_tmp_bytes(nv);
+        est += sizeof(GridParams) + 8 * (ncap + 1) + 4 * ns + 8 * 2 * ncap + grid_tmp_bytes(ns, ncap) + 16 * ns + 8 * ns +
+               4 * nv * c->K + 8 * nv + knn_tmp_bytes(nv);
     } else {
         cand_plan(c->h_voff.data(), c->h_toff.data(), c->h_soff.data(), c->nshapes, nv, nt, ns, c->plan);
         est += cand_tmp_bytes(c->plan, nt, nv, ns);
@@ -605,38 +606,27 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     const long long nv = c->nv, nt = c->nt, ns = c->ns;
     BinStreams* bs = bin_streams();
     // ---- A1
-    // one grid (2 ns + 64 cells), or one per shape of a batch (2 n_s + 64
-    // cells and an end offset each, laid end to end)
-    const bool batch = c->nshapes > 1;
-    long long ncap = batch ? 2 * ns + 65ll * c->nshapes : 2 * ns + 64;
-    const bool lists = per_vertex_lists(c);
-    int4* cell_sph = nullptr;
-    long long* cell_w = nullptr;
+    const long long ncap = 2 * ns + 64;       // cells of the sphere grid
+    const bool lists = per_vertex_lists(c);   // one shape: batches refuse the debug bit
+    int32_t* knn = nullptr;
+    long long* dplus = nullptr;
     if (lists) {
-        c->gp = c->alloc<GridParams>(c->nshapes);
+        c->gp = c->alloc<GridParams>(1);
         c->cell_start = c->alloc<int64_t>(ncap + 1);
         c->cell_ids = c->alloc<int32_t>(ns);
         c->cell_wmax = c->alloc<long long>(2 * ncap);
         void* gtmp = c->alloc<char>(grid_tmp_bytes(ns, ncap));
-        cell_sph = c->alloc<int4>(ns);
-        cell_w = c->alloc<long long>(ns);
+        int4* cell_sph = c->alloc<int4>(ns);
+        long long* cell_w = c->alloc<long long>(ns);
         NEED(c->gp && c->cell_start && c->cell_ids && c->cell_wmax && gtmp && cell_sph && cell_w);
-        if (batch)
-            launch_sphere_grid_batch(c->Ci, c->W, c->d_soff, c->nshapes, ncap, c->gp, c->cell_start, c->cell_ids,
-                                     cell_sph, cell_w, c->cell_wmax, c->max_shape_ncap, s);
-        else
-            launch_sphere_grid(c->Ci, c->W, ns, ncap, c->gp, c->cell_start, c->cell_ids, cell_sph, cell_w,
-                               c->cell_wmax, gtmp, s);
-    }
-    int32_t* knn = nullptr;
-    long long* dplus = nullptr;
-    if (lists) {
+        launch_sphere_grid(c->Ci, c->W, ns, ncap, c->gp, c->cell_start, c->cell_ids, cell_sph, cell_w, c->cell_wmax,
+                           gtmp, s);
         knn = c->alloc<int32_t>(nv * c->K);
         dplus = c->alloc<long long>(nv);
         void* ktmp = c->alloc<char>(knn_tmp_bytes(nv));
         NEED(knn && dplus && ktmp);
         launch_knn(c->Xi, nv, ns, c->gp, c->cell_start, cell_sph, cell_w, c->cell_wmax, ncap, c->K, knn, dplus, ktmp,
-                   &c->st->err, true, s, c->d_voff, c->nshapes);
+                   &c->st->err, true, s);
     }
     TRY(cuda_check(c, "neighbour launch"));
     record(c, 3);
@@ -656,8 +646,7 @@ rpd_status build_rest(rpd_ctx* c, rpd_ctx* old) {
     c->qcount = bc.qcount;
     if (lists) {
         launch_candidates(c->tets, nt, nv, c->Xi, c->Ci, c->W, knn, dplus, c->K, c->gp, c->cell_start, c->cell_ids,
-                          c->cell_wmax, c->cand_cnt, c->cand, c->cand_ord, c->fb_list, c->fb_count, c->st, s,
-                          c->d_voff, c->nshapes);
+                          c->cell_wmax, c->cand_cnt, c->cand, c->cand_ord, c->fb_list, c->fb_count, c->st, s);
     } else {
         void* ctmp = c->alloc<char>(cand_tmp_bytes(c->plan, nt, nv, ns));
         NEED(ctmp);
@@ -991,20 +980,20 @@ rpd_status rpd_build_batch(const double* d_verts, const int32_t* d_tets, const d
     if (nshapes < 1 || nshapes > (1 << 20)) return reject("nshapes must be in [1, 2^20]");
     if (!h_vert_off || !h_tet_off || !h_sphere_off) return reject("null offset array");
     if (h_vert_off[0] != 0 || h_tet_off[0] != 0 || h_sphere_off[0] != 0) return reject("offsets must start at 0");
-    long long max_ncap = 0;
+    long long max_ns = 0;
     for (int s = 0; s < nshapes; s++) {
         const long long nv_s = h_vert_off[s + 1] - h_vert_off[s], nt_s = h_tet_off[s + 1] - h_tet_off[s],
                         ns_s = h_sphere_off[s + 1] - h_sphere_off[s];
         if (nv_s < 4 || nt_s < 1 || ns_s < 1) return reject("every shape needs >= 4 vertices, a tet and a sphere");
-        max_ncap = std::max(max_ncap, 2 * ns_s + 64);
+        max_ns = std::max(max_ns, ns_s);
     }
-    if (max_ncap > batch_grid_cap()) return reject("a shape of a batch has more spheres than its grid takes");
+    if (max_ns > BATCH_SPHERES) return reject("a shape of a batch has more than 5600 spheres");
     const long long nv = h_vert_off[nshapes], nt = h_tet_off[nshapes], ns = h_sphere_off[nshapes];
     if (ns >= (1ll << 21)) return reject("a batch holds fewer than 2^21 spheres");
     rpd_options o;
     rpd_default_options(&o);
     if (opt) o = *opt;
-    if (o.debug_checks & 4) return reject("the tiled neighbour search does not take batches");
+    if (o.debug_checks & 4) return reject("the per-vertex neighbour lists do not take batches");
     if (nshapes == 1) return rpd_build(d_verts, nv, d_tets, nt, d_centers, d_radii, ns, &o, cuda_stream, out);
     if (nv >= (1ll << 21)) return reject("nv must be < 2^21");
     if (nt >= (1ll << 31) / RPD_MAXC) return reject("nt must be < 2^26");
@@ -1024,7 +1013,6 @@ rpd_status rpd_build_batch(const double* d_verts, const int32_t* d_tets, const d
     c->h_voff.assign(h_vert_off, h_vert_off + nshapes + 1);
     c->h_toff.assign(h_tet_off, h_tet_off + nshapes + 1);
     c->h_soff.assign(h_sphere_off, h_sphere_off + nshapes + 1);
-    c->max_shape_ncap = max_ncap;
     rpd_status st = build(c, d_verts, d_tets, d_centers, d_radii);
     if (st != RPD_OK) {
         g_build_error = c->last_error.empty() ? "build failed" : c->last_error;

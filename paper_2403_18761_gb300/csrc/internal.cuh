@@ -13,8 +13,6 @@ struct GridParams {
     int3 dim;          // cells per axis
     int ncell;
     long long wmax;    // largest power weight r^2
-    long long cbase;   // offset of this grid's cells in the cell arrays (batches: one grid per shape)
-    long long sbase;   // id of the grid's first sphere (its slots hold ids relative to it)
 };
 
 // ---------------------------------------------------------------- prep.cu
@@ -44,27 +42,14 @@ void launch_sphere_grid(const int32_t* Ci, const long long* W, long long ns, lon
 size_t knn_tmp_bytes(long long nv);
 void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams* gp, const int64_t* cell_start,
                 const int4* cell_sph, const long long* cell_w, const long long* cell_wmax, long long ncap, int K,
-                int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s,
-                const long long* voff = nullptr, int nshapes = 1);
-// Batches: one grid per shape, all built by one launch (a block per shape).
-// Shape s owns spheres [soff[s], soff[s + 1]) (device array) and cells
-// [2 soff[s] + 65 s, 2 soff[s + 1] + 65 (s + 1)) of cell_start (its
-// 2 n_s + 64 cells and one end offset) and of both halves of cell_wmax
-// (cell maxima, then row maxima at + ncap_total).  Every shape needs
-// 2 n_s + 64 <= batch_grid_cap() cells.
-long long batch_grid_cap();
-void launch_sphere_grid_batch(const int32_t* Ci, const long long* W, const long long* soff, int nshapes,
-                              long long ncap_total, GridParams* gp, int64_t* cell_start, int32_t* cell_ids,
-                              int4* cell_sph, long long* cell_w, long long* cell_wmax, long long max_shape_ncap,
-                              cudaStream_t s);
+                int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s);
 // Candidate spheres of every tet (superset of the spheres whose cell meets
 // the tet with positive volume), sorted by index, at most RPD_MAXC.
 void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const int32_t* Xi, const int32_t* Ci,
                        const long long* W, const int32_t* knn, const long long* dplus, int K,
                        const GridParams* gp, const int64_t* cell_start, const int32_t* cell_ids,
                        const long long* cell_wmax, int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord,
-                       int32_t* fb_list, int32_t* fb_count, DevState* st, cudaStream_t s,
-                       const long long* voff = nullptr, int nshapes = 1);
+                       int32_t* fb_list, int32_t* fb_count, DevState* st, cudaStream_t s);
 
 // ---------------------------------------------------------------- cand.cu
 // A shape's ranges of vertices, tets and spheres, its first vertex and tet

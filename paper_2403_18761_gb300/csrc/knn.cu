@@ -87,8 +87,6 @@ __device__ GridParams grid_params(const int* mn, const int* mx, long long wm, lo
     g.dim = make_int3((int)d[0], (int)d[1], (int)d[2]);
     g.ncell = (int)(d[0] * d[1] * d[2]);
     g.wmax = wm;
-    g.cbase = 0;
-    g.sbase = 0;
     return g;
 }
 
@@ -225,67 +223,6 @@ __global__ void __launch_bounds__(1024) k_grid_small(const int32_t* __restrict__
         ids[pos] = (int32_t)i;
         sph[pos] = make_int4(ci.x, ci.y, ci.z, (int)i);
         sw[pos] = W[i];
-    }
-}
-
-// One grid per shape of a batch, a block per shape: as k_grid_small on the
-// shape's spheres, with cell offsets relative to the shape's cell base and
-// sorted slots at the shape's sphere offset.
-__global__ void __launch_bounds__(1024) k_grid_batch(const int32_t* __restrict__ Ci, const long long* __restrict__ W,
-                                                     const long long* __restrict__ soff, long long ncap_total,
-                                                     GridParams* gp, int64_t* __restrict__ start_all,
-                                                     int32_t* __restrict__ ids, int4* __restrict__ sph,
-                                                     long long* __restrict__ sw, long long* __restrict__ cwmax_all) {
-    extern __shared__ int scount[];
-    __shared__ GridParams sg;
-    const int sh = blockIdx.x;
-    const long long s0 = soff[sh], ns = soff[sh + 1] - s0;
-    const long long ncap = 2 * ns + 64, cbase = 2 * s0 + 65ll * sh;
-    int64_t* start = start_all + cbase;
-    long long* cwmax = cwmax_all + cbase;
-    long long* rwmax = cwmax_all + ncap_total + cbase;
-    block_grid_params(Ci + 3 * s0, W + s0, ns, ncap, &sg);
-    for (long long q = threadIdx.x; q < ncap; q += blockDim.x) {
-        scount[q] = 0;
-        cwmax[q] = 0;
-        rwmax[q] = 0;
-    }
-    __syncthreads();
-    GridParams g = sg;
-    g.cbase = cbase;
-    g.sbase = s0;
-    if (threadIdx.x == 0) gp[sh] = g;
-    for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-        const int3 c = cell_of(ld_int3(Ci, s0 + i), g);
-        const int q = (c.z * g.dim.y + c.y) * g.dim.x + c.x;
-        atomicAdd(&scount[q], 1);
-        atomicMax((unsigned long long*)&cwmax[q], (unsigned long long)W[s0 + i]);
-        atomicMax((unsigned long long*)&rwmax[c.z * g.dim.y + c.y], (unsigned long long)W[s0 + i]);
-    }
-    __syncthreads();
-    const int per = (int)((ncap + blockDim.x - 1) / blockDim.x);
-    const int lo = min((long long)threadIdx.x * per, ncap), hi = min((long long)lo + per, ncap);
-    int sum = 0;
-    for (int q = lo; q < hi; q++) sum += scount[q];
-    int total;
-    int run = block_excl_scan(sum, &total);
-    for (int q = lo; q < hi; q++) {
-        const int n = scount[q];
-        start[q] = s0 + run;
-        scount[q] = run;
-        run += n;
-    }
-    if (threadIdx.x == 0) start[ncap] = s0 + total;
-    __syncthreads();
-    for (long long i = threadIdx.x; i < ns; i += blockDim.x) {
-        const long long gi = s0 + i;
-        const int3 ci = ld_int3(Ci, gi);
-        const int3 c = cell_of(ci, g);
-        const int q = (c.z * g.dim.y + c.y) * g.dim.x + c.x;
-        const long long pos = s0 + atomicAdd(&scount[q], 1);
-        ids[pos] = (int32_t)gi;
-        sph[pos] = make_int4(ci.x, ci.y, ci.z, (int)i);   // shape-local id: 17 bits of the kNN key suffice
-        sw[pos] = W[gi];
     }
 }
 
@@ -692,11 +629,10 @@ __device__ __forceinline__ void knn_insert(unsigned long long key, unsigned long
 
 __global__ void __launch_bounds__(256, 4) k_knn_warp(const int32_t* __restrict__ Xi, const uint32_t* __restrict__ vorder,
                                                   long long nv, const GridParams* __restrict__ gp,
-                                                  const int64_t* __restrict__ start_all, const int4* __restrict__ sph,
+                                                  const int64_t* __restrict__ start, const int4* __restrict__ sph,
                                                   const long long* __restrict__ sw,
-                                                  const long long* __restrict__ rwmax_all, int K,
-                                                  int32_t* __restrict__ knn, long long* __restrict__ dplus,
-                                                  const long long* __restrict__ voff, int nshapes) {
+                                                  const long long* __restrict__ rwmax, int K,
+                                                  int32_t* __restrict__ knn, long long* __restrict__ dplus) {
     typedef unsigned long long U;
     const unsigned FULL = 0xffffffffu;
     const U EMPTY = ~0ull;
@@ -704,9 +640,7 @@ __global__ void __launch_bounds__(256, 4) k_knn_warp(const int32_t* __restrict__
     const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= nv) return;   // warp-uniform
     const long long v = vorder ? (long long)vorder[w] : w;
-    const GridParams g = gp[shape_of(voff, nshapes, v)];   // the vertex's own shape's grid
-    const int64_t* __restrict__ start = start_all + g.cbase;
-    const long long* __restrict__ rwmax = rwmax_all + g.cbase;
+    const GridParams g = *gp;
     const int3 x = ld_int3(Xi, v);
     const int3 c = cell_of(x, g);
     U L = EMPTY;               // lane j: the j-th smallest key so far
@@ -791,7 +725,7 @@ __global__ void __launch_bounds__(256, 4) k_knn_warp(const int32_t* __restrict__
     if (lb2 != LLONG_MAX) dp = min(dp, lb2 - g.wmax);   // whatever was not explored
 #pragma unroll
     for (int o = 16; o; o >>= 1) dp = min(dp, __shfl_xor_sync(FULL, dp, o));
-    if (lane < K) knn[v * K + lane] = L == EMPTY ? -1 : (int)(L & 0x1ffffu) + (int)g.sbase;
+    if (lane < K) knn[v * K + lane] = L == EMPTY ? -1 : (int)(L & 0x1ffffu);
     if (lane == 0) dplus[v] = dp;
 }
 
@@ -1019,8 +953,8 @@ constexpr int FB_THREADS = 256;
 __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
     const int32_t* __restrict__ T, long long nv, const int32_t* __restrict__ Xi, const int32_t* __restrict__ Ci,
     const long long* __restrict__ W, FallbackTree tree, const int32_t* __restrict__ knn, int K,
-    const GridParams* __restrict__ gp, const int64_t* __restrict__ start_all, const int32_t* __restrict__ ids,
-    const long long* __restrict__ cwmax_all,
+    const GridParams* __restrict__ gp, const int64_t* __restrict__ start, const int32_t* __restrict__ ids,
+    const long long* __restrict__ cwmax,
     const int32_t* __restrict__ fb_list, const int32_t* __restrict__ fb_count, int32_t* __restrict__ cand_cnt,
     int32_t* __restrict__ cand, uint8_t* __restrict__ cand_ord, DevState* st, const long long* __restrict__ voff,
     int nshapes) {
@@ -1039,13 +973,8 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             if (tid == 0) cand_cnt[t] = 0;
             continue;
         }
-        // the grid, or the leaves, of the tet's shape (its first corner's)
-        const int shp = shape_of(voff, nshapes, v[0]);
         GridParams g{};
-        if (gp) g = gp[shp];
-        const int64_t* __restrict__ start = start_all + g.cbase;
-        const long long* __restrict__ cwmax = cwmax_all + g.cbase;
-
+        if (gp) g = *gp;
         // spheres whose corner distances are the thresholds to choose from:
         // the corners' owners, or the one sphere the packet search left
         int o[4];
@@ -1082,7 +1011,8 @@ __global__ void __launch_bounds__(FB_THREADS) k_candidates_fallback(
             if (pos < FB_GATHER) sid[pos] = sph;
         };
         if (!gp) {   // the leaves that may hold a sphere within a threshold, 32 at a time
-            const CandShape& S = tree.shapes ? tree.shapes[shp] : tree.one;
+            // (of the tet's shape: its first corner's)
+            const CandShape& S = tree.shapes ? tree.shapes[shape_of(voff, nshapes, v[0])] : tree.one;
             const long long nl = (S.s1 - S.s0 + 31) / 32;
             for (long long l0 = tid & ~31; l0 < nl; l0 += FB_THREADS) {
                 bool open = false;
@@ -1241,22 +1171,9 @@ size_t knn_tmp_bytes(long long nv) {
     return 2 * al(sizeof(uint64_t) * nv) + 2 * al(sizeof(uint32_t) * nv) + radix_tmp_bytes(nv);
 }
 
-long long batch_grid_cap() { return GRID_SMALL_CAP; }
-
-void launch_sphere_grid_batch(const int32_t* Ci, const long long* W, const long long* soff, int nshapes,
-                              long long ncap_total, GridParams* gp, int64_t* cell_start, int32_t* cell_ids,
-                              int4* cell_sph, long long* cell_w, long long* cell_wmax, long long max_shape_ncap,
-                              cudaStream_t s) {
-    if (nshapes <= 0) return;
-    k_grid_batch<<<(unsigned)nshapes, 1024, sizeof(int) * max_shape_ncap, s>>>(Ci, W, soff, ncap_total, gp, cell_start,
-                                                                                cell_ids, cell_sph, cell_w, cell_wmax);
-    note_launch();
-}
-
 void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams* gp, const int64_t* cell_start,
                 const int4* cell_sph, const long long* cell_w, const long long* cell_wmax, long long ncap, int K,
-                int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s,
-                const long long* voff, int nshapes) {
+                int32_t* knn, long long* dplus, void* tmp, int* d_err, bool two_word, cudaStream_t s) {
     if (nv == 0) return;
     char* p = (char*)tmp;
     uint64_t* k0 = (uint64_t*)p; p += al(sizeof(uint64_t) * nv);
@@ -1265,10 +1182,10 @@ void launch_knn(const int32_t* Xi, long long nv, long long ns, const GridParams*
     uint32_t* v1 = (uint32_t*)p; p += al(sizeof(uint32_t) * nv);
     int bits = 1;
     while ((1ll << bits) < ncap) bits++;
-    if ((ns <= (1 << 17) || nshapes > 1) && !two_word) {   // batches: shape-local ids in the key
+    if (ns <= (1 << 17) && !two_word) {
         // one vertex per warp in input order: the sphere grid stays in cache
         k_knn_warp<<<nblk(32 * nv, 256), 256, 0, s>>>(Xi, nullptr, nv, gp, cell_start, cell_sph, cell_w,
-                                                       cell_wmax + ncap, K, knn, dplus, voff, nshapes);
+                                                       cell_wmax + ncap, K, knn, dplus);
     } else {
         k_vertex_cells<<<nblk(nv, 256), 256, 0, s>>>(Xi, nv, gp, k0, v0);
         note_launch();
@@ -1283,7 +1200,7 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                        const long long* W, const int32_t* knn, const long long* dplus, int K, const GridParams* gp,
                        const int64_t* cell_start, const int32_t* cell_ids, const long long* cell_wmax,
                        int32_t* cand_cnt, int32_t* cand, uint8_t* cand_ord, int32_t* fb_list, int32_t* fb_count,
-                       DevState* st, cudaStream_t s, const long long* voff, int nshapes) {
+                       DevState* st, cudaStream_t s) {
     if (nt == 0) return;
     cudaMemsetAsync(fb_count, 0, sizeof(int32_t), s);
     k_candidates_warp<<<nblk(32 * nt, 256), 256, 0, s>>>(d_tets, nt, nv, Xi, Ci, W, knn, dplus, K, cand_cnt, cand,
@@ -1291,7 +1208,7 @@ void launch_candidates(const int32_t* d_tets, long long nt, long long nv, const 
                                                fb_list, fb_count, st);
     note_launch();
     launch_candidates_fallback(d_tets, nv, Xi, Ci, W, FallbackTree{}, knn, K, gp, cell_start, cell_ids, cell_wmax, fb_list,
-                               fb_count, cand_cnt, cand, cand_ord, st, voff, nshapes, s);
+                               fb_count, cand_cnt, cand, cand_ord, st, nullptr, 1, s);
 }
 
 void launch_candidates_fallback(const int32_t* T, long long nv, const int32_t* Xi, const int32_t* Ci,
