@@ -273,11 +273,14 @@ struct Store {
     static constexpr int VW = PrecTraits<Real>::VW;
     static constexpr int NC = (VMAX - 2) / 2;    // candidates of a tet
     static constexpr int SCR = NC + 3;           // faces of a piece
-    // FP64 rows take 32 bytes: for the bins of many candidates they would cost
-    // a quarter of the resident warps, more than computing a row again does
-    // (the 60k-tet blob in FP64: clip kernels 1.02 ms without any rows kept,
-    // 1.15 ms with all, see launch_clip)
-    static constexpr bool ROWS = sizeof(Real) == 4 || VMAX < 18;
+    // For the bins of many candidates the rows would cost a quarter of the
+    // resident warps, more than computing a row again does.  FP64 (32 bytes a
+    // row) from 7 candidates on: the 60k-tet blob, clip kernels 1.02 ms without
+    // any rows kept, 1.15 ms with all (see launch_clip).  FP32 from 9 on: 60,000
+    // spheres in 205k tets, 1.36 M pairs of 9 to 32 candidates, 16.6 ms a build
+    // with rows and 15.4 without (16.3 before rows were kept); 20,000 spheres
+    // 5.15 and 5.05; the 2 M-tet blob 7.70 either way.
+    static constexpr bool ROWS = VMAX < (sizeof(Real) == 4 ? 34 : 18);
     static constexpr int RW = ROWS ? 4 * sizeof(Real) / 4 : 0;   // words of a row
     static constexpr int WORDS = VMAX * VW + NC * RW + 12 + SCR;   // per lane
     __device__ __forceinline__ void put_row(int s, const Real R[4]) const {
