@@ -47,12 +47,14 @@ PLANNED_FLOP_PER_PIECE = {16: 2500.0, 32: 4500.0}
 # constructed on a new plane takes the cofactors of its m radical-plane rows
 # (m = 1: a selection, 0 flop; m = 2: three 2x2 minors, 9 flop; m = 3: four
 # 3x3 cofactors, 56 flop) plus its orientation test and stored bound (17).
+# The vertices of two-candidate tets (k_clip2) are booked at the same 17: their
+# closed form computes no cofactors, but the signs at the tet's corners instead.
 FLOP_SIGN_TEST = 7
 FLOP_NEW_VERTEX = (17, 26, 73)   # by m = 1, 2, 3
 # DRAM bytes (read + write) per step of the clip kernels (k_clip over its bins,
 # k_clip2 and k_whole), from one ncu capture of the current kernels per workload and
 # precision; a workload missing here reports traffic null.
-CLIP_TRAFFIC_BYTES = {("blob_c3", "fp32"): 915.0e6}
+CLIP_TRAFFIC_BYTES = {("blob_c3", "fp32"): 916.2e6}
 # CPU legs per workload, sized for 10-30 s each on the 16 host cores: tets of
 # the brute-force oracle sample, of its 1-thread sample, fraction of tets for
 # the same-algorithm baseline, tets per step of the reference arm.

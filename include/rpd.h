@@ -65,7 +65,9 @@ typedef struct {
     int32_t precision;    /* rpd_precision                                        */
     int32_t k;            /* power neighbours per tet corner, 1..32: a tet with more
                              than min(4 k, 32) spheres near it takes the slower
-                             grid search (the diagram does not depend on k)       */
+                             search over the sphere tree's leaves.  The diagram
+                             does not depend on k, and from k = 8 on neither does
+                             the work (with debug bit 4: lists of k per vertex)   */
     int32_t grid_bits;    /* coordinates and radii are rounded to multiples of
                              2^-grid_bits; |x|*2^grid_bits must stay < 2^21       */
     int32_t debug_checks; /* test switches (0 in production): value 1 sends every
@@ -89,14 +91,22 @@ typedef struct {
     int64_t pred_fast;        /* clip predicates decided by the first-stage filter */
     int64_t pred_fp64;        /* ... by the FP64 re-evaluation                     */
     int64_t pred_exact;       /* ... by exact 256-bit integer arithmetic          */
-    int64_t cand_fallback;    /* tets whose candidate set needed the grid search  */
+    int64_t cand_fallback;    /* tets whose candidate set needed the slower search
+                                 (over the tree's leaves; with debug bit 4 and in
+                                 rpd_euler_static over the sphere grid)           */
     int64_t whole_tets;       /* tets inside a single cell (no clipping)          */
     int64_t clip_vertices[3]; /* polytope vertices constructed by clipping, by the
                                  number of radical planes through them (1, 2, 3) */
     int64_t bin_pairs[8];     /* candidate pairs by candidate count of their tet:
                                  1, 2, 3, 4, 5-6, 7-8, 9-16, 17-32                */
     int64_t bin_cut[8];       /* nonempty pieces that were cut, per bin           */
-    float ms_prep, ms_knn, ms_cand, ms_clip, ms_finalize[4];
+    float ms_prep;            /* snapping and mesh combinatorics                  */
+    float ms_knn;             /* per-vertex neighbour lists: about 0 unless debug
+                                 bit 4 asks for them                              */
+    float ms_cand;            /* orders, owners and candidates                    */
+    float ms_clip;            /* end of the candidates to end of the clip kernels  */
+    float ms_finalize[4];     /* element tables; the four kinds share their
+                                 launches, so all four hold the same time         */
     float ms_clip_kernels;    /* from the start of the clip launches to the end of
                                  the last clip kernel (volume pass excluded)      */
     float ms_clip_span;       /* same start to the end of the last volume kernel  */
@@ -167,9 +177,11 @@ rpd_status rpd_batch_offsets(rpd_ctx* ctx, int32_t kind, int64_t* h_off);
  * warm-up per k (reps <= 64), CUDA events on the stream, and returns in
  * *best the base options (NULL = defaults) with the k of the fastest median
  * build, and that median in *ms_best (may be NULL).  The diagram does not
- * depend on k (the candidate sets are exact), only the time does.  The clip's
- * tiles follow each tet's candidate count and need no tuning.  Errors of a
- * build are returned as they are.
+ * depend on k (the candidate sets are exact), only the time does, and that only
+ * below k = 8: all larger k are the same build, and which of them is returned
+ * is decided by the noise of their times (with debug bit 4 they differ).  The
+ * clip's tiles follow each tet's candidate count and need no tuning.  Errors of
+ * a build are returned as they are.
  */
 rpd_status rpd_autotune(const double* d_verts, int64_t nv, const int32_t* d_tets, int64_t nt, const double* d_centers,
                         const double* d_radii, int64_t ns, const rpd_options* base, const int32_t* ks, int32_t nk,
@@ -366,7 +378,9 @@ rpd_status rpd_surface_samples(rpd_ctx* ctx, double* d_points, double* d_normals
  *   d_dist    f32[n]    distances (world units)
  *   d_prim    i32[n]    nearest primitive: row of the RPC table, then n_RPC +
  *                       row of the RPF table, then n_RPC + n_RPF + row of the
- *                       RPE table; -1 when there is none
+ *                       RPE table; -1 (and distance +infinity) when there is
+ *                       none, or for a sample whose squared coordinates are
+ *                       not finite in FP32
  * Synchronises the stream once (the mesh origin).
  */
 rpd_status rpd_envelope_distance(rpd_ctx* ctx, const double* d_samples, int64_t n, float* d_dist, int32_t* d_prim);

@@ -158,7 +158,8 @@ constexpr int IW0 = 0, IW1 = IW0 + HID * NIN, IW2 = IW1 + HID * HID, IW1T = IW2 
 // to each other and the blocks TR_LBO bytes apart: the lanes of a warp hold
 // consecutive columns, and this stride spreads their eight-column blocks over
 // the banks (consecutive core matrices along K put them all on the same eight:
-// four-way conflicts on every transposed store, 11k a CTA; now 330).
+// four-way conflicts on every transposed store, 11k a CTA; the whole kernel has
+// 870 in 14.4k wavefronts now).
 constexpr uint32_t TR_LBO = 16 * 128 + 32;
 constexpr int TR_ELEMS = 16 * (int)TR_LBO / 2;
 struct StepSmem {

@@ -634,7 +634,8 @@ def rpd_build_batch(shapes, precision="fp32", k=16, grid_bits=20, stream=None, d
 
 def rpd_autotune(verts, tets, centers, radii, ks=(8, 16, 24, 32), reps=3, precision="fp32", grid_bits=20,
                  stream=None):
-    """The library's autotuner: (fastest k, its median build time in ms)."""
+    """The library's autotuner: (fastest k, its median build time in ms).  From
+    k = 8 on every k is the same build, so among those the answer is noise."""
     lib = load()
     if not torch.cuda.is_available():
         raise RuntimeError("librpd needs a CUDA device; there is no CPU fallback")
